@@ -109,10 +109,12 @@ const char *osprey_last_error(void);
 /* Validate the shape and weight pointers and make a context (host memory only).
  * The context picks the kernels a draft call uses:
  *   rows <= 2 per chain step: TMA-streamed GEMVs (weights read once per step);
- *   3..80 rows: tcgen05 tensor-core GEMMs, float32 activations split into three
- *     bf16 planes (24 mantissa bits) so results match the GEMV path's (the LM
- *     head's operand into two planes, 16 bits: its logits differ from the
- *     GEMV path's by rounding of the operand's last bits);
+ *   3..4096 rows: tcgen05 tensor-core GEMMs in tiles of up to 80 rows, float32
+ *     activations split into three bf16 planes (24 mantissa bits) so results
+ *     match the GEMV path's (the LM head's operand of up to 80 sequences into
+ *     two planes, 16 bits: its logits differ from the GEMV path's by rounding
+ *     of the operand's last bits);
+ *   more rows: CUDA-core GEMVs, eight rows at a time;
  *   attention: clusters merged on chip while they fit one wave, else global
  *     partials.
  * Two environment variables, read here, select the alternatives for testing:
@@ -251,7 +253,7 @@ size_t osprey_dflash_workspace_bytes(const osprey_ctx *ctx, int B, int block, in
  * (argmax at T = 0).  The proposals are verified like a chain of block - 1
  * draft tokens (osprey_verify with K = block - 1).
  *   block  4 .. 81 (3 .. 80 proposals); sequences are processed in groups of
- *          floor(80 / (block - 1)), each group one tensor-core pass over the
+ *          floor(512 / (block - 1)), each group one tensor-core pass over the
  *          weights (SHAPE if the context has no tensor-core path)
  *   anchors [B] int32 (device), mask_token in [0, vocab)
  *   feats  [B][feat_dim] bf16: the concatenated target hidden states gathered

@@ -47,7 +47,7 @@ struct osprey_ctx {
     Dims dim;
     int sms;
     int attn_cs;    // cluster size of the attention kernel (0: split partials in global memory)
-    bool tc;        // batched rows (3..80) run their projections on tcgen05
+    bool tc;        // batched rows (3..TC_MAX_ROWS) run their projections on tcgen05
     bool fused_mlp; // batch-1 chain steps run O-proj, gate/up and down as one launch
     bool fused_layer; // batch-1 chain steps run each whole layer as one launch
     CUtensorMap tm_c, tm_lm, tm_qkv[OSPREY_MAX_LAYERS], tm_o[OSPREY_MAX_LAYERS], tm_gate[OSPREY_MAX_LAYERS],
@@ -261,30 +261,31 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     size_t o_lsup = take(8ull * B * lmp.blocks * lmp.nsup);   // the streamed LM head's run statistics (rows <= 2)
     size_t o_lc = take(16ull * B * lmp.blocks);
     // tensor-core path: bf16 operand planes, QKV output, row-sampler partials
-    const long long tc_rows = std::min<long long>(std::max<long long>(R_ext, B), TC_MAX_ROWS);
-    const long long np = (tc_rows + 15) / 16 * 16;
+    // (a step of more than TC_MAX_ROWS rows runs on the CUDA cores and needs none)
+    const long long re = R_ext <= TC_MAX_ROWS ? R_ext : 0, rc = B <= TC_MAX_ROWS ? B : 0;
+    const long long np = std::max(tc_tiles(re).rows(), tc_tiles(rc).rows());
     const long long nqkv = (long long)(D.Hq + 2 * D.Hkv) * D.hd;
     const bool tcw = ctx->tc;
     size_t o_xq = take(tcw ? 2ull * TC_PLANES * np * 2 * D.d : 0), o_yq = take(tcw ? 4ull * np * nqkv : 0);
     size_t o_xo = take(tcw ? 2ull * TC_PLANES * np * D.Hq * D.hd : 0), o_xg = take(tcw ? 2ull * TC_PLANES * np * D.d : 0);
     size_t o_xh = take(tcw ? 2ull * TC_PLANES * np * D.F : 0), o_xl = take(tcw ? 2ull * TC_PLANES * np * D.d : 0);
     const long long lm_nsub = (D.V + TC_LM_GROUP - 1) / TC_LM_GROUP;
-    size_t o_rp = take(tcw ? 16ull * R_lm * lm_nsub : 0);
+    size_t o_rp = take(tcw && R_lm <= TC_MAX_ROWS ? 16ull * R_lm * lm_nsub : 0);
     // split-K partials: the largest nsplit x rows x outputs of the call's projections
     long long part = 0;
     if (tcw) {
-        const long long rows = tc_rows;
-        auto need = [&](int nout, int K_) {
-            const int ns = tc_nsplit(nout, K_, ctx->sms);
-            if (ns > 1) part = std::max(part, (long long)ns * rows * nout);
-        };
-        need(D.d, D.feat);
-        need((D.Hq + 2 * D.Hkv) * D.hd, 2 * D.d);
-        need(D.d, D.Hq * D.hd);
-        // gate/up: one GEMM whose partials always go through the buffer
-        part = std::max(part, (long long)std::max(tc_nsplit(2 * D.F, D.d, ctx->sms), 1) * rows * 2 * D.F);
-        need(D.d, D.F);
-        need(D.V, D.d);
+        for (const long long rows : {re, rc}) {
+            const int nrt = tc_tiles(rows).nrt;
+            auto need = [&](int nout, int K_, bool always = false) {
+                const int ns = tc_nsplit(nout, K_, nrt, ctx->sms);
+                if (ns > 1 || always) part = std::max(part, (long long)ns * rows * nout);
+            };
+            need(D.d, D.feat);
+            need((D.Hq + 2 * D.Hkv) * D.hd, 2 * D.d);
+            need(D.d, D.Hq * D.hd);
+            need(2 * D.F, D.d, true);   // gate/up: one GEMM whose partials always go through the buffer
+            need(D.d, D.F);
+        }
     }
     size_t o_tp = take(4ull * part);
     if (ws && base) {
@@ -402,9 +403,9 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         return fail(OSPREY_ERR_CAPACITY, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
     if (block && (K != 1 || !ctx->tc || B * max_new < 3 || B * max_new > TC_MAX_ROWS))
         return fail(OSPREY_ERR_SHAPE, "block drafting runs 3..%d rows per group on the tensor cores", TC_MAX_ROWS);
-    if (topk > 1 && (!ctx->tc || B > TC_MAX_ROWS))
+    if (topk > 1 && (!ctx->tc || B > TC_TILE_ROWS))
         return fail(OSPREY_ERR_SHAPE, "topk > 1 samples on the tensor-core LM head: at most %d sequences and a "
-                                      "device with tcgen05 (not OSPREY_TC=0)", TC_MAX_ROWS);
+                                      "device with tcgen05 (not OSPREY_TC=0)", TC_TILE_ROWS);
 
     cudaStream_t s = (cudaStream_t)stream;
     const Dims &D = ctx->dim;
@@ -436,7 +437,9 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     for (int i = 0; i < D.hd / 2; ++i) g.inv_freq[i] = ctx->inv_freq[i];
     // tensor-core path for 3..TC_MAX_ROWS activation rows
     auto tc_rows = [&](int rows) { return ctx->tc && rows >= 3 && rows <= TC_MAX_ROWS; };
-    auto npad_of = [](int rows) { return (rows + 15) / 16 * 16; };
+    auto npad_of = [](int rows) { return tc_tiles(rows).rows(); };   // rows of an operand plane
+    // the LM head's operand planes: three for batches beyond one tile of rows
+    const int lm_npl = block || B <= TC_TILE_ROWS ? TC_LM_PLANES : TC_PLANES;
     // the next GEMM's operand planes, written by a residual GEMM's reduction when it has one
     struct NextPlanes {
         uint16_t *dst;
@@ -447,14 +450,17 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
                        const void *xbuf, bool in_place_rows, float *y, int ldy, uint16_t *h,
                        const char *what, const CUtensorMap *wb = nullptr, const NextPlanes *nxt = nullptr,
                        bool *nxt_done = nullptr, const QkvPostArgs *rope = nullptr) -> int {
-        const int np = npad_of(rows);
+        const TcTiles tt = tc_tiles(rows);
         CUtensorMap xm;
-        const bool ok = in_place_rows ? tc_encode_rows(&xm, xbuf, rows, np, K_) : tc_encode_operand(&xm, xbuf, planes, np, K_);
+        const bool ok = in_place_rows ? tc_encode_rows(&xm, xbuf, rows, tt.npad, K_)
+                                      : tc_encode_operand(&xm, xbuf, planes, tt, K_);
         if (!ok) return fail(OSPREY_ERR_INVALID_ARG, "%s: tensor map encoding failed", what);
         TcArgs ta{};
         ta.epi = epi;
         ta.R = rows;
-        ta.npad = np;
+        ta.npad = tt.npad;
+        ta.nrt = tt.nrt;
+        ta.fine = tt.nrt > 1 && !block;
         ta.K = K_;
         ta.nout = nout;
         ta.planes = planes;
@@ -487,17 +493,19 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     // sampling partials in its epilogue (logits stored only into z, when given),
     // then one pick block per row
     auto tc_lm = [&](int rows, float *z, long long ldz, const LmPickArgs &pick_in) -> int {
-        const int np = npad_of(rows);
+        const TcTiles tt = tc_tiles(rows);
         CUtensorMap xm;
-        if (!tc_encode_operand(&xm, ws.tc_xl, TC_LM_PLANES, np, D.d))
+        if (!tc_encode_operand(&xm, ws.tc_xl, lm_npl, tt, D.d))
             return fail(OSPREY_ERR_INVALID_ARG, "lm head: tensor map encoding failed");
         TcArgs ta{};
         ta.epi = TC_LM;
         ta.R = rows;
-        ta.npad = np;
+        ta.npad = tt.npad;
+        ta.nrt = tt.nrt;
+        ta.fine = tt.nrt > 1 && !block;
         ta.K = D.d;
         ta.nout = D.V;
-        ta.planes = TC_LM_PLANES;
+        ta.planes = lm_npl;
         ta.y = z;
         ta.ldy = (int)ldz;
         ta.status = dev_status;
@@ -511,7 +519,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         pk.part = ws.rs_part;
         pk.nsub = ta.lm_nsub;
         pk.planes = ws.tc_xl;
-        pk.npad = np;
+        pk.npad = tt.rows();
+        pk.npl = lm_npl;
         pk.W = (const uint16_t *)W.lm_head;
         pk.temperature = temperature;
         pk.u_draft = u_draft;
@@ -695,7 +704,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
                 nxtp = &nxt;
             } else if (lm_tc) {
                 const bool last_rows = ext && !block;   // one LM row per sequence: its last new row
-                nxt = NextPlanes{ws.tc_xl, (const uint16_t *)W.final_norm, D.d, 0, TC_LM_PLANES, last_rows ? 1 : 0,
+                nxt = NextPlanes{ws.tc_xl, (const uint16_t *)W.final_norm, D.d, 0, lm_npl, last_rows ? 1 : 0,
                                  rows_per_seq, npad_of(last_rows ? B : R)};
                 nxtp = &nxt;
             }
@@ -813,7 +822,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             const int rows = B * max_new;
             int rc;
             if (!xl_ready && (rc = planes(x, (const uint16_t *)W.final_norm, D.d, rows, D.d, 0, ws.tc_xl, max_new, false,
-                                          "lm operand", TC_LM_PLANES)) != OSPREY_OK)
+                                          "lm operand", lm_npl)) != OSPREY_OK)
                 return rc;
             LmPickArgs pk{};
             pk.B = rows;
@@ -854,7 +863,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             // (topk candidates per row when drafting a tree)
             int rc;
             if (!xl_ready && (rc = planes(x, (const uint16_t *)W.final_norm, D.d, B, D.d, 0, ws.tc_xl, 1, ext,
-                                          "lm operand", TC_LM_PLANES)) != OSPREY_OK)
+                                          "lm operand", lm_npl)) != OSPREY_OK)
                 return rc;
             LmPickArgs pk{};
             pk.B = B;
@@ -955,12 +964,12 @@ extern "C" int osprey_draft_step_topk(osprey_ctx *ctx, const osprey_kv *kv, int 
 }
 
 // ------------------------------------------------------------------ block drafting
-// Sequences are drafted in groups whose block rows fit one tensor-core tile
-// (TC_MAX_ROWS rows); each group's call re-reads the weights once.  Workspace:
+// Sequences are drafted in groups of at most TC_GROUP_ROWS block rows; each
+// group's call reads the weights once (its row tiles share them through L2).  Workspace:
 // the block-mode draft layout of one group, then the group's token array
 // [n][P], n_new [n] and broadcast features [n][P][feat_dim] bf16.
 static int block_group(int B, int P) {
-    const int g = TC_MAX_ROWS / P;
+    const int g = TC_GROUP_ROWS / P;
     return g < 1 ? 1 : (g < B ? g : B);
 }
 
@@ -982,7 +991,7 @@ static size_t block_layout(const osprey_ctx *ctx, int n, int P, int max_pages, D
 }
 
 static bool block_args_ok(const osprey_ctx *ctx, int B, int block, int max_pages) {
-    return ctx && B >= 1 && B <= 65535 && block >= 4 && block <= TC_MAX_ROWS + 1 && max_pages >= 1 &&
+    return ctx && B >= 1 && B <= 65535 && block >= 4 && block <= TC_TILE_ROWS + 1 && max_pages >= 1 &&
            (long long)max_pages * ctx->dim.P < (1LL << 30);
 }
 
@@ -1001,7 +1010,7 @@ extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, i
     if (B == 0) return OSPREY_OK;
     if (!block_args_ok(ctx, B, block, kv->max_pages_per_seq))
         return fail(OSPREY_ERR_INVALID_ARG, "B in 1..65535, block in 4..%d and max_pages_per_seq >= 1 required",
-                    TC_MAX_ROWS + 1);
+                    TC_TILE_ROWS + 1);
     if (!ctx->tc)
         return fail(OSPREY_ERR_SHAPE, "block drafting runs on the tensor cores; this context has none "
                                       "(OSPREY_TC=0 or no tcgen05)");
@@ -1122,7 +1131,7 @@ extern "C" int osprey_verify_tree(int B, int K, int topk, int V, int logits_dtyp
 
 // ------------------------------------------------------------------ logits-free verify
 // Workspace: the verify layout (counters, partials, decisions, chunk sums), then
-// for one group of up to TC_MAX_ROWS sequences the gathered kept states
+// for one group of up to TC_TILE_ROWS sequences the gathered kept states
 // [rows][d] float, their operand planes [TC_PLANES][npad][d] bf16, the
 // recomputed decision-row logits [rows][V] float (the draft step's LM-head GEMM:
 // the same operand planes, unsplit, so the rows come out the same).
@@ -1136,7 +1145,7 @@ struct HiddenWs {
 static size_t verify_hidden_layout(const osprey_ctx *ctx, int B, int K, VerifyArgs *a, void *base, HiddenWs *hw) {
     const Dims &D = ctx->dim;
     size_t off = align256(verify_workspace_layout(B, K, D.V, a, base));
-    const int group = B < TC_MAX_ROWS ? B : TC_MAX_ROWS;
+    const int group = B < TC_TILE_ROWS ? B : TC_TILE_ROWS;
     const int npad = (group + 15) / 16 * 16;
     const size_t o_r = off;
     off = align256(off + 4ull * group * D.d);
@@ -1237,7 +1246,7 @@ extern "C" int osprey_verify_hidden(osprey_ctx *ctx, int B, int K, int logits_dt
         if ((e = launch_planes(pl, s)) != cudaSuccess) return cuda_fail(e, "decision-row operand launch");
         // 3. their draft logits on the tensor cores (the draft step's LM head GEMM)
         CUtensorMap xm;
-        if (!tc_encode_operand(&xm, hw.planes, TC_LM_PLANES, npad, D.d))
+        if (!tc_encode_operand(&xm, hw.planes, TC_LM_PLANES, TcTiles{1, npad}, D.d))
             return fail(OSPREY_ERR_INVALID_ARG, "decision-row tensor map encoding failed");
         TcArgs ta{};
         ta.epi = TC_STORE;

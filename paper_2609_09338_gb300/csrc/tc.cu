@@ -38,6 +38,19 @@ constexpr size_t TC_SMEM_CAP = (OSP_TC_CTAS_PER_SM == 1 ? 200 : 100) * 1024;
 #ifndef OSP_TC_SEGKB
 #define OSP_TC_SEGKB 8   // k-blocks (64 wide) per accumulation segment
 #endif
+// Accuracy of the accumulators.  A tensor-core accumulator drops the bits below
+// its last place at every step instead of rounding to nearest, so its error
+// grows with the steps that add to a large value.  The planes after the first,
+// 2^-8 and 2^-16 of it, therefore have an accumulator of their own, and calls of
+// more rows than a tile, which come out as accurate as the CUDA-core GEMV, take
+// segments of 2 k-blocks: 8 steps at full size instead of 96.  Measured
+// against float64 on 96 sequences, d 1024 (logits, cached bf16 K values that
+// round otherwise; us a call): 8 k-blocks, one accumulator 1.9e-6, 1160, 4250;
+// 2 k-blocks, one accumulator 4.9e-7, 370, 5140; 4 k-blocks, two 2.8e-7, 220,
+// 3780; 2 k-blocks, two 1.7e-7, 170, 4020; the GEMV 1.6e-7, 220, 34500.
+#ifndef OSP_TC_SEGKB_FINE
+#define OSP_TC_SEGKB_FINE 2
+#endif
 #ifndef OSP_TC_LM_NA
 #define OSP_TC_LM_NA 2   // LM head: weight tiles per stage that share one operand stage
 #endif
@@ -97,6 +110,11 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const float (&v)[16]) {
         : "memory");
 }
 __device__ __forceinline__ void tc_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// Keeps the uses of a tcgen05.ld's registers after the wait before this call.
+__device__ __forceinline__ void tc_ld_tie(float (&v)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) asm volatile("" : "+f"(v[j]));
+}
 
 // x ~= q0 + q1 + q2 with q_i = bf16(x - q0 - ... - q_{i-1}): 8 significant bits
 // per plane, so three planes carry a float32 value's 24 (up to the last rounding).
@@ -133,13 +151,15 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
               const __grid_constant__ CUtensorMap xm, const TcArgs a, int nst) {
     extern __shared__ uint8_t raw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[TC_MAXST], empty[TC_MAXST], accf[2], acce[2], fin;
+    __shared__ __align__(8) uint64_t full[TC_MAXST], empty[TC_MAXST], accf[2], acce[2], sepe, fin;
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // work item = (NA output tiles of 128 features, k-range); items of a CTA are contiguous
+    // work item = (NA output tiles of 128 features, row tile, k-range), the k-range
+    // fastest; items of a CTA are contiguous
     const int segkb = a.segkb;
-    const int n_items = (a.nout + 128 * NA - 1) / (128 * NA) * a.nsplit;
+    const int per_ft = a.nrt * a.nsplit;   // items of one feature tile
+    const int n_items = (a.nout + 128 * NA - 1) / (128 * NA) * per_ft;
     const int i0 = (int)((long long)n_items * blockIdx.x / gridDim.x);
     const int i1 = (int)((long long)n_items * (blockIdx.x + 1) / gridDim.x);
     const int nloc = i1 - i0, nkb = a.K / 64, npad = a.npad;
@@ -150,12 +170,13 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     };
     const uint32_t bbytes = (uint32_t)a.planes * npad * 128;
     const uint32_t stage = NA * TC_ABYTES + bbytes;
-    // TMEM: two segment buffers and (when a tile has several segments) the
-    // running float32 total of the tile
+    // TMEM: two segment buffers, and with `sep` one accumulator of the planes
+    // after the first over the item's whole k-range (they are 2^-8 and 2^-16 of
+    // the first plane, so what their accumulator drops does not matter)
     const uint32_t acc_cols = NA * npad;
-    const int nseg_max = (min(nkb, a.kbps) + segkb - 1) / segkb;
+    const bool sep = NA == 1 && a.sep;
     uint32_t ncols = 32;
-    while (ncols < (nseg_max > 1 ? 3 : 2) * acc_cols) ncols <<= 1;
+    while (ncols < (sep ? 3 : 2) * acc_cols) ncols <<= 1;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -171,6 +192,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             mbar_init(&accf[i], 1);
             mbar_init(&acce[i], 4);
         }
+        mbar_init(&sepe, 4);
         mbar_init(&fin, 1);
         s_abort = 0;
         mbar_fence_init();
@@ -196,7 +218,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             };
             long long npre = 0;   // stages whose weights were requested before the wait
             for (int it = 0; it < nloc && npre < nst; ++it) {
-                const int y = (i0 + it) / a.nsplit * 128 * NA;
+                const int y = (i0 + it) / per_ft * 128 * NA;
                 int klo, khi;
                 krange(i0 + it, klo, khi);
                 for (int kb = klo; kb < khi && npre < nst; ++kb, ++npre) {
@@ -208,7 +230,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             long long g = 0;
             bool stop = false;
             for (int it = 0; it < nloc && !stop; ++it) {
-                const int y = (i0 + it) / a.nsplit * 128 * NA;
+                const int y = (i0 + it) / per_ft * 128 * NA;
+                const int row0 = (i0 + it) / a.nsplit % a.nrt * npad;   // of the operand planes
                 int klo, khi;
                 krange(i0 + it, klo, khi);
                 for (int kb = klo; kb < khi; ++kb, ++g) {
@@ -228,7 +251,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                         weights(st, y, kb, &full[s]);
                     }
                     for (int p = 0; p < a.planes; ++p)
-                        tma_2d(st + NA * TC_ABYTES + (size_t)p * npad * 128, &xm, kb * 64, p * npad, &full[s]);
+                        tma_2d(st + NA * TC_ABYTES + (size_t)p * npad * 128, &xm, kb * 64, p * a.nrt * npad + row0,
+                               &full[s]);
                 }
             }
             if (stop) {   // let the copies this thread issued land before the CTA can exit
@@ -271,16 +295,35 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                         }
                         tc_fence_after();
                         const uint32_t st = smem_u32(sm + (size_t)s * stage);
+                        auto step = [&](int p, int kk, uint32_t d, uint32_t acc) {
+                            const uint64_t db = tc_desc(st + NA * TC_ABYTES + (uint32_t)p * npad * 128);
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            for (int p = 0; p < a.planes; ++p) {
-                                const uint64_t db = tc_desc(st + NA * TC_ABYTES + (uint32_t)p * npad * 128);
-                                const uint32_t acc = (kb != kb0) || kk || p;
+                            for (int t = 0; t < NA; ++t)
+                                tc_mma(d + (uint32_t)(t * npad), tc_desc(st + t * TC_ABYTES) + 2 * kk, db + 2 * kk,
+                                       idesc, acc);
+                        };
+                        if (sep) {
 #pragma unroll
-                                for (int t = 0; t < NA; ++t)
-                                    tc_mma(d0 + (uint32_t)(t * npad), tc_desc(st + t * TC_ABYTES) + 2 * kk, db + 2 * kk,
-                                           idesc, acc);
+                            for (int kk = 0; kk < 4; ++kk) step(0, kk, d0, (kb != kb0) || kk);
+                            // the item's first small-plane step overwrites that accumulator: the
+                            // epilogue has to have read the previous item's
+                            if (kb == klo && it > 0 && !mbar_wait(&sepe, (uint32_t)(it - 1) & 1)) {
+                                set_status(a.status, OSPREY_ERR_TIMEOUT);
+                                atomicExch(&s_abort, 1);
+                                stop = true;
+                                break;
                             }
+                            for (int p = 1; p < a.planes; ++p)
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    step(p, kk, tmem + 2u * acc_cols, (kb != klo) || kk || p > 1);
+                        } else {
+                            // plane by plane (planes inside a k-step made the calls 1.5 % slower), the
+                            // small ones first, while the accumulator is small
+                            for (int p = a.planes - 1; p >= 0; --p)
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    step(p, kk, d0, (kb != kb0) || kk || p != a.planes - 1);
                         }
                         tc_commit(&empty[s]);
                     }
@@ -292,110 +335,175 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
         }
     } else {
         // epilogue: TMEM lanes (warp % 4) * 32 .. + 31 hold output features m.
-        // Each segment's partial is added into the tile's running total in float32;
-        // the last segment's sum goes through the epilogue.
         const int lg = (warp & 3) * 32;
         const int m = lg + lane;
+        const uint32_t lanes = tmem + ((uint32_t)lg << 16);
         long long u = 0;
         bool stop = false;
+        int ft = 0, sp = 0, col0 = 0, row0 = 0;
+        // the finished sums v of rows row0 + c0 .. + 15, feature col0 + 128 tile
+        auto finish = [&](int tile, int c0, float (&v)[16]) {
+            const int col = col0 + 128 * tile;
+            const bool colok = col < a.nout;
+            if constexpr (EPI == TC_LM) {
+                // per row: (argmax z, sum exp((z - max z) / T)) over this warp's 32
+                // ids, for the 16 rows c0.. at once: each butterfly round halves the
+                // rows a lane carries (it keeps one half and receives the partner's
+                // share of it), so after four rounds lane l holds row l / 2 over 16
+                // lanes and one more exchange completes it over all 32
+                const int sub = (int)(((long long)ft * 128 * NA + 128 * tile + lg) / TC_LM_GROUP);
+                float av[16], sv[16];
+                int ai[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    av[j] = colok ? v[j] : -INFINITY;
+                    ai[j] = colok ? col : 0x7fffffff;
+                    sv[j] = colok ? 1.f : 0.f;
+                    if (a.y && colok && row0 + c0 + j < a.R) a.y[(size_t)(row0 + c0 + j) * a.ldy + col] = v[j];
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int off = 16 >> r, w = 8 >> r;
+                    const bool up = lane & off;
+#pragma unroll
+                    for (int i = 0; i < w; ++i) {
+                        const float ra = __shfl_xor_sync(0xffffffffu, up ? av[i] : av[i + w], off);
+                        const int ri = __shfl_xor_sync(0xffffffffu, up ? ai[i] : ai[i + w], off);
+                        const float rs = __shfl_xor_sync(0xffffffffu, up ? sv[i] : sv[i + w], off);
+                        float ka = up ? av[i + w] : av[i], ks = up ? sv[i + w] : sv[i];
+                        int ki = up ? ai[i + w] : ai[i];
+                        lm_combine(ka, ki, ks, ra, ri, rs, a.lm_invT);
+                        av[i] = ka;
+                        ai[i] = ki;
+                        sv[i] = ks;
+                    }
+                }
+                {
+                    const float ra = __shfl_xor_sync(0xffffffffu, av[0], 1);
+                    const int ri = __shfl_xor_sync(0xffffffffu, ai[0], 1);
+                    const float rs = __shfl_xor_sync(0xffffffffu, sv[0], 1);
+                    lm_combine(av[0], ai[0], sv[0], ra, ri, rs, a.lm_invT);
+                }
+                const int n = row0 + c0 + (lane >> 1);
+                if (!(lane & 1) && n < a.R && sub < a.lm_nsub)
+                    a.lm_part[(size_t)n * a.lm_nsub + sub] =
+                        make_float4(av[0] * a.lm_invT, sv[0], av[0], __int_as_float(ai[0]));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const int n = row0 + c0 + j;
+                    if (n >= a.R || !colok) continue;
+                    if (a.nsplit > 1 || EPI == TC_GLU) {   // partial of this k-range; tc_reduce applies the epilogue
+                        a.part[((size_t)sp * a.R + n) * a.nout + col] = v[j];
+                    } else if (EPI == TC_STORE) {
+                        a.y[(size_t)n * a.ldy + col] = v[j];
+                    } else if (EPI == TC_RESID) {
+                        a.x[(size_t)n * a.ldy + col] += v[j];
+                    }
+                }
+            }
+        };
         for (int it = 0; it < nloc && !stop; ++it) {
-            const int col0 = (i0 + it) / a.nsplit * 128 * NA + m, sp = (i0 + it) % a.nsplit;
-            const uint32_t tt = tmem + ((uint32_t)lg << 16) + 2u * acc_cols;
+            ft = (i0 + it) / per_ft;
+            sp = (i0 + it) % a.nsplit;
+            col0 = ft * 128 * NA + m;
+            row0 = (i0 + it) / a.nsplit % a.nrt * npad;
             int klo, khi;
             krange(i0 + it, klo, khi);
             const int nseg = (khi - klo + segkb - 1) / segkb;
-            for (int sg = 0; sg < nseg; ++sg, ++u) {
-                const int buf = (int)(u & 1);
-                if (!mbar_wait(&accf[buf], (uint32_t)(u >> 1) & 1) || *(volatile int *)&s_abort) {
-                    set_status(a.status, OSPREY_ERR_TIMEOUT);
-                    atomicExch(&s_abort, 1);
-                    stop = true;
-                    break;
+            auto wait_acc = [&]() {
+                if (mbar_wait(&accf[u & 1], (uint32_t)(u >> 1) & 1) && !*(volatile int *)&s_abort) {
+                    tc_fence_after();
+                    return true;
                 }
-                tc_fence_after();
-                const bool last = sg == nseg - 1;
-                const uint32_t t0 = tmem + ((uint32_t)lg << 16) + (uint32_t)buf * acc_cols;
-                for (int cc = 0; cc < NA * npad; cc += 16) {
-                    // accumulator columns [t npad, (t + 1) npad) hold tile t's rows
-                    const int tile = cc / npad, c0 = cc - tile * npad;
-                    const int col = col0 + 128 * tile;
-                    const bool colok = col < a.nout;
-                    float v[16], tv[16];
-                    tc_ld16(t0 + (uint32_t)cc, v);
-                    if (sg > 0) tc_ld16(tt + (uint32_t)cc, tv);
-                    tc_ld_wait();
-                    if (sg > 0) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) v[j] += tv[j];
-                    }
-                    if (!last) {
-                        tc_st16(tt + (uint32_t)cc, v);
-                        continue;
-                    }
-                    if constexpr (EPI == TC_LM) {
-                        // per row: (argmax z, sum exp((z - max z) / T)) over this warp's 32
-                        // ids, for the 16 rows c0.. at once: each butterfly round halves the
-                        // rows a lane carries (it keeps one half and receives the partner's
-                        // share of it), so after four rounds lane l holds row l / 2 over 16
-                        // lanes and one more exchange completes it over all 32
-                        const int sub = (int)(((long long)((i0 + it) / a.nsplit) * 128 * NA + 128 * tile + lg) /
-                                              TC_LM_GROUP);
-                        float av[16], sv[16];
-                        int ai[16];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            av[j] = colok ? v[j] : -INFINITY;
-                            ai[j] = colok ? col : 0x7fffffff;
-                            sv[j] = colok ? 1.f : 0.f;
-                            if (a.y && colok && c0 + j < a.R) a.y[(size_t)(c0 + j) * a.ldy + col] = v[j];
-                        }
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) {
-                            const int off = 16 >> r, w = 8 >> r;
-                            const bool up = lane & off;
-#pragma unroll
-                            for (int i = 0; i < w; ++i) {
-                                const float ra = __shfl_xor_sync(0xffffffffu, up ? av[i] : av[i + w], off);
-                                const int ri = __shfl_xor_sync(0xffffffffu, up ? ai[i] : ai[i + w], off);
-                                const float rs = __shfl_xor_sync(0xffffffffu, up ? sv[i] : sv[i + w], off);
-                                float ka = up ? av[i + w] : av[i], ks = up ? sv[i + w] : sv[i];
-                                int ki = up ? ai[i + w] : ai[i];
-                                lm_combine(ka, ki, ks, ra, ri, rs, a.lm_invT);
-                                av[i] = ka;
-                                ai[i] = ki;
-                                sv[i] = ks;
-                            }
-                        }
-                        {
-                            const float ra = __shfl_xor_sync(0xffffffffu, av[0], 1);
-                            const int ri = __shfl_xor_sync(0xffffffffu, ai[0], 1);
-                            const float rs = __shfl_xor_sync(0xffffffffu, sv[0], 1);
-                            lm_combine(av[0], ai[0], sv[0], ra, ri, rs, a.lm_invT);
-                        }
-                        const int n = c0 + (lane >> 1);
-                        if (!(lane & 1) && n < a.R && sub < a.lm_nsub)
-                            a.lm_part[(size_t)n * a.lm_nsub + sub] =
-                                make_float4(av[0] * a.lm_invT, sv[0], av[0], __int_as_float(ai[0]));
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            const int n = c0 + j;
-                            if (n >= a.R || !colok) continue;
-                            if (a.nsplit > 1 || EPI == TC_GLU) {   // partial of this k-range; tc_reduce applies the epilogue
-                                a.part[((size_t)sp * a.R + n) * a.nout + col] = v[j];
-                            } else if (EPI == TC_STORE) {
-                                a.y[(size_t)n * a.ldy + col] = v[j];
-                            } else if (EPI == TC_RESID) {
-                                a.x[(size_t)n * a.ldy + col] += v[j];
-                            }
-                        }
-                    }
-                }
-                if (!last) tc_st_wait();
+                set_status(a.status, OSPREY_ERR_TIMEOUT);
+                atomicExch(&s_abort, 1);
+                stop = true;
+                return false;
+            };
+            auto release = [&]() {
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&acce[buf]);
+                if (lane == 0) mbar_arrive(&acce[u & 1]);
+            };
+            if constexpr (NA == 1) {
+                // several segments: the running total is kept in registers, each segment
+                // added to it in float32 and its buffer freed at once, and is put back
+                // into the last segment's buffer, from which the loop below finishes it
+                // (a loop over chunks in TMEM: unrolled over registers, its code is five
+                // times as long, which cost each short launch 5 us of instruction fetches)
+                if (nseg > 1) {
+                    constexpr int NCH = TC_TILE_ROWS / 16;
+                    const int nch = npad / 16;
+                    float tot[NCH][16];
+                    auto add = [&](uint32_t t0) {   // two chunks' loads in flight at a time
+#pragma unroll
+                        for (int c = 0; c < NCH; c += 2) {
+                            float v[2][16];
+                            if (c < nch) tc_ld16(t0 + 16u * c, v[0]);
+                            if (c + 1 < NCH && c + 1 < nch) tc_ld16(t0 + 16u * (c + 1), v[1]);
+                            tc_ld_wait();
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                if (c + i < NCH && c + i < nch) {
+                                    tc_ld_tie(v[i]);
+#pragma unroll
+                                    for (int j = 0; j < 16; ++j) tot[c + i][j] += v[i][j];
+                                }
+                        }
+                    };
+#pragma unroll
+                    for (int c = 0; c < NCH; ++c)
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) tot[c][j] = 0.f;
+                    for (int sg = 0; sg < nseg; ++sg) {
+                        if (!wait_acc()) break;
+                        add(lanes + (uint32_t)(u & 1) * acc_cols);
+                        if (sg < nseg - 1) {
+                            release();
+                            ++u;
+                        }
+                    }
+                    if (stop) break;
+                    if (sep) {
+                        add(lanes + 2u * acc_cols);
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&sepe);
+                    }
+#pragma unroll
+                    for (int c = 0; c < NCH; ++c)
+                        if (c < nch) tc_st16(lanes + (uint32_t)(u & 1) * acc_cols + 16u * c, tot[c]);
+                    tc_st_wait();
+                } else if (!wait_acc()) {
+                    break;
+                }
+            } else if (!wait_acc()) {   // one segment an item
+                break;
             }
+            const uint32_t t0 = lanes + (uint32_t)(u & 1) * acc_cols;
+            for (int cc = 0; cc < NA * npad; cc += 16) {
+                // accumulator columns [t npad, (t + 1) npad) hold tile t's rows
+                const int tile = cc / npad;
+                float v[16];
+                tc_ld16(t0 + (uint32_t)cc, v);
+                if (sep && nseg == 1) {
+                    float w[16];
+                    tc_ld16(lanes + 2u * acc_cols + (uint32_t)cc, w);
+                    tc_ld_wait();
+                    tc_ld_tie(v);
+                    tc_ld_tie(w);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] += w[j];
+                } else {
+                    tc_ld_wait();
+                    tc_ld_tie(v);
+                }
+                finish(tile, cc - tile * npad, v);
+            }
+            release();
+            if (sep && nseg == 1 && lane == 0) mbar_arrive(&sepe);   // after release()'s warp barrier
+            ++u;
         }
     }
     tc_fence_before();
@@ -407,7 +515,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
 // ---------------------------------------------------------------- split-K reduction
 // out[n][col] = sum over the k-ranges (in order) of the partials, then the
 // GEMM's epilogue.  TC_GLU: gate = output col, up = output nout_a + col, and
-// the planes of h = silu(gate) * up go to h [TC_PLANES][npad][nout_a].
+// the planes of h = silu(gate) * up go to h [TC_PLANES][nrt npad][nout_a].
 template <int EPI>
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const TcArgs a) {
     pdl_trigger();
@@ -429,7 +537,7 @@ __global__ void __launch_bounds__(256) tc_reduce_kernel(const TcArgs a) {
         uint16_t q[TC_PLANES];
         tc_split(h, q);
 #pragma unroll
-        for (int i = 0; i < TC_PLANES; ++i) a.h[((size_t)i * a.npad + n) * w + col] = q[i];
+        for (int i = 0; i < TC_PLANES; ++i) a.h[((size_t)i * a.nrt * a.npad + n) * w + col] = q[i];
     }
 }
 
@@ -733,7 +841,8 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
         for (int k = t; k < D.d; k += PK_THREADS) {
             float h = 0.f;
 #pragma unroll
-            for (int i = 0; i < TC_LM_PLANES; ++i) h += bf_to_f(q[i * plane + k]);
+            for (int i = 0; i < TC_PLANES; ++i)
+                if (i < a.npl) h += bf_to_f(q[i * plane + k]);
             hrow[k] = h;
         }
     }
@@ -932,8 +1041,8 @@ static bool encode2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t 
 
 bool tc_encode_weight(CUtensorMap *m, const void *w, int rows, int K) { return encode2d(m, w, K, rows, 128); }
 bool tc_encode_rows(CUtensorMap *m, const void *x, int rows, int npad, int K) { return encode2d(m, x, K, rows, npad); }
-bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, int npad, int K) {
-    return encode2d(m, x, K, (uint64_t)planes * npad, npad);
+bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, const TcTiles &t, int K) {
+    return encode2d(m, x, K, (uint64_t)planes * t.rows(), t.npad);
 }
 
 static int tc_stages(int npad, int planes, int na) {
@@ -982,8 +1091,8 @@ static cudaError_t pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t sme
 #ifndef OSP_TC_MIN_KB
 #define OSP_TC_MIN_KB 1   // k-blocks (of 64) per range at least: fewer, longer ranges write fewer partials
 #endif
-int tc_nsplit(int nout, int K, int sms) {
-    const int tiles = (nout + 127) / 128, nkb = K / 64;
+int tc_nsplit(int nout, int K, int nrt, int sms) {
+    const int tiles = (nout + 127) / 128 * nrt, nkb = K / 64;
     // at most one item per CTA slot: one item more than the slots would take two
     // item times for barely more than one wave of work
     int want = OSP_TC_CTAS_PER_SM * sms / tiles;
@@ -1003,17 +1112,20 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
                        cudaStream_t s, bool *planes_done, const QkvPostArgs *rope) {
     TcArgs a = a_in;
     if (planes_done) *planes_done = false;
-    if (a.npad % 16 || a.npad < 16 || a.npad > TC_MAX_ROWS || a.K % 64 || a.R > a.npad) return cudaErrorInvalidValue;
+    if (a.nrt < 1) a.nrt = 1;
+    if (a.npad % 16 || a.npad < 16 || a.npad > TC_TILE_ROWS || a.K % 64 || a.R > (long long)a.nrt * a.npad)
+        return cudaErrorInvalidValue;
     if (a.nout_a < 1 || a.nout_a > a.nout || (a.nout_a < a.nout && a.nout_a % 128)) return cudaErrorInvalidValue;
     if (a.epi == TC_GLU && (a.nout != 2 * a.nout_a || !a.part || !a.h)) return cudaErrorInvalidValue;
     const int nkb = a.K / 64;
     if (a.epi == TC_LM && (!a.lm_part || a.lm_nsub != (a.nout + TC_LM_GROUP - 1) / TC_LM_GROUP))
         return cudaErrorInvalidValue;
-    a.nsplit = a.part && a.epi != TC_LM ? tc_nsplit(a.nout, a.K, sms) : 1;   // the LM epilogue needs whole sums
+    a.nsplit = a.part && a.epi != TC_LM ? tc_nsplit(a.nout, a.K, a.nrt, sms) : 1;   // the LM epilogue needs whole sums
     if ((long long)a.nsplit * a.R * a.nout > a.part_cap) a.nsplit = 1;
     if (a.epi == TC_GLU && (long long)a.nsplit * a.R * a.nout > a.part_cap) return cudaErrorInvalidValue;
     a.kbps = (nkb + a.nsplit - 1) / a.nsplit;
-    a.segkb = OSP_TC_SEGKB;
+    a.sep = a.planes > 1;   // (0.1 % of a call, for a third of the accumulators' error)
+    a.segkb = a.fine ? OSP_TC_SEGKB_FINE : OSP_TC_SEGKB;
     constexpr int tmem_cols = 512 / OSP_TC_CTAS_PER_SM;
     // the LM head takes OSP_TC_LM_NA weight tiles per stage when two stages fit
     // and the double-buffered accumulators fit TMEM in one segment (the LM head's
@@ -1021,15 +1133,14 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     // per plane)
     int na = 1;
     if (a.epi == TC_LM && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA) >= 2 &&
-        2 * OSP_TC_LM_NA * a.npad <= tmem_cols && a.kbps <= 32) {
+        2 * OSP_TC_LM_NA * a.npad <= tmem_cols && a.kbps <= 32 && a.planes <= TC_LM_PLANES) {
         na = OSP_TC_LM_NA;
         a.segkb = a.kbps;
     }
     const int nst = tc_stages(a.npad, a.planes, na);
     if (nst < 2) return cudaErrorInvalidValue;
-    const int nseg = (a.kbps + a.segkb - 1) / a.segkb;
-    if ((nseg > 1 ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
-    const int items = (a.nout + 128 * na - 1) / (128 * na) * a.nsplit;
+    if ((na == 1 && a.sep ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
+    const int items = (a.nout + 128 * na - 1) / (128 * na) * a.nrt * a.nsplit;
     const int grid = items < OSP_TC_CTAS_PER_SM * sms ? items : OSP_TC_CTAS_PER_SM * sms;
     const size_t smem = tc_smem_bytes(a.npad, a.planes, na);
     cudaError_t e;

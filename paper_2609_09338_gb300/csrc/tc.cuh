@@ -1,10 +1,11 @@
 // Batched-row draft step on the 5th-generation tensor cores (tcgen05): the
 // projections of Sec. 3.3 (Eq. 1-3, the MLP and the LM head) as streamed
-// swap-AB GEMMs, Y[R x Nout] = X[R x K] . W[Nout x K]^T, for 3..80 rows.
+// swap-AB GEMMs, Y[R x Nout] = X[R x K] . W[Nout x K]^T, for 3..4096 rows.
 //
 // Weights are the M = 128 operand, streamed tile by tile with 2-D TMA (128-byte
-// swizzle); the R activation rows are the N operand (padded to a multiple of
-// 16).  The LM head multiplies two weight tiles against each stage's operand
+// swizzle); the R activation rows are the N operand, in equal tiles of at most
+// 80 rows (padded to a multiple of 16).  The row tiles of one weight tile are
+// adjacent work items, so all but the first read the weights from L2.  The LM head multiplies two weight tiles against each stage's operand
 // planes (twice the weight bytes in flight per byte of operand reloaded).  Activations are float32 between kernels; for the tensor cores each is
 // split into three bf16 planes, q0 = bf16(x), q1 = bf16(x - q0), q2 =
 // bf16(x - q0 - q1), and every k-step issues one MMA per plane into the same
@@ -35,13 +36,34 @@ constexpr int TC_LM_GROUP = 32;    // vocabulary ids per LM-head partial (one ep
 // 2^-17 |h_k| |W_jk|, about 5e-6 at d 1024, the float32 GEMV's own level; the
 // smaller stage lets three weight tiles per CTA be in flight instead of two.
 constexpr int TC_LM_PLANES = 2;
+// Batches of more than TC_TILE_ROWS sequences keep all three planes: their
+// logits were float32 dot products before they ran on the tensor cores, and two
+// planes would put q(token) 1e-4 off at logits of 40 (three: 1e-6).
 
-constexpr int TC_MAX_ROWS = 80;    // activation rows per GEMM: three accumulators fit a CTA's 256 TMEM columns
+constexpr int TC_TILE_ROWS = 80;   // activation rows per tile: three accumulators fit a CTA's 256 TMEM columns
+constexpr int TC_MAX_ROWS = 4096;  // rows of a call on the tensor cores (beyond: the CUDA-core GEMV, whose workspace is smaller)
+constexpr int TC_GROUP_ROWS = 512; // rows of one pass of block drafting
 constexpr int TC_PLANES = 3;       // bf16 planes of a float32 operand
+
+// A call's rows as equal tiles of at most TC_TILE_ROWS (the MMA's N, a multiple
+// of 16).  80 rows a tile keep two CTAs per SM (two accumulators of 80 columns
+// and a running total in 256 TMEM columns, two stages of three planes in 100 KB).
+struct TcTiles {
+    int nrt, npad;     // row tiles, rows per tile
+    __host__ __device__ int rows() const { return nrt * npad; }   // rows of an operand plane
+};
+inline TcTiles tc_tiles(long long rows) {
+    TcTiles t;
+    t.nrt = (int)((rows + TC_TILE_ROWS - 1) / TC_TILE_ROWS);
+    if (t.nrt < 1) t.nrt = 1;
+    t.npad = (int)(((rows + t.nrt - 1) / t.nrt + 15) / 16 * 16);
+    return t;
+}
 
 struct TcArgs {
     int epi;           // TcEpi
-    int R, npad;       // rows, rows padded to a multiple of 16
+    int R;             // rows
+    int npad, nrt;     // rows per tile (a multiple of 16), row tiles; an operand plane has nrt * npad rows
     int K;             // reduction length (multiple of 64)
     int nout;          // output features (tiles of 128, the last one may be partial)
     int nout_a;        // features [0, nout_a) from the first weight map, the rest from the second
@@ -49,7 +71,7 @@ struct TcArgs {
     float *y;          // TC_STORE: [R][ldy] float32 output
     int ldy;
     float *x;          // TC_RESID: [R][ldy] float32, +=
-    uint16_t *h;       // TC_GLU: [TC_PLANES][npad][nout_a] bf16 planes of silu(gate) * up
+    uint16_t *h;       // TC_GLU: [TC_PLANES][nrt npad][nout_a] bf16 planes of silu(gate) * up
     int32_t *status;
     // TC_LM: partials [R][lm_nsub] (lm_nsub = ceil(nout / 32)), 1/T (1 for greedy)
     float4 *lm_part;
@@ -72,13 +94,15 @@ struct TcArgs {
     long long part_cap;   // floats available in part
     int nsplit, kbps;     // set by launch_tc
     int segkb;            // k-blocks per accumulation segment, set by launch_tc
+    bool fine;            // short accumulation segments (calls of more rows than a tile, block drafting aside)
+    bool sep;             // planes after the first accumulate by themselves, set by launch_tc
 };
 
 // Host side.  Tensor maps: weights [rows][K] bf16 with a 64 x 128 box, operand
-// planes [planes * npad][K] bf16 with a 64 x npad box, both 128-byte swizzled.
+// planes [planes * tiles.rows()][K] bf16 with a 64 x npad box, both 128-byte swizzled.
 bool tc_available();   // the driver exposes tensor-map encoding and the device is sm_100+
 bool tc_encode_weight(CUtensorMap *m, const void *w, int rows, int K);
-bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, int npad, int K);
+bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, const TcTiles &t, int K);
 // a single bf16 plane of `rows` rows read in place (rows past `rows` read as zero)
 bool tc_encode_rows(CUtensorMap *m, const void *x, int rows, int npad, int K);
 size_t tc_smem_bytes(int npad, int planes, int na);
@@ -86,9 +110,9 @@ cudaError_t tc_set_attributes();
 // SwiGLU runs as one GEMM over the gate rows (map wa) and the up rows (map wb),
 // nout = 2 nout_a; its partials always go to `part`, and the reduction forms
 // silu(gate) * up.  Outputs narrower than the CTA slots are split along K
-// (tc_nsplit ranges per 128-feature tile); the float32 partials are then summed
+// (tc_nsplit ranges per 128-feature, npad-row tile); the float32 partials are then summed
 // in range order by a reduction kernel that applies the epilogue.
-int tc_nsplit(int nout, int K, int sms);
+int tc_nsplit(int nout, int K, int nrt, int sms);
 cudaError_t launch_tc(const TcArgs &a, const CUtensorMap &wa, const CUtensorMap &xm, int sms, cudaStream_t s);
 // *planes_done (when given) tells whether the reduction did the follow-up work:
 // wrote the pl_* planes (TC_RESID), or RoPE and the K/V write of `rope`
@@ -99,7 +123,8 @@ cudaError_t launch_tc2(const TcArgs &a, const CUtensorMap &wa, const CUtensorMap
                        cudaStream_t s, bool *planes_done = nullptr, const QkvPostArgs *rope = nullptr);
 
 // Operand preparation: rows of float32 (optionally RMS-normalised with a bf16
-// gain) written as bf16 planes [TC_PLANES][npad][ld] starting at column col0.
+// gain) written as bf16 planes [npl][npad][ld] (npad: the rows of a plane,
+// TcTiles::rows()) starting at column col0.
 struct PlaneArgs {
     const float *src;          // row r at src + src_row(r) * d
     const uint16_t *gain;      // RMSNorm gain, or null for a plain copy
@@ -150,7 +175,7 @@ struct LmPickArgs {
     const float4 *part;        // [B][nsub] TC_LM partials
     int nsub;
     const uint16_t *planes;    // [TC_PLANES][npad][d] bf16 planes of the LM head's rows
-    int npad;
+    int npad, npl;             // rows of a plane, planes
     const uint16_t *W;         // LM head [V][d]
     float temperature;
     const float *u_draft;
