@@ -1131,12 +1131,11 @@ extern "C" int osprey_verify_tree(int B, int K, int topk, int V, int logits_dtyp
 
 // ------------------------------------------------------------------ logits-free verify
 // Workspace: the verify layout (counters, partials, decisions, chunk sums), then
-// for one group of up to TC_TILE_ROWS sequences the gathered kept states
-// [rows][d] float, their operand planes [TC_PLANES][npad][d] bf16, the
+// for one group of up to TC_TILE_ROWS sequences the operand planes of their
+// decision rows [TC_PLANES][npad][d] bf16, the
 // recomputed decision-row logits [rows][V] float (the draft step's LM-head GEMM:
 // the same operand planes, unsplit, so the rows come out the same).
 struct HiddenWs {
-    float *rows;
     uint16_t *planes;
     float *z;
     int group, npad;
@@ -1147,15 +1146,12 @@ static size_t verify_hidden_layout(const osprey_ctx *ctx, int B, int K, VerifyAr
     size_t off = align256(verify_workspace_layout(B, K, D.V, a, base));
     const int group = B < TC_TILE_ROWS ? B : TC_TILE_ROWS;
     const int npad = (group + 15) / 16 * 16;
-    const size_t o_r = off;
-    off = align256(off + 4ull * group * D.d);
     const size_t o_p = off;
     off = align256(off + 2ull * TC_PLANES * npad * D.d);
     const size_t o_z = off;
     off = align256(off + 4ull * group * D.V);
     if (hw && base) {
         char *p = (char *)base;
-        hw->rows = (float *)(p + o_r);
         hw->planes = (uint16_t *)(p + o_p);
         hw->z = (float *)(p + o_z);
         hw->group = group;
@@ -1228,10 +1224,11 @@ extern "C" int osprey_verify_hidden(osprey_ctx *ctx, int B, int K, int logits_dt
         const int n = B - b0 < hw.group ? B - b0 : hw.group;
         const int npad = (n + 15) / 16 * 16;
         // 2. the kept state of each decision row -> final RMSNorm -> bf16 planes
-        if ((e = launch_decision_rows(a.dec, draft_hidden, K, D.d, b0, n, hw.rows, s)) != cudaSuccess)
-            return cuda_fail(e, "decision-row launch");
         PlaneArgs pl{};
-        pl.src = hw.rows;
+        pl.src = draft_hidden;
+        pl.dec = (const Decision *)a.dec;
+        pl.dec_b0 = b0;
+        pl.dec_K = K;
         pl.gain = (const uint16_t *)ctx->w.final_norm;
         pl.eps = D.eps;
         pl.d = D.d;

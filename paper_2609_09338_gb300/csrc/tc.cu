@@ -633,7 +633,11 @@ __global__ void __launch_bounds__(256) planes_kernel(const PlaneArgs a) {
     pdl_wait();
     bool act;
     int srow;
-    if (a.last_of_seq) {
+    if (a.dec) {
+        const int dr = __ldcg(&a.dec[a.dec_b0 + r].r);
+        act = dr >= 0 && dr < a.dec_K;
+        srow = act ? (a.dec_b0 + r) * a.dec_K + dr : 0;
+    } else if (a.last_of_seq) {
         act = !a.valid || a.valid[r];
         srow = act ? r * a.max_new + a.nnew[r] - 1 : 0;
     } else {

@@ -23,6 +23,7 @@
 #include <stdint.h>
 
 #include "draft.cuh"
+#include "internal.h"
 
 namespace osp {
 
@@ -139,6 +140,11 @@ struct PlaneArgs {
     int npl;                   // planes written (0: TC_PLANES)
     const float *src2;         // optional second source, same rows, written plain at column col2
     int col2;
+    // when set (logits-free verification): row r is the kept state of sequence
+    // b0 + r at its decision row, src row (b0 + r) K + dec[b0 + r].r; zeros when
+    // every draft token was accepted
+    const Decision *dec;
+    int dec_b0, dec_K;
 };
 cudaError_t launch_planes(const PlaneArgs &a, cudaStream_t s);
 

@@ -466,6 +466,7 @@ static bool hidden_vec(const VerifyArgs &a) {
 }
 
 cudaError_t launch_verify_hidden_stats(const VerifyArgs &a, cudaStream_t s) {
+    if (verify_stream_mode(a)) return launch_verify_stream(a, VS_HIDDEN_STATS, s);
     const unsigned g1 = (unsigned)a.nch * (a.K + 1) * a.B;
     const bool vec = hidden_vec(a);
     if (a.dtype == OSPREY_F32) {
@@ -482,6 +483,8 @@ cudaError_t launch_verify_hidden_stats(const VerifyArgs &a, cudaStream_t s) {
 cudaError_t launch_verify_hidden_sample(const VerifyArgs &a_in, int b0, int n, cudaStream_t s) {
     VerifyArgs a = a_in;
     a.b0 = b0;
+    a.n_group = n;
+    if (verify_stream_mode(a)) return launch_verify_stream(a, VS_HIDDEN_SAMPLE, s);
     const unsigned g2 = (unsigned)a.nch * n;
     const bool vec = hidden_vec(a);
     if (a.dtype == OSPREY_F32) {
@@ -495,31 +498,8 @@ cudaError_t launch_verify_hidden_sample(const VerifyArgs &a_in, int b0, int n, c
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(256) decision_rows_kernel(const Decision *dec, const float *hidden, int K, int d,
-                                                            int b0, float *dst) {
-    const int j = blockIdx.x, b = b0 + j;
-    const int r = dec[b].r;   // written by verify_stats
-    const bool act = r >= 0 && r < K;
-    const float *src = hidden + ((size_t)b * K + (act ? r : 0)) * d;
-    float *out = dst + (size_t)j * d;
-    for (int k = threadIdx.x; k < d; k += blockDim.x) out[k] = act ? src[k] : 0.f;
-}
-
-cudaError_t launch_decision_rows(const void *dec, const float *hidden, int K, int d, int b0, int n, float *dst,
-                                 cudaStream_t s) {
-    decision_rows_kernel<<<n, 256, 0, s>>>((const Decision *)dec, hidden, K, d, b0, dst);
-    count_launch();
-    return cudaGetLastError();
-}
-
 cudaError_t launch_verify(const VerifyArgs &a, cudaStream_t s) {
-    if (verify_stream_ok(a)) {
-        int dev = 0, sms = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        return launch_verify_stream(a, sms, s);
-    }
+    if (verify_stream_mode(a)) return launch_verify_stream(a, VS_WHOLE, s);
     const bool f32 = a.dtype == OSPREY_F32;
     const int W = f32 ? 4 : 8;
     bool vec = (a.V % W) == 0 && ((uintptr_t)a.target % 16) == 0 &&

@@ -1,5 +1,5 @@
-// Streamed speculative-sampling verification (Sec. 3.1) for 16-byte-aligned
-// logits: persistent blocks (8 consumer warps + 1 producer warp, three per SM)
+// Streamed speculative-sampling verification (Sec. 3.1) for logits whose base is
+// 16-byte aligned: persistent blocks (8 consumer warps + 1 producer warp, three per SM)
 // pull 4 KB chunks of the target row (and of the draft row, for rows i < K)
 // through an 8-slot shared-memory ring with 1-D bulk copies (TMA): the copies
 // of the other warps' tiles stay in flight while a warp works on its own, 24
@@ -23,9 +23,22 @@
 //   order, loads the chosen chunk (two halves of loads in flight) and walks its
 //   8 segments, then its lanes, then one lane's elements (inverse CDF at
 //   u_sample[r]).
+// Rows that are no multiple of 16 bytes (UA): a copy takes the aligned 16-byte
+// vectors around its ids, so a row's ids start `m` elements into the slot, m the
+// row's own misalignment.  The sums mask the vectors at the ends; the draw, which
+// pairs the target and draft logits of an id (their m differ), reads elements.
+// V 151643, B 32, K 5, float32 (213 MB): 66 us; with one element per load
+// straight from global memory 88.
+// Logits-free form (HID): vs_stats reads the target rows only and the decision
+// takes q_i(x_i) and (M, log S) from the draft step; vs_sample takes a group's
+// draft rows from `zrec` (float32 whatever the target's type).  V 200064, B 64,
+// K 8, bf16: 176 us a call, of which the target's 230 MB take 45; with unstreamed
+// kernels for the rows and two launches for the decision rows' operand 238.
 // Both kernels are launched as programmatic dependents: barrier set-up overlaps
 // the previous kernel's tail, and every global read follows griddepcontrol.wait.
 #include <math.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -39,9 +52,6 @@ namespace osp {
 
 #ifndef OSP_VS_NST
 #define OSP_VS_NST 8   // ring slots per block: 3 x 8 x 8 KB of the SM's shared memory
-#endif
-#ifndef OSP_VS_EARLY
-#define OSP_VS_EARLY 0   // 1: a consumer copies both rows of its tile to registers and frees the slot first
 #endif
 #ifndef OSP_VS_ROWB
 #define OSP_VS_ROWB 4096   // bytes of one row chunk (the workspace holds 4 KB float32 chunks at least)
@@ -59,7 +69,6 @@ static_assert(VS_ROWB % 4096 == 0, "row chunks are whole multiples of 4 KB");
 // (vs_wait_slot).  That wait is itself exact because use u - 2 belongs to the
 // same warp, which has freed it: 2 NST must be a multiple of CW.
 static_assert((2 * VS_NST) % VS_CW == 0, "ring slots: 2 x slots must be a multiple of the consumer warps");
-constexpr int VS_SLOT = 2 * VS_ROWB;       // target chunk + draft chunk
 constexpr int VS_NV = VS_ROWB / 16 / 32;   // 16-byte vectors per lane per row chunk (8)
 
 // 2^x on the special-function unit (PTX ex2.approx, flush-to-zero)
@@ -69,6 +78,45 @@ __device__ __forceinline__ float vs_ex2(float x) {
     return y;
 }
 constexpr float VS_LOG2E = 1.4426950408889634f;
+
+// One row chunk of EL elements of type U in a slot: its bytes, and with UA one
+// vector more at each end.
+template <typename U, int EL, bool UA>
+constexpr int vs_region() { return EL * (int)sizeof(U) + (UA ? 32 : 0); }
+
+// The 16-byte vectors of elements [e0, e0 + nel) of a tensor of `total` elements.
+// UA: from the aligned vector before e0 to the one after the end; where that
+// would pass the tensor's end, the last elements are copied by this thread.
+template <typename U>
+struct VsSpan {
+    const U *src;
+    uint32_t bytes;
+    int tail, tail_at;   // elements after `bytes`, and where they go
+};
+template <typename U, bool UA>
+__device__ __forceinline__ VsSpan<U> vs_span(const U *base, long long total, long long e0, int nel) {
+    if (!UA) return VsSpan<U>{base + e0, (uint32_t)(nel * sizeof(U)), 0, 0};
+    constexpr int VW = 16 / sizeof(U);
+    const int m = (int)(e0 % VW);
+    long long n = (m + nel + VW - 1) / VW * VW;
+    int tail = 0;
+    if (e0 - m + n > total) {
+        n -= VW;
+        tail = (int)(m + nel - n);
+    }
+    return VsSpan<U>{base + (e0 - m), (uint32_t)(n * sizeof(U)), tail, (int)n};
+}
+template <typename U>
+__device__ __forceinline__ void vs_copy(uint8_t *dst, const VsSpan<U> &s, uint64_t *bar, uint64_t pol) {
+    if (s.bytes) bulk_g2s_hint(dst, s.src, s.bytes, bar, pol);
+}
+// before the arrival that publishes the slot
+template <typename U>
+__device__ __forceinline__ void vs_copy_tail(uint8_t *dst, const VsSpan<U> &s) {
+    for (int i = 0; i < s.tail; ++i) ((U *)dst)[s.tail_at + i] = s.src[s.tail_at + i];
+    // a later bulk copy into this slot comes after these stores
+    if (s.tail) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
 
 // Consumer wait for tile j of a block: the slot's previous use (another warp's
 // tile) freed, then tile j's copy complete.  False when a bounded wait ran out.
@@ -113,10 +161,10 @@ template <> struct VsT<float> {
         f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);
         f[2] = __uint_as_float(v.z); f[3] = __uint_as_float(v.w);
     }
-    __device__ static float vmax(const uint4 (&r)[VS_NV]) {
+    template <int N> __device__ static float vmax(const uint4 (&r)[N]) {
         float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-        for (int k = 0; k < VS_NV; ++k) {
+        for (int k = 0; k < N; ++k) {
             m[0] = fmaxf(m[0], __uint_as_float(r[k].x)); m[1] = fmaxf(m[1], __uint_as_float(r[k].y));
             m[2] = fmaxf(m[2], __uint_as_float(r[k].z)); m[3] = fmaxf(m[3], __uint_as_float(r[k].w));
         }
@@ -134,10 +182,10 @@ template <> struct VsT<uint16_t> {
         return d;
     }
     // max of the packed pairs, widened once at the end
-    __device__ static float vmax(const uint4 (&r)[VS_NV]) {
+    template <int N> __device__ static float vmax(const uint4 (&r)[N]) {
         uint32_t m[4] = {r[0].x, r[0].y, r[0].z, r[0].w};
 #pragma unroll
-        for (int k = 1; k < VS_NV; ++k) {
+        for (int k = 1; k < N; ++k) {
             m[0] = max2(m[0], r[k].x); m[1] = max2(m[1], r[k].y);
             m[2] = max2(m[2], r[k].z); m[3] = max2(m[3], r[k].w);
         }
@@ -156,20 +204,23 @@ __device__ __forceinline__ void vs_mask(uint4 (&r)[VS_NV], int lane, int nel) {
         if ((lane + 32 * k) * L::VW >= nel) r[k] = make_uint4(L::NEG, L::NEG, L::NEG, L::NEG);
 }
 
-// Sum over the lane's vectors of 2^(x*c - mc) = exp((x - m) / T) with c =
-// log2(e)/T and mc = m*c.
-template <typename T>
-__device__ __forceinline__ float vs_sum_exp(const uint4 (&r)[VS_NV], float c, float mc) {
+// Sum over the lane's vectors of exp((x - m) / T) = 2^((x - m) c), c = log2(e)/T.
+// SUB: the difference first, which is exact near the maximum; else as
+// 2^(x c - m c), one operation less, off by the rounding of m c (1e-6 where
+// logits reach 40).
+template <typename T, bool SUB, int N>
+__device__ __forceinline__ float vs_sum_exp(const uint4 (&r)[N], float c, float m) {
     using L = VsT<T>;
+    const float mc = m * c;
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-    for (int k = 0; k < VS_NV; ++k) {
+    for (int k = 0; k < N; ++k) {
         float f[L::VW];
         L::unpack(r[k], f);
 #pragma unroll
         for (int e = 0; e < L::VW; e += 2) {
-            s0 += vs_ex2(fmaf(f[e], c, -mc));
-            s1 += vs_ex2(fmaf(f[e + 1], c, -mc));
+            s0 += vs_ex2(SUB ? (f[e] - m) * c : fmaf(f[e], c, -mc));
+            s1 += vs_ex2(SUB ? (f[e + 1] - m) * c : fmaf(f[e + 1], c, -mc));
         }
     }
     return s0 + s1;
@@ -179,10 +230,38 @@ __device__ __forceinline__ float vs_logit(const void *base, int dtype, size_t i)
     return dtype == OSPREY_F32 ? __ldg((const float *)base + i) : bf_to_f(__ldg((const uint16_t *)base + i));
 }
 
-// Copy one row chunk (lane's 8 vectors, interleaved by 32 lanes) from the ring.
-__device__ __forceinline__ void vs_stage(const uint8_t *chunk, int lane, uint4 (&r)[VS_NV]) {
+// Copy one row chunk (lane's 8 vectors, interleaved by 32 lanes) from the ring;
+// elements outside the row's ids read as -inf.  UA: the ids start at element m,
+// and a 9th vector (lane 0's) holds what m pushes past the 8th.
+template <typename T, bool UA>
+__device__ __forceinline__ void vs_stage(const uint8_t *chunk, int lane, int m, int nel, uint4 (&r)[VS_NV + UA]) {
+    using L = VsT<T>;
+    if constexpr (!UA) {
 #pragma unroll
-    for (int k = 0; k < VS_NV; ++k) r[k] = ((const uint4 *)chunk)[lane + 32 * k];
+        for (int k = 0; k < VS_NV; ++k) r[k] = ((const uint4 *)chunk)[lane + 32 * k];
+        if (nel != L::EL) vs_mask<T>(r, lane, nel);
+    } else {
+        const int end = m + nel;
+#pragma unroll
+        for (int k = 0; k <= VS_NV; ++k) {
+            const int e0 = (lane + 32 * k) * L::VW;
+            uint4 v = make_uint4(L::NEG, L::NEG, L::NEG, L::NEG);
+            if (e0 < end && (k < VS_NV || lane == 0)) {
+                v = ((const uint4 *)chunk)[lane + 32 * k];
+                if (e0 < m || e0 + L::VW > end) {   // a vector at an end of the row
+                    uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < L::VW; ++e)
+                        if (e0 + e < m || e0 + e >= end) {
+                            if constexpr (sizeof(T) == 4) w[e] = L::NEG;
+                            else w[e / 2] = (w[e / 2] & (e & 1 ? 0xffffu : 0xffff0000u)) | (L::NEG & (e & 1 ? 0xffff0000u : 0xffffu));
+                        }
+                    v = make_uint4(w[0], w[1], w[2], w[3]);
+                }
+            }
+            r[k] = v;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -247,22 +326,28 @@ __device__ void vs_row_reduce(const VerifyArgs &a, size_t row) {
 
 // The warp that completes sequence b: lane i holds row i's summary; accept
 // while u_i < p_i(x_i) / q_i(x_i) (greedy: while argmax p_i == x_i).
-template <bool GREEDY>
+template <bool GREEDY, bool HID>
 __device__ void vs_decide(const VerifyArgs &a, int b) {
     const int lane = threadIdx.x & 31;
     const int K = a.K, V = a.V;
     const int xi = lane < K ? __ldg(a.tokens + (size_t)b * K + lane) : 0;
     const bool ok = __all_sync(0xffffffffu, lane >= K || (xi >= 0 && xi < V));
     // everything below but the summaries is independent of the reduction: load it together
-    float zpx = 0.f, zqx = 0.f, ua = 0.f;
+    float zpx = 0.f, zqx = 0.f, ua = 0.f, hM = 0.f, hS = 0.f;
     if (!GREEDY && ok && lane < K) {
         zpx = vs_logit(a.target, a.dtype, ((size_t)b * (K + 1) + lane) * V + xi);
-        zqx = vs_logit(a.draft, a.dtype, ((size_t)b * K + lane) * V + xi);
+        if (HID) {   // the draft step's q_i(x_i) and (M, log S)
+            zqx = __ldg(a.qx_in + (size_t)b * K + lane);
+            hM = __ldg(a.stats_in + ((size_t)b * K + lane) * 2);
+            hS = __ldg(a.stats_in + ((size_t)b * K + lane) * 2 + 1);
+        } else {
+            zqx = vs_logit(a.draft, a.dtype, ((size_t)b * K + lane) * V + xi);
+        }
         ua = __ldg(a.u_accept + (size_t)b * K + lane);
     }
     const float4 rs = lane <= K ? __ldcg((const float4 *)a.rowstat + (size_t)b * (K + 1) + lane)
                                 : make_float4(0.f, 1.f, 0.f, 1.f);
-    const float rMp = rs.x, rSp = rs.y, rMq = rs.z, rSq = rs.w;
+    const float rMp = rs.x, rSp = rs.y, rMq = HID ? hM : rs.z, rSq = HID ? expf(hS) : rs.w;
     const int ram = __float_as_int(rs.y);
     int32_t *out = a.out_tokens + (size_t)b * (K + 1);
     uint8_t *fl = a.flags + (size_t)b * (K + 1);
@@ -283,7 +368,7 @@ __device__ void vs_decide(const VerifyArgs &a, int b) {
     } else if (lane < K) {
         const float invT = 1.f / a.temperature;
         const float px = expf(zpx * invT - rMp) / rSp;
-        const float qx = expf(zqx * invT - rMq) / rSq;
+        const float qx = HID ? zqx : expf(zqx * invT - rMq) / rSq;
         if (a.probs) {
             a.probs[((size_t)b * K + lane) * 2 + 0] = px;
             a.probs[((size_t)b * K + lane) * 2 + 1] = qx;
@@ -325,20 +410,22 @@ __device__ __forceinline__ bool vs_arrive(int *counter, int pend, int total) {
 
 // A warp finished `pend` tiles of row `row`: count them; the warp completing
 // the row summarises it, and the one completing the sequence decides.
-template <bool GREEDY>
+template <bool GREEDY, bool HID>
 __device__ __forceinline__ void vs_row_done(const VerifyArgs &a, size_t row, int pend) {
     if (!vs_arrive(a.trow + row, pend, a.nch3)) return;
     vs_row_reduce<GREEDY>(a, row);
     const int b = (int)(row / (a.K + 1));
-    if (vs_arrive(a.ticket1 + b, 1, a.K + 1)) vs_decide<GREEDY>(a, b);
+    if (vs_arrive(a.ticket1 + b, 1, a.K + 1)) vs_decide<GREEDY, HID>(a, b);
 }
 
-template <typename T, bool GREEDY>
+template <typename T, bool GREEDY, bool HID, bool UA>
 __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_stats(const VerifyArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[VS_NST], empty[VS_NST];
     __shared__ int s_abort;
     using L = VsT<T>;
+    constexpr int REG = vs_region<T, L::EL, UA>(), SLOT = 2 * REG;   // target chunk + draft chunk
+    constexpr bool SUB = HID || UA;   // the exponent's form that these calls have always had
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = a.K, V = a.V, nch = a.nch3;
     const long long NT = (long long)a.B * (K + 1) * nch;
@@ -370,21 +457,27 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_stats(const VerifyA
                 }
                 const int b = cur.b, i = cur.i, c = cur.c;
                 const int nel = min(L::EL, V - c * L::EL);
-                uint8_t *dst = smem + (size_t)slot * VS_SLOT;
+                uint8_t *dst = smem + (size_t)slot * SLOT;
                 issued = j + 1;
                 if (nel <= 0) {   // never issue a copy outside the row
                     set_status(a.status, OSPREY_ERR_INVALID_ARG);
                     mbar_arrive_expect_tx(&full[slot], 0);
                     continue;
                 }
-                const uint32_t bytes = (uint32_t)nel * sizeof(T);
-                const bool has_q = !GREEDY && i < K;
-                mbar_arrive_expect_tx(&full[slot], has_q ? 2 * bytes : bytes);
-                bulk_g2s_hint(dst, (const T *)a.target + ((size_t)b * (K + 1) + i) * V + (size_t)c * L::EL, bytes,
-                              &full[slot], pol);
+                const bool has_q = !GREEDY && !HID && i < K;
+                const long long rp = (long long)b * (K + 1) + i, rq = (long long)b * K + i;
+                const VsSpan<T> sp = vs_span<T, UA>((const T *)a.target, (long long)a.B * (K + 1) * V,
+                                                    rp * V + (long long)c * L::EL, nel);
+                VsSpan<T> sq{nullptr, 0, 0, 0};
                 if (has_q)
-                    bulk_g2s_hint(dst + VS_ROWB, (const T *)a.draft + ((size_t)b * K + i) * V + (size_t)c * L::EL,
-                                  bytes, &full[slot], pol);
+                    sq = vs_span<T, UA>((const T *)a.draft, (long long)a.B * K * V, rq * V + (long long)c * L::EL, nel);
+                if (UA) {
+                    vs_copy_tail(dst, sp);
+                    vs_copy_tail(dst + REG, sq);
+                }
+                mbar_arrive_expect_tx(&full[slot], sp.bytes + sq.bytes);
+                vs_copy(dst, sp, &full[slot], pol);
+                vs_copy(dst + REG, sq, &full[slot], pol);
             }
             if (s_abort)
                 for (int j = max(0, issued - VS_NST); j < issued; ++j)
@@ -403,7 +496,7 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_stats(const VerifyA
         const int i = cur.i, c = cur.c;
         const long long row = cur.row;
         if (row != cur_row) {
-            if (pend) vs_row_done<GREEDY>(a, (size_t)cur_row, pend);
+            if (pend) vs_row_done<GREEDY, HID>(a, (size_t)cur_row, pend);
             cur_row = row;
             pend = 0;
         }
@@ -416,58 +509,38 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_stats(const VerifyA
             break;
         }
         const int nel = min(L::EL, V - c * L::EL);
-        const bool whole = nel == L::EL;
-        const bool has_q = !GREEDY && i < K;
-        const uint8_t *chunk = smem + (size_t)slot * VS_SLOT;
+        const bool has_q = !GREEDY && !HID && i < K;
+        const uint8_t *chunk = smem + (size_t)slot * SLOT;
+        // the rows' misalignment in elements
+        const int mp = UA ? (int)(row * V % L::VW) : 0;
         // one row at a time through registers; the slot is freed after both
         float4 part;
-        uint4 rv[VS_NV];
-        vs_stage(chunk, lane, rv);
-        if (!whole) vs_mask<T>(rv, lane, nel);
+        uint4 rv[VS_NV + UA];
+        vs_stage<T, UA>(chunk, lane, mp, nel, rv);
         if (GREEDY) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[slot]);
             AM am{-INFINITY, 0x7fffffff};
 #pragma unroll
-            for (int k = 0; k < VS_NV; ++k) {
+            for (int k = 0; k < VS_NV + UA; ++k) {
                 float f[L::VW];
                 L::unpack(rv[k], f);
 #pragma unroll
                 for (int e = 0; e < L::VW; ++e)
-                    if (f[e] > am.v) am = AM{f[e], c * L::EL + (lane + 32 * k) * L::VW + e};
+                    if (f[e] > am.v) am = AM{f[e], c * L::EL + (lane + 32 * k) * L::VW + e - mp};
             }
             am = warp_am(am);
             part = make_float4(am.v, __int_as_float(am.i), 0.f, 0.f);
-        } else if (OSP_VS_EARLY) {
-            // both rows to registers, the slot freed, then the sums
-            uint4 rq[VS_NV];
-            if (has_q) {
-                vs_stage(chunk + VS_ROWB, lane, rq);
-                if (!whole) vs_mask<T>(rq, lane, nel);
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[slot]);
-            const float xp = L::vmax(rv);
-            const float sp = xp == -INFINITY ? 0.f : vs_sum_exp<T>(rv, cexp, xp * cexp);
-            float xq = -INFINITY, sq = 0.f;
-            if (has_q) {
-                xq = L::vmax(rq);
-                sq = xq == -INFINITY ? 0.f : vs_sum_exp<T>(rq, cexp, xq * cexp);
-            }
-            const MS p = vs_warp_ms(xp * invT, sp);
-            const MS q = has_q ? vs_warp_ms(xq * invT, sq) : MS{-INFINITY, 0.f};
-            part = make_float4(p.m, p.s, q.m, q.s);
         } else {
             // maxima of the raw logits (order is kept by the positive 1/T), then
             // sums of exp((z - max) / T)
             const float xp = L::vmax(rv);
-            const float sp = xp == -INFINITY ? 0.f : vs_sum_exp<T>(rv, cexp, xp * cexp);
+            const float sp = xp == -INFINITY ? 0.f : vs_sum_exp<T, SUB>(rv, cexp, xp);
             float xq = -INFINITY, sq = 0.f;
             if (has_q) {
-                vs_stage(chunk + VS_ROWB, lane, rv);
-                if (!whole) vs_mask<T>(rv, lane, nel);
+                vs_stage<T, UA>(chunk + REG, lane, UA ? (int)((row - cur.b) * V % L::VW) : 0, nel, rv);
                 xq = L::vmax(rv);
-                sq = xq == -INFINITY ? 0.f : vs_sum_exp<T>(rv, cexp, xq * cexp);
+                sq = xq == -INFINITY ? 0.f : vs_sum_exp<T, SUB>(rv, cexp, xq);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[slot]);
@@ -478,35 +551,72 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_stats(const VerifyA
         if (lane == 0) ((float4 *)a.tpart)[t0 + j] = part;
         ++pend;
     }
-    if (!aborted && pend) vs_row_done<GREEDY>(a, (size_t)cur_row, pend);
+    if (!aborted && pend) vs_row_done<GREEDY, HID>(a, (size_t)cur_row, pend);
 }
 
 // ---------------------------------------------------------------------------
-// Normalisers of the decision row in exp2 form: p(z) = 2^(z c - Mp log2 e) / Sp.
+__device__ __forceinline__ float vs_el(float x) { return x; }
+__device__ __forceinline__ float vs_el(uint16_t x) { return bf_to_f(x); }
+
+// Normalisers of the decision row: p(z) = exp(z / T - Mp) / Sp, as
+// 2^(z c - Mp log2 e), or with SUB as 2^((z / T - Mp) log2 e) (see vs_sum_exp).
 struct VsNorm {
-    float c, mcp, mcq, isp, isq;
+    float c, invT, mp, mq, mcp, mcq, isp, isq;
 };
 __device__ __forceinline__ VsNorm vs_norm(const Decision &d, float temperature) {
-    return VsNorm{VS_LOG2E / temperature, d.Mp * VS_LOG2E, d.Mq * VS_LOG2E, 1.f / d.Sp, 1.f / d.Sq};
+    return VsNorm{VS_LOG2E / temperature, 1.f / temperature, d.Mp, d.Mq, d.Mp * VS_LOG2E, d.Mq * VS_LOG2E, 1.f / d.Sp,
+                  1.f / d.Sq};
 }
 // p and the draw weight (max(0, p - q) on a rejection, p for the bonus draw),
 // computed the same way by the tile sums and by the final walk.
+template <bool SUB>
 __device__ __forceinline__ float vs_pw(float zp, float zq, const VsNorm &n, bool residual, float &p) {
-    p = vs_ex2(fmaf(zp, n.c, -n.mcp)) * n.isp;
-    return residual ? fmaxf(0.f, p - vs_ex2(fmaf(zq, n.c, -n.mcq)) * n.isq) : p;
+    p = vs_ex2(SUB ? fmaf(zp, n.invT, -n.mp) * VS_LOG2E : fmaf(zp, n.c, -n.mcp)) * n.isp;
+    return residual ? fmaxf(0.f, p - vs_ex2(SUB ? fmaf(zq, n.invT, -n.mq) * VS_LOG2E : fmaf(zq, n.c, -n.mcq)) * n.isq) : p;
 }
+template <bool SUB>
 __device__ __forceinline__ float vs_weight(float zp, float zq, const VsNorm &n, bool residual, bool use_p) {
     float p;
-    const float w = vs_pw(zp, zq, n, residual, p);
+    const float w = vs_pw<SUB>(zp, zq, n, residual, p);
     return use_p ? p : w;
 }
+
+// Ids v VW .. + VW - 1 of a chunk of `nel` ids (VW that of the target's type T):
+// loaded as they are, so that many loads in flight take few registers, and
+// widened by get(); zero where the chunk has none.
+template <typename T, typename U, bool UA>
+struct VsVec {
+    static constexpr int VW = VsT<T>::VW, PER = 16 / sizeof(U), NR = UA ? VW : VW / PER;
+    using R = std::conditional_t<UA, U, uint4>;
+    R r[NR];
+    __device__ __forceinline__ void load(const U *row, int v, int nel) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int e = v * VW + i * (VW / NR);
+            r[i] = e < nel ? __ldg((const R *)(row + e)) : R{};
+        }
+    }
+    __device__ __forceinline__ void get(float (&f)[VW]) const {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            if constexpr (UA) {
+                f[i] = vs_el(r[i]);
+            } else {
+                float p[PER];
+                VsT<U>::unpack(r[i], p);
+#pragma unroll
+                for (int e = 0; e < PER; ++e) f[i * PER + e] = p[e];
+            }
+        }
+    }
+};
 
 // The sampling warp of sequence b (inverse CDF at t = u_sample[r] * S over
 // ascending ids): pick the chunk by the chunk sums, then load the chunk once
 // and walk its 8 segments (segment k = the k-th vector of every lane, 32 x VW
 // consecutive ids), then the lanes of the chosen segment, then one lane's VW
 // elements.  Two dependent loads in all.
-template <typename T>
+template <typename T, typename TQ, bool HID, bool UA>
 __device__ void vs_pick(const VerifyArgs &a, int b, const Decision &d) {
     using L = VsT<T>;
     constexpr int CPL = 8;   // chunk sums a lane holds per round (256 chunks a round)
@@ -576,30 +686,35 @@ __device__ void vs_pick(const VerifyArgs &a, int b, const Decision &d) {
     // the chosen chunk, once: lane l holds vectors l + 32k, k < 8
     const size_t rowp = ((size_t)b * (K + 1) + r) * V + (size_t)chunk * L::EL;
     const size_t rowq = ((size_t)b * K + r) * V + (size_t)chunk * L::EL;
-    const uint4 *gp = (const uint4 *)((const T *)a.target + rowp);
-    const uint4 *gq = (const uint4 *)((const T *)a.draft + rowq);
-    const int nel = min(L::EL, V - chunk * L::EL);   // a multiple of VW (rows are 16-byte multiples)
-    // in two halves, so that the loads in flight stay in registers next to the
-    // walk's state (the kernel keeps two blocks per SM)
+    const T *gp = (const T *)a.target + rowp;
+    const TQ *gq = HID ? (const TQ *)a.zrec + (size_t)(b - a.b0) * V + (size_t)chunk * L::EL
+                       : (const TQ *)a.draft + rowq;
+    const int nel = min(L::EL, V - chunk * L::EL);   // a multiple of VW unless UA
+    auto inside = [&](int v) { return UA ? v * L::VW < nel : v * L::VW + L::VW <= nel; };
+    // a part at a time, so that the loads in flight stay in registers next to the
+    // walk's state (the kernel keeps three blocks per SM)
+    constexpr int HB = sizeof(T) == 2 && (UA || sizeof(TQ) == 4) ? VS_NV / 4 : VS_NV / 2;
     float seg[VS_NV];
 #pragma unroll
-    for (int h = 0; h < VS_NV; h += VS_NV / 2) {
-        uint4 vp[VS_NV / 2], vq[VS_NV / 2];
+    for (int h = 0; h < VS_NV; h += HB) {
+        VsVec<T, T, UA> vp[HB];
+        VsVec<T, TQ, UA> vq[HB];
 #pragma unroll
-        for (int k = 0; k < VS_NV / 2; ++k) {
-            const bool in = (lane + 32 * (h + k)) * L::VW < nel;
-            vp[k] = in ? __ldg(gp + lane + 32 * (h + k)) : make_uint4(0, 0, 0, 0);
-            vq[k] = in && residual ? __ldg(gq + lane + 32 * (h + k)) : make_uint4(0, 0, 0, 0);
+        for (int k = 0; k < HB; ++k) {
+            vp[k].load(gp, lane + 32 * (h + k), nel);
+            vq[k].load(gq, lane + 32 * (h + k), residual ? nel : 0);
         }
 #pragma unroll
-        for (int k = 0; k < VS_NV / 2; ++k) {
+        for (int k = 0; k < HB; ++k) {
             float f[L::VW], g[L::VW];
-            L::unpack(vp[k], f);
-            L::unpack(vq[k], g);
+            vp[k].get(f);
+            vq[k].get(g);
             float w = 0.f;
-            if ((lane + 32 * (h + k)) * L::VW < nel) {
+            const int v = lane + 32 * (h + k);
+            if (inside(v)) {
 #pragma unroll
-                for (int e = 0; e < L::VW; ++e) w += vs_weight(f[e], g[e], nrm, residual, fallback);
+                for (int e = 0; e < L::VW; ++e)
+                    if (!UA || v * L::VW + e < nel) w += vs_weight<HID || UA>(f[e], g[e], nrm, residual, fallback);
             }
             seg[h + k] = w;
         }
@@ -643,13 +758,18 @@ __device__ void vs_pick(const VerifyArgs &a, int b, const Decision &d) {
     if (lane == hl) {
         const int vi = hl + 32 * sk;
         float f[L::VW], g[L::VW];
-        L::unpack(__ldg(gp + vi), f);
-        if (residual) L::unpack(__ldg(gq + vi), g);
+        VsVec<T, T, UA> vp;
+        VsVec<T, TQ, UA> vq;
+        vp.load(gp, vi, nel);
+        vq.load(gq, vi, residual ? nel : 0);
+        vp.get(f);
+        vq.get(g);
         float cum = lane_before;
         int found = -1, lastp = 0;
 #pragma unroll
         for (int e = 0; e < L::VW; ++e) {
-            const float w = vs_weight(f[e], residual ? g[e] : 0.f, nrm, residual, fallback);
+            if (UA && vi * L::VW + e >= nel) break;
+            const float w = vs_weight<HID || UA>(f[e], residual ? g[e] : 0.f, nrm, residual, fallback);
             cum += w;
             if (w > 0.f) lastp = e;
             if (found < 0 && w > 0.f && t < cum) found = e;
@@ -664,15 +784,17 @@ __device__ void vs_pick(const VerifyArgs &a, int b, const Decision &d) {
     }
 }
 
-template <typename T>
+template <typename T, typename TQ, bool HID, bool UA>
 __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const VerifyArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full[VS_NST], empty[VS_NST];
     __shared__ int s_abort;
     using L = VsT<T>;
+    constexpr int REG = vs_region<T, L::EL, UA>(), SLOT = REG + vs_region<TQ, L::EL, UA>();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int K = a.K, V = a.V, nch = a.nch3;
-    const long long NT = (long long)a.B * nch;
+    const int b0 = HID ? a.b0 : 0, nseq = HID ? a.n_group : a.B;   // the sequences of this launch
+    const long long NT = (long long)nseq * nch;
     const long long t0 = NT * blockIdx.x / gridDim.x, t1 = NT * (blockIdx.x + 1) / gridDim.x;
     const int n = (int)(t1 - t0);
     const Decision *decs = (const Decision *)a.dec;
@@ -700,7 +822,7 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
                     atomicExch(&s_abort, 1);
                     break;
                 }
-                const int b = (int)cur.row, c = cur.c;
+                const int b = b0 + (int)cur.row, c = cur.c;
                 if (b != rb) {
                     r = __ldcg(&decs[b].r);
                     rb = b;
@@ -709,7 +831,7 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
                         r = -1;
                     }
                 }
-                uint8_t *dst = smem + (size_t)slot * VS_SLOT;
+                uint8_t *dst = smem + (size_t)slot * SLOT;
                 const int nel = min(L::EL, V - c * L::EL);
                 issued = j + 1;
                 if (r < 0 || nel <= 0) {   // nothing to copy: complete the slot's phase
@@ -717,14 +839,21 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
                     mbar_arrive_expect_tx(&full[slot], 0);
                     continue;
                 }
-                const uint32_t bytes = (uint32_t)nel * sizeof(T);
-                const bool has_q = r < K;
-                mbar_arrive_expect_tx(&full[slot], has_q ? 2 * bytes : bytes);
-                bulk_g2s_hint(dst, (const T *)a.target + ((size_t)b * (K + 1) + r) * V + (size_t)c * L::EL, bytes,
-                              &full[slot], pol);
-                if (has_q)
-                    bulk_g2s_hint(dst + VS_ROWB, (const T *)a.draft + ((size_t)b * K + r) * V + (size_t)c * L::EL,
-                                  bytes, &full[slot], pol);
+                const VsSpan<T> sp = vs_span<T, UA>((const T *)a.target, (long long)a.B * (K + 1) * V,
+                                                    ((long long)b * (K + 1) + r) * V + (long long)c * L::EL, nel);
+                VsSpan<TQ> sq{nullptr, 0, 0, 0};
+                if (r < K)
+                    sq = HID ? vs_span<TQ, UA>((const TQ *)a.zrec, (long long)nseq * V,
+                                               (long long)(b - b0) * V + (long long)c * L::EL, nel)
+                             : vs_span<TQ, UA>((const TQ *)a.draft, (long long)a.B * K * V,
+                                               ((long long)b * K + r) * V + (long long)c * L::EL, nel);
+                if (UA) {
+                    vs_copy_tail(dst, sp);
+                    vs_copy_tail(dst + REG, sq);
+                }
+                mbar_arrive_expect_tx(&full[slot], sp.bytes + sq.bytes);
+                vs_copy(dst, sp, &full[slot], pol);
+                vs_copy(dst + REG, sq, &full[slot], pol);
             }
             if (s_abort)
                 for (int j = max(0, issued - VS_NST); j < issued; ++j)
@@ -740,9 +869,10 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
     // at batch 1 (cause not identified)
     for (int j = warp; j < n; j += VS_CW) {
         const long long t = t0 + j;
-        const int b = (int)(t / nch), c = (int)(t % nch);
+        const int b = b0 + (int)(t / nch), c = (int)(t % nch);
         if (b != cur_b) {
-            if (pend && vs_arrive(a.ticket2 + cur_b, pend, nch) && d.r >= 0) vs_pick<T>(a, cur_b, d);
+            if (pend && vs_arrive(a.ticket2 + cur_b, pend, nch) && d.r >= 0)
+                vs_pick<T, TQ, HID, UA>(a, cur_b, d);
             cur_b = b;
             pend = 0;
             d = decs[b];
@@ -760,22 +890,45 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
         if (d.r >= 0) {
             const bool residual = d.r < K;
             const int nel = min(L::EL, V - c * L::EL);
-            const bool whole = nel == L::EL;
-            const uint8_t *chunk = smem + (size_t)slot * VS_SLOT;
-            // the vectors are read straight from the slot, which is freed afterwards
+            const uint8_t *chunk = smem + (size_t)slot * SLOT;
+            // the logits are read straight from the slot, which is freed afterwards
             const VsNorm nrm = vs_norm(d, a.temperature);
             float sw = 0.f, sp = 0.f;
-#pragma unroll 4
-            for (int k = 0; k < VS_NV; ++k) {
-                if (!whole && (lane + 32 * k) * L::VW >= nel) continue;
-                float f[L::VW], g[L::VW];
-                L::unpack(((const uint4 *)chunk)[lane + 32 * k], f);
-                if (residual) L::unpack(((const uint4 *)(chunk + VS_ROWB))[lane + 32 * k], g);
-#pragma unroll
-                for (int e = 0; e < L::VW; ++e) {
+            if constexpr (UA) {
+                // ids lane, lane + 32, ... of both rows, each at its own misalignment
+                const int mp = (int)(((long long)b * (K + 1) + d.r) * V % L::VW);
+                const int mq = (int)((HID ? (long long)(b - b0) : (long long)b * K + d.r) * V % (16 / (int)sizeof(TQ)));
+                const T *zp = (const T *)chunk + mp;
+                const TQ *zq = (const TQ *)(chunk + REG) + mq;
+#pragma unroll 8
+                for (int e = lane; e < nel; e += 32) {
                     float p;
-                    sw += vs_pw(f[e], residual ? g[e] : 0.f, nrm, residual, p);
+                    sw += vs_pw<HID || UA>(vs_el(zp[e]), residual ? vs_el(zq[e]) : 0.f, nrm, residual, p);
                     sp += p;
+                }
+            } else {
+                const bool whole = nel == L::EL;
+#pragma unroll 4
+                for (int k = 0; k < VS_NV; ++k) {
+                    if (!whole && (lane + 32 * k) * L::VW >= nel) continue;
+                    float f[L::VW], g[L::VW];
+                    L::unpack(((const uint4 *)chunk)[lane + 32 * k], f);
+                    if (residual) {
+                        constexpr int PER = 16 / sizeof(TQ);
+#pragma unroll
+                        for (int i = 0; i < L::VW / PER; ++i) {
+                            float q[PER];
+                            VsT<TQ>::unpack(((const uint4 *)(chunk + REG))[(lane + 32 * k) * (L::VW / PER) + i], q);
+#pragma unroll
+                            for (int e = 0; e < PER; ++e) g[i * PER + e] = q[e];
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < L::VW; ++e) {
+                        float p;
+                        sw += vs_pw<HID || UA>(f[e], residual ? g[e] : 0.f, nrm, residual, p);
+                        sp += p;
+                    }
                 }
             }
             __syncwarp();
@@ -785,38 +938,38 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[slot]);
         }
-        if (lane == 0) ((float2 *)a.tsum)[t] = sums;
+        if (lane == 0) ((float2 *)a.tsum)[(size_t)b * nch + c] = sums;
         ++pend;
     }
-    if (!aborted && pend && vs_arrive(a.ticket2 + cur_b, pend, nch) && d.r >= 0) vs_pick<T>(a, cur_b, d);
+    if (!aborted && pend && vs_arrive(a.ticket2 + cur_b, pend, nch) && d.r >= 0)
+        vs_pick<T, TQ, HID, UA>(a, cur_b, d);
 }
 
 // ---------------------------------------------------------------------------
-bool verify_stream_ok(const VerifyArgs &a) {
+// 0: not streamed; 1: every row starts on 16 bytes; 2: the tensors do, their rows
+// need not.
+int verify_stream_mode(const VerifyArgs &a) {
+    if ((uintptr_t)a.target % 16 || (uintptr_t)a.draft % 16 || a.K + 1 > 32) return 0;
     const int s = a.dtype == OSPREY_F32 ? 4 : 2;
-    const size_t row = (size_t)a.V * s;
-    return row % 16 == 0 && (uintptr_t)a.target % 16 == 0 && (a.draft == nullptr || (uintptr_t)a.draft % 16 == 0) &&
-           a.K + 1 <= 32;
+    return (size_t)a.V * s % 16 == 0 ? 1 : 2;
 }
 
 // Opt each kernel into the ring's shared memory once per device.  The flag
 // lives in a per-kernel template (the kernels share one function type).
 template <auto Kernel>
-static cudaError_t vs_allow_smem() {
+static cudaError_t vs_launch(const VerifyArgs &a, long long tiles, int slot, int sms, cudaStream_t s) {
     static std::atomic<int> done[kMaxDevices];
-    return once_per_device(done, [] {
-        return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, VS_NST * VS_SLOT);
+    cudaError_t e = once_per_device(done, [&] {
+        return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, VS_NST * slot);
     });
-}
-
-template <auto Kernel>
-static cudaError_t vs_launch(const VerifyArgs &a, int blocks, cudaStream_t s) {
-    cudaError_t e = vs_allow_smem<Kernel>();
     if (e != cudaSuccess) return e;
+    // blocks of larger slots (the logits-free draw) fit an SM twice instead of three times
+    const long long per_sm = 3 * (VS_NST * slot + 1024) <= 227 * 1024 ? OSP_VS_BPS : 2;
+    const long long cap = per_sm * sms;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = dim3((unsigned)(tiles < cap ? tiles : cap));
     cfg.blockDim = dim3(VS_THREADS);
-    cfg.dynamicSmemBytes = (size_t)VS_NST * VS_SLOT;
+    cfg.dynamicSmemBytes = (size_t)VS_NST * slot;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -828,26 +981,32 @@ static cudaError_t vs_launch(const VerifyArgs &a, int blocks, cudaStream_t s) {
     return e;
 }
 
-template <typename T>
-static cudaError_t launch_vs(const VerifyArgs &a, int sms, cudaStream_t s) {
-    const long long nt1 = (long long)a.B * (a.K + 1) * a.nch3, nt2 = (long long)a.B * a.nch3;
-    const long long cap = (long long)OSP_VS_BPS * sms;
-    const int g1 = (int)(nt1 < cap ? nt1 : cap), g2 = (int)(nt2 < cap ? nt2 : cap);
-    if (a.temperature == 0.f) return vs_launch<vs_stats<T, true>>(a, g1, s);
-    cudaError_t e = vs_launch<vs_stats<T, false>>(a, g1, s);
+template <typename T, bool UA>
+static cudaError_t launch_vs(const VerifyArgs &a, VsPart part, int sms, cudaStream_t s) {
+    constexpr int EL = VsT<T>::EL, REG = vs_region<T, EL, UA>(), REGF = vs_region<float, EL, UA>();
+    VerifyArgs b = a;
+    b.nch3 = (a.V + EL - 1) / EL;   // for this type (the workspace holds enough for float32)
+    const long long rows = (long long)a.B * (a.K + 1) * b.nch3;
+    switch (part) {
+    case VS_HIDDEN_STATS: return vs_launch<vs_stats<T, false, true, UA>>(b, rows, 2 * REG, sms, s);
+    case VS_HIDDEN_SAMPLE:
+        return vs_launch<vs_sample<T, float, true, UA>>(b, (long long)a.n_group * b.nch3, REG + REGF, sms, s);
+    default: break;
+    }
+    if (a.temperature == 0.f) return vs_launch<vs_stats<T, true, false, UA>>(b, rows, 2 * REG, sms, s);
+    cudaError_t e = vs_launch<vs_stats<T, false, false, UA>>(b, rows, 2 * REG, sms, s);
     if (e != cudaSuccess) return e;
-    return vs_launch<vs_sample<T>>(a, g2, s);
+    return vs_launch<vs_sample<T, T, false, UA>>(b, (long long)a.B * b.nch3, 2 * REG, sms, s);
 }
 
-cudaError_t launch_verify_stream(const VerifyArgs &a, int sms, cudaStream_t s) {
-    // chunks per row for this dtype (the workspace holds enough for float32)
-    VerifyArgs b = a;
-    if (a.dtype == OSPREY_F32) {
-        b.nch3 = (a.V + VsT<float>::EL - 1) / VsT<float>::EL;
-        return launch_vs<float>(b, sms, s);
-    }
-    b.nch3 = (a.V + VsT<uint16_t>::EL - 1) / VsT<uint16_t>::EL;
-    return launch_vs<uint16_t>(b, sms, s);
+cudaError_t launch_verify_stream(const VerifyArgs &a, VsPart part, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const bool ua = verify_stream_mode(a) == 2;
+    if (a.dtype == OSPREY_F32) return ua ? launch_vs<float, true>(a, part, sms, s) : launch_vs<float, false>(a, part, sms, s);
+    return ua ? launch_vs<uint16_t, true>(a, part, sms, s) : launch_vs<uint16_t, false>(a, part, sms, s);
 }
 
 }  // namespace osp
