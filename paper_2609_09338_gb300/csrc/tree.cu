@@ -11,11 +11,20 @@
 // end it with a draw from the last residual.  Greedy: the node's argmax is
 // accepted if it is a candidate (the first such).
 //
-// One block (512 threads) per sequence walks its tree.  A node's row statistics
-// are computed when the walk reaches it (rows off the path are never read); every pass
-// streams one or two rows with 16-byte loads, 256 ids per warp-iteration
-// ("chunk"), several chunks per warp in flight.  A draw keeps its chunk sums
-// in shared memory, picks the chunk by a block scan and the id by a warp scan.
+// One cluster of 8 blocks (512 threads each) per sequence walks its tree: block k
+// takes the k-th range of the vocabulary.  A walk is a chain of dependent passes
+// over one or two rows, so its time is the passes' latency.  One block a sequence
+// pulled 1.2 MB a depth through one SM; 8 blocks pull it through as many, by bulk
+// copies to shared memory, so the passes after the first (a rejection's residual
+// mass, the draw) touch no global memory.  Every pass ends in one exchange of the
+// warps' partials through distributed shared memory, after which all threads hold
+// the same sums and take the same branch; the rows that the chain candidate leads
+// to are on their way to L2 while a depth is decided.  Rows off the path are not
+// waited for.  8 sequences, V 151936, float32, K 5, topk 4: 204 us with one block
+// a sequence, 50 now; a depth is 7 us (rows 1.8, exponentials 3.3, exchange and
+// the reduction after it 1.9).  16 blocks of 256 threads were within 5 %, 4 blocks
+// 1.5 times slower.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -24,10 +33,16 @@
 
 namespace osp {
 
+namespace cg = cooperative_groups;
+
+constexpr int TR_CS = 8;          // blocks per cluster (an exchange has a lane per block)
 constexpr int TR_THREADS = 512;
 constexpr int TR_WARPS = TR_THREADS / 32;
 constexpr int TR_CH = 256;       // ids per chunk: 32 lanes x 8
-constexpr int TR_U = 4;          // chunks a warp loads before using them
+constexpr int TR_U = 1;          // chunks a warp loads before using them
+constexpr int TR_UG = 4;         // ... in an argmax pass
+constexpr int TR_NP = 4;         // pieces a slice arrives in
+constexpr size_t TREE_SMEM_CAP = 216 * 1024;
 constexpr float TR_LOG2E = 1.4426950408889634f;
 
 __device__ __forceinline__ float tr_ex2(float x) {
@@ -71,206 +86,402 @@ __device__ __forceinline__ float tr_at(const T *row, int x) { return tr_f<T>(row
 struct TrNorm {   // p(x) = 2^(z c2 - mp) / Sp (and q alike), c2 = log2(e) / T
     float c2, mp, isp, mq, isq;
 };
+// P, Q: (max, sum exp) of z / T.  A row without a finite logit has no mass.
+__device__ __forceinline__ TrNorm tr_norm(float invT, MS P, MS Q) {
+    const bool np = P.m == -INFINITY, nq = Q.m == -INFINITY;
+    return TrNorm{invT * TR_LOG2E, np ? 0.f : P.m * TR_LOG2E, np ? 0.f : 1.f / P.s, nq ? 0.f : Q.m * TR_LOG2E,
+                  nq ? 0.f : 1.f / Q.s};
+}
 
-// (max, sum exp) of y = z / T over row p (and row q when q != null).
+// One block's view of the cluster and of its slice, chunks [c_lo, c_hi) of the
+// vocabulary.
+template <typename T>
+struct TrCtx {
+    cg::cluster_group cluster;
+    int rank, cs, c_lo, c_hi, V, n_ex, n_fill;
+    bool cached;         // the slice fits shared memory
+    float *csum;         // [slice chunks]
+    T *zp, *zq;          // [slice chunks][256] the current node's rows (when cached)
+    float4 (*slots)[TR_CS * TR_WARPS];   // [2][cs][warps] exchange slots, used in turn
+    uint64_t *full;      // [TR_NP] pieces of the slice landed
+    int32_t *status;
+};
+
+// Every warp's v of every block, in (block, warp) order, through distributed
+// shared memory: one cluster barrier an exchange.  The slots alternate: a slot
+// is written again only after the next exchange's barrier, which every block
+// reaches after it has read this one.  v is lane 0's.
+template <typename T>
+__device__ __forceinline__ const float4 *tr_exchange(TrCtx<T> &t, float4 v) {
+    float4 *slot = t.slots[t.n_ex++ & 1];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    v.x = __shfl_sync(0xffffffffu, v.x, 0);
+    v.y = __shfl_sync(0xffffffffu, v.y, 0);
+    v.z = __shfl_sync(0xffffffffu, v.z, 0);
+    v.w = __shfl_sync(0xffffffffu, v.w, 0);
+    if (lane < t.cs) *t.cluster.map_shared_rank(&slot[t.rank * TR_WARPS + warp], lane) = v;
+    t.cluster.sync();
+    return slot;
+}
+
+// Sum of the exchanged values' x, the same in every thread of the cluster.
+template <typename T>
+__device__ __forceinline__ float tr_sum(const TrCtx<T> &t, const float4 *all) {
+    float w = 0.f;
+    for (int i = threadIdx.x & 31; i < t.cs * TR_WARPS; i += 32) w += all[i].x;
+    return warp_sum(w);
+}
+
+// Piece p of the slice's chunks.
+template <typename T>
+__device__ __forceinline__ void tr_piece(const TrCtx<T> &t, int p, int &lo, int &hi) {
+    const int n = t.c_hi - t.c_lo;
+    lo = t.c_lo + n * p / TR_NP;
+    hi = t.c_lo + n * (p + 1) / TR_NP;
+}
+__device__ __forceinline__ void tr_prefetch_l2(const void *p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// The slices of row zp (and zq when given) on their way to shared memory: bulk
+// copies in TR_NP pieces where rows are 16-byte aligned, else plain loads (32
+// consecutive ids each) and a block barrier.  The block has read the slices'
+// last contents (a barrier before the call).
 template <typename T, bool VEC>
-__device__ void tr_stats(const T *zp, const T *zq, int V, float invT, MS *shm, MS &P, MS &Q) {
-    const int warp = threadIdx.x >> 5, nch = (V + TR_CH - 1) / TR_CH;
-    float mp = -INFINITY, sp = 0.f, mq = -INFINITY, sq = 0.f;
-    for (int c0 = warp; c0 < nch; c0 += TR_WARPS * TR_U) {
-        float f[TR_U][8], g[TR_U][8];
-#pragma unroll
-        for (int u = 0; u < TR_U; ++u) {
-            const int c = c0 + u * TR_WARPS;
-            tr_load8<T, VEC>(zp, c < nch ? c : nch, V, f[u]);
-            if (zq) tr_load8<T, VEC>(zq, c < nch ? c : nch, V, g[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < TR_U; ++u) {
-            float lm = -INFINITY;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) lm = fmaxf(lm, f[u][e] * invT);
-            if (lm > mp) {
-                sp = mp == -INFINITY ? 0.f : sp * tr_ex2((mp - lm) * TR_LOG2E);
-                mp = lm;
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) sp += f[u][e] == -INFINITY ? 0.f : tr_ex2((f[u][e] * invT - mp) * TR_LOG2E);
-            if (zq) {
-                float lq = -INFINITY;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) lq = fmaxf(lq, g[u][e] * invT);
-                if (lq > mq) {
-                    sq = mq == -INFINITY ? 0.f : sq * tr_ex2((mq - lq) * TR_LOG2E);
-                    mq = lq;
+__device__ void tr_fill(TrCtx<T> &t, const T *zp, const T *zq) {
+    if (VEC) {
+        if (threadIdx.x == 0) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+#pragma unroll 1
+            for (int p = 0; p < TR_NP; ++p) {
+                int lo, hi;
+                tr_piece(t, p, lo, hi);
+                const int e0 = lo * TR_CH, e1 = min(t.V, hi * TR_CH);
+                const uint32_t bytes = e1 > e0 ? (uint32_t)(e1 - e0) * sizeof(T) : 0;   // a multiple of 16 (V % 8 == 0)
+                const size_t at = (size_t)(lo - t.c_lo) * TR_CH;
+                mbar_arrive_expect_tx(&t.full[p], zq ? 2 * bytes : bytes);
+                if (bytes) {
+                    bulk_g2s(t.zp + at, zp + e0, bytes, &t.full[p]);
+                    if (zq) bulk_g2s(t.zq + at, zq + e0, bytes, &t.full[p]);
                 }
-#pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    sq += g[u][e] == -INFINITY ? 0.f : tr_ex2((g[u][e] * invT - mq) * TR_LOG2E);
             }
         }
+    } else {
+        const int e1 = min(t.V, t.c_hi * TR_CH);
+#pragma unroll 4
+        for (int e = t.c_lo * TR_CH + (int)threadIdx.x; e < e1; e += TR_THREADS) {
+            t.zp[e - t.c_lo * TR_CH] = zp[e];
+            if (zq) t.zq[e - t.c_lo * TR_CH] = zq[e];
+        }
+        __syncthreads();
     }
-    P = block_ms(MS{mp, sp}, shm);
-    Q = zq ? block_ms(MS{mq, sq}, shm) : MS{-INFINITY, 0.f};
+}
+
+// The lane's 8 logits of chunk c of the current node's row, -inf past V.
+template <typename T, bool VEC>
+__device__ __forceinline__ void tr_get8(const TrCtx<T> &t, const T *slice, const T *row, int c, float (&f)[8]) {
+    if (t.cached) {
+        const int lane = threadIdx.x & 31;
+        const T *d = slice + (size_t)(c - t.c_lo) * TR_CH + lane * 8;
+        if constexpr (sizeof(T) == 4) {
+            const float4 a = *(const float4 *)d, b = *(const float4 *)(d + 4);
+            f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
+            f[4] = b.x; f[5] = b.y; f[6] = b.z; f[7] = b.w;
+        } else {
+            unpack8(*(const uint4 *)d, f);
+        }
+        if ((c + 1) * TR_CH > t.V) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (c * TR_CH + lane * 8 + e >= t.V) f[e] = -INFINITY;
+        }
+    } else {
+        tr_load8<T, VEC>(row, c, t.V, f);
+    }
+}
+
+// (max, sum exp) of y = z / T over row zp (and row zq when given), whose slices
+// tr_fill has requested (when cached).
+template <typename T, bool VEC>
+__device__ void tr_stats(TrCtx<T> &t, const T *zp, const T *zq, float invT, MS &P, MS &Q) {
+    const int warp = threadIdx.x >> 5;
+    // maxima of the raw logits (order is kept by the positive 1/T), sums of
+    // 2^((z - max) c2); four sums a row, the loads and exponentials of TR_U chunks
+    // independent of one another (16 warps an SM hide little latency)
+    const float c2 = invT * TR_LOG2E;
+    float mp = -INFINITY, sp = 0.f, mq = -INFINITY, sq = 0.f;
+    auto fold = [&](const float (&f)[TR_U][8], float &m, float &s) {
+        float x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            x[j] = fmaxf(f[0][j], f[0][j + 4]);
+#pragma unroll
+            for (int u = 1; u < TR_U; ++u) x[j] = fmaxf(x[j], fmaxf(f[u][j], f[u][j + 4]));
+        }
+        const float lm = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+        if (lm > m) {
+            s = m == -INFINITY ? 0.f : s * tr_ex2((m - lm) * c2);
+            m = lm;
+        }
+        if (m == -INFINITY) return;
+        float e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) e[j & 3] += tr_ex2((f[u][j] - m) * c2);
+        s += (e[0] + e[1]) + (e[2] + e[3]);
+    };
+    {
+        // a warp waits for a piece when it comes to the first of its chunks there;
+        // on expiry the walk goes on (every block takes part in the cluster's
+        // barriers) and its result is void, which the status word says
+        const bool pieces = t.cached && VEC;
+        int p = -1, plo, phi = t.c_lo;
+        for (int c0 = t.c_lo + warp; c0 < t.c_hi; c0 += TR_WARPS * TR_U) {
+            const int last = min(t.c_hi - 1, c0 + (TR_U - 1) * TR_WARPS);
+            while (pieces && last >= phi) {
+                tr_piece(t, ++p, plo, phi);
+                if (!mbar_wait(&t.full[p], t.n_fill & 1)) set_status(t.status, OSPREY_ERR_TIMEOUT);
+            }
+            float f[TR_U][8], g[TR_U][8];
+#pragma unroll
+            for (int u = 0; u < TR_U; ++u) {
+                const int c = c0 + u * TR_WARPS;
+                if (c < t.c_hi) {
+                    tr_get8<T, VEC>(t, t.zp, zp, c, f[u]);
+                    if (zq) tr_get8<T, VEC>(t, t.zq, zq, c, g[u]);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) f[u][e] = g[u][e] = -INFINITY;
+                }
+            }
+            fold(f, mp, sp);
+            if (zq) fold(g, mq, sq);
+        }
+        // the pieces that a warp without chunks there has not waited for
+        while (pieces && ++p < TR_NP)
+            if (!mbar_wait(&t.full[p], t.n_fill & 1)) set_status(t.status, OSPREY_ERR_TIMEOUT);
+    }
+    ++t.n_fill;
+    auto reduce = [&](float m, float s) {   // the warp maximum first, then each sum rescaled once
+        const float M = warp_max(m);
+        return MS{M * invT, warp_sum(m == -INFINITY ? 0.f : s * tr_ex2((m - M) * c2))};
+    };
+    P = reduce(mp, sp);
+    Q = zq ? reduce(mq, sq) : MS{-INFINITY, 0.f};
+    const float4 *all = tr_exchange(t, make_float4(P.m, P.s, Q.m, Q.s));
+    float m1 = -INFINITY, m2 = -INFINITY;
+    const int lane = threadIdx.x & 31, n = t.cs * TR_WARPS;
+    for (int i = lane; i < n; i += 32) {
+        m1 = fmaxf(m1, all[i].x);
+        m2 = fmaxf(m2, all[i].z);
+    }
+    m1 = warp_max(m1);
+    m2 = warp_max(m2);
+    float s1 = 0.f, s2 = 0.f;
+    for (int i = lane; i < n; i += 32) {
+        const float4 v = all[i];
+        s1 += v.x == -INFINITY ? 0.f : v.y * tr_ex2((v.x - m1) * TR_LOG2E);
+        s2 += v.z == -INFINITY ? 0.f : v.w * tr_ex2((v.z - m2) * TR_LOG2E);
+    }
+    P = MS{m1, warp_sum(s1)};
+    Q = MS{m2, warp_sum(s2)};
 }
 
 // argmax (lowest id on ties) of a row
 template <typename T, bool VEC>
-__device__ int tr_argmax(const T *z, int V, AM *sha) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nch = (V + TR_CH - 1) / TR_CH;
+__device__ int tr_argmax(TrCtx<T> &t, const T *z) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, V = t.V;
     AM am{-INFINITY, 0x7fffffff};
-    for (int c0 = warp; c0 < nch; c0 += TR_WARPS * TR_U) {
-        float f[TR_U][8];
+    for (int c0 = t.c_lo + warp; c0 < t.c_hi; c0 += TR_WARPS * TR_UG) {
+        float f[TR_UG][8];
 #pragma unroll
-        for (int u = 0; u < TR_U; ++u) tr_load8<T, VEC>(z, min(c0 + u * TR_WARPS, nch), V, f[u]);
+        for (int u = 0; u < TR_UG; ++u) {
+            const int c = c0 + u * TR_WARPS;
+            if (c >= t.c_hi) continue;
+            if (VEC) {
+                tr_load8<T, VEC>(z, c, V, f[u]);
+            } else {   // unaligned rows: 32 consecutive ids a load instead of a vector per lane
 #pragma unroll
-        for (int u = 0; u < TR_U; ++u) {
-            const int base = (c0 + u * TR_WARPS) * TR_CH + lane * 8;
+                for (int e = 0; e < 8; ++e) {
+                    const int id = c * TR_CH + e * 32 + lane;
+                    f[u][e] = id < V ? tr_f<T>(z[id]) : -INFINITY;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < TR_UG; ++u) {
+            const int c = c0 + u * TR_WARPS;
+            if (c >= t.c_hi) continue;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                if (f[u][e] > am.v) am = AM{f[u][e], base + e};
+                if (f[u][e] > am.v) am = AM{f[u][e], c * TR_CH + (VEC ? lane * 8 + e : e * 32 + lane)};
         }
     }
-    return block_am(am, sha).i;
+    am = warp_am(am);
+    const float4 *all = tr_exchange(t, make_float4(am.v, __int_as_float(am.i), 0.f, 0.f));
+    AM r{-INFINITY, 0x7fffffff};
+    for (int i = lane; i < t.cs * TR_WARPS; i += 32) r = am_combine(r, AM{all[i].x, __float_as_int(all[i].y)});
+    return warp_am(r).i;
 }
 
-// Weight of one id in a draw: the residual max(0, p - c q) (c > 0) or p.
-__device__ __forceinline__ float tr_weight(float zp, float zq, const TrNorm &n, float c) {
-    const float p = zp == -INFINITY ? 0.f : tr_ex2(zp * n.c2 - n.mp) * n.isp;
-    if (c == 0.f) return p;
-    const float q = zq == -INFINITY ? 0.f : tr_ex2(zq * n.c2 - n.mq) * n.isq;
-    return fmaxf(0.f, p - c * q);
+// Weight of one id in a draw: the residual max(0, p - c q) (c > 0; ciq = c / Sq)
+// or p.  A logit of -inf weighs 0 (2^-inf).
+__device__ __forceinline__ float tr_weight(float zp, float zq, const TrNorm &n, float c, float ciq) {
+    const float p = tr_ex2(fmaf(zp, n.c2, -n.mp)) * n.isp;
+    return c == 0.f ? p : fmaxf(0.f, fmaf(-ciq, tr_ex2(fmaf(zq, n.c2, -n.mq)), p));
 }
 
-// sum over the ids of tr_weight; with csum, each chunk's sum is kept there
+// The warp's sum over its chunks of tr_weight; `sums`: each chunk's sum is kept.
 template <typename T, bool VEC>
-__device__ float tr_mass(const T *zp, const T *zq, int V, const TrNorm &n, float c, float *csum, float *shf) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nch = (V + TR_CH - 1) / TR_CH;
+__device__ float tr_warp_mass(TrCtx<T> &t, const T *zp, const T *zq, const TrNorm &n, float c, bool sums) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const float ciq = c * n.isq;
     float acc = 0.f;
-    for (int c0 = warp; c0 < nch; c0 += TR_WARPS * TR_U) {
+    for (int c0 = t.c_lo + warp; c0 < t.c_hi; c0 += TR_WARPS * TR_U) {
         float f[TR_U][8], g[TR_U][8];
 #pragma unroll
         for (int u = 0; u < TR_U; ++u) {
-            const int ch = min(c0 + u * TR_WARPS, nch);
-            tr_load8<T, VEC>(zp, ch, V, f[u]);
-            if (c != 0.f) tr_load8<T, VEC>(zq, ch, V, g[u]);
+            const int ch = c0 + u * TR_WARPS;
+            if (ch < t.c_hi) {
+                tr_get8<T, VEC>(t, t.zp, zp, ch, f[u]);
+                if (c != 0.f) tr_get8<T, VEC>(t, t.zq, zq, ch, g[u]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) f[u][e] = g[u][e] = -INFINITY;
+            }
         }
 #pragma unroll
         for (int u = 0; u < TR_U; ++u) {
-            float s = 0.f;
+            const int ch = c0 + u * TR_WARPS;
+            float e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int e = 0; e < 8; ++e) s += tr_weight(f[u][e], c != 0.f ? g[u][e] : -INFINITY, n, c);
-            if (csum) {
+            for (int j = 0; j < 8; ++j) e[j & 3] += tr_weight(f[u][j], g[u][j], n, c, ciq);
+            float s = (e[0] + e[1]) + (e[2] + e[3]);
+            if (sums) {
                 s = warp_sum(s);
-                if (lane == 0 && c0 + u * TR_WARPS < nch) csum[c0 + u * TR_WARPS] = s;
+                if (lane == 0 && ch < t.c_hi) t.csum[ch - t.c_lo] = s;
+                acc += lane == 0 ? s : 0.f;   // every lane holds the chunk's sum: count it once
+            } else {
+                acc += s;
             }
-            acc += s;
         }
     }
-    // with csum every lane holds its warp's chunk sums: count them once
-    if (csum) acc = lane == 0 ? acc : 0.f;
-    float tot = 0.f;
-    {
-        const float w = warp_sum(acc);
-        if (lane == 0) shf[warp] = w;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            float v = threadIdx.x < TR_WARPS ? shf[threadIdx.x] : 0.f;
-            v = warp_sum(v);
-            if (threadIdx.x == 0) shf[32] = v;
-        }
-        __syncthreads();
-        tot = shf[32];
-        __syncthreads();
-    }
-    return tot;
+    return warp_sum(acc);
 }
 
-// Inverse CDF over ascending ids of tr_weight at u (a mass pass with chunk
-// sums first).  flag |= 16 when rounding leaves u*S past the last sum (the
-// last id with weight is taken).
 template <typename T, bool VEC>
-__device__ int tr_draw(const T *zp, const T *zq, int V, const TrNorm &n, float c, float u, float *csum, float *shf,
-                       int *shi, int &flag) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nch = (V + TR_CH - 1) / TR_CH;
-    const float S = tr_mass<T, VEC>(zp, zq, V, n, c, csum, shf);
+__device__ float tr_mass(TrCtx<T> &t, const T *zp, const T *zq, const TrNorm &n, float c) {
+    const float w = tr_warp_mass<T, VEC>(t, zp, zq, n, c, false);
+    return tr_sum(t, tr_exchange(t, make_float4(w, 0.f, 0.f, 0.f)));
+}
+
+// Inverse CDF over ascending ids of tr_weight at u: a mass pass with chunk sums,
+// then the block whose range holds the point finds the chunk by a scan over its
+// chunk sums and the id by a warp scan, and writes the token and its flags
+// (flag | 16 when rounding leaves u*S past the last sum: the last id with weight
+// is taken).  The walk ends with it.
+template <typename T, bool VEC>
+__device__ void tr_draw(TrCtx<T> &t, const T *zp, const T *zq, const TrNorm &n, float c, float u, float *shf, int *shi,
+                        int flag, int32_t *out, uint8_t *fl) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nch = t.c_hi - t.c_lo;
+    const float w0 = tr_warp_mass<T, VEC>(t, zp, zq, n, c, true);
+    const float4 *all = tr_exchange(t, make_float4(w0, 0.f, 0.f, 0.f));
+    // block totals in vocabulary order (lane k: block k), their prefix, the owner
+    float bt = 0.f;
+    if (lane < t.cs)
+        for (int w = 0; w < TR_WARPS; ++w) bt += all[lane * TR_WARPS + w].x;
+    const float incl = warp_incl_scan(bt);
+    const float S = __shfl_sync(0xffffffffu, incl, t.cs - 1);
     const float target = u * S;
+    const unsigned hits = __ballot_sync(0xffffffffu, bt > 0.f && target < incl);
+    const unsigned some = __ballot_sync(0xffffffffu, bt > 0.f);
+    const int owner = hits ? __ffs(hits) - 1 : (some ? 31 - __clz(some) : 0);
+    const float before = __shfl_sync(0xffffffffu, incl - bt, owner);
+    bool past = !hits;
+    if (owner != t.rank) return;
     // chunks per thread, in order
     const int per = (nch + TR_THREADS - 1) / TR_THREADS;
-    const int k0 = min(nch, threadIdx.x * per), k1 = min(nch, k0 + per);
-    float mine = 0.f;
-    for (int k = k0; k < k1; ++k) mine += csum[k];
+    const int k0 = min(nch, (int)threadIdx.x * per), k1 = min(nch, k0 + per);
+    float mine_w = 0.f;
+    for (int k = k0; k < k1; ++k) mine_w += t.csum[k];   // the exchange's barrier made them visible
     float tot;
-    const float ex = block_excl_scan(mine, shf, &tot);
+    const float ex = before + block_excl_scan(mine_w, shf, &tot);
     if (threadIdx.x == 0) { shi[0] = 0x7fffffff; shi[1] = -1; }
     __syncthreads();
-    if (mine > 0.f && target < ex + mine) atomicMin(&shi[0], (int)threadIdx.x);
-    if (mine > 0.f) atomicMax(&shi[1], (int)threadIdx.x);
+    if (mine_w > 0.f && target < ex + mine_w) atomicMin(&shi[0], (int)threadIdx.x);
+    if (mine_w > 0.f) atomicMax(&shi[1], (int)threadIdx.x);
     __syncthreads();
     const int ct = shi[0] != 0x7fffffff ? shi[0] : (shi[1] >= 0 ? shi[1] : 0);
-    const bool past = shi[0] == 0x7fffffff;
+    past |= shi[0] == 0x7fffffff;
     __syncthreads();
     if ((int)threadIdx.x == ct) {
         float cum = ex;
         int ch = -1, lastc = k0;
-        float lastb = ex;
+        float lb = ex;
         for (int k = k0; k < k1; ++k) {
-            if (csum[k] > 0.f) { lastc = k; lastb = cum; }
-            if (csum[k] > 0.f && target < cum + csum[k]) { ch = k; break; }
-            cum += csum[k];
+            if (t.csum[k] > 0.f) { lastc = k; lb = cum; }
+            if (t.csum[k] > 0.f && target < cum + t.csum[k]) { ch = k; break; }
+            cum += t.csum[k];
         }
-        shi[2] = ch >= 0 ? ch : lastc;
-        shf[33] = ch >= 0 ? cum : lastb;
+        shi[2] = min(ch >= 0 ? ch : lastc, nch - 1);
+        shf[33] = ch >= 0 ? cum : lb;
         shi[3] = ch < 0 || past;
     }
     __syncthreads();
     if (warp == 0) {
-        const int ch = shi[2];
+        const int ch = t.c_lo + shi[2];
         float f[8], g[8];
-        tr_load8<T, VEC>(zp, ch, V, f);
-        if (c != 0.f) tr_load8<T, VEC>(zq, ch, V, g);
+        tr_get8<T, VEC>(t, t.zp, zp, ch, f);
+        if (c != 0.f) tr_get8<T, VEC>(t, t.zq, zq, ch, g);
         float w[8], s = 0.f;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            w[e] = tr_weight(f[e], c != 0.f ? g[e] : -INFINITY, n, c);
+            w[e] = tr_weight(f[e], g[e], n, c, c * n.isq);
             s += w[e];
         }
-        const float incl = warp_incl_scan(s);
-        const float before = shf[33] + incl - s;
+        const float run = warp_incl_scan(s);
+        float cum = shf[33] + run - s;
         int found = -1, lastp = -1;
-        float run = before;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            run += w[e];
+            cum += w[e];
             if (w[e] > 0.f) lastp = e;
-            if (found < 0 && w[e] > 0.f && target < run) found = e;
+            if (found < 0 && w[e] > 0.f && target < cum) found = e;
         }
         const unsigned hit = __ballot_sync(0xffffffffu, found >= 0);
         const unsigned pos = __ballot_sync(0xffffffffu, lastp >= 0);
         const int l = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
         if (lane == l) {
             const int e = found >= 0 ? found : (lastp >= 0 ? lastp : 0);
-            shi[4] = ch * TR_CH + l * 8 + e;
-            if (!hit || shi[3]) shi[5] = 16;
-            else shi[5] = 0;
+            *out = ch * TR_CH + l * 8 + e;
+            *fl = (uint8_t)(flag | (!hit || shi[3] ? 16 : 0));
         }
     }
-    __syncthreads();
-    flag |= shi[5];
-    const int tok = shi[4];
-    __syncthreads();
-    return tok;
 }
 
 template <typename T, bool VEC, bool GREEDY>
-__global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTreeArgs a) {
-    extern __shared__ float csum[];   // [chunks of a row]
-    __shared__ MS shm[32];
-    __shared__ AM sha[32];
+__global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTreeArgs a, int slice_chunks, int cached) {
+    extern __shared__ __align__(128) uint8_t dyn[];   // cached: [2][slice][256] logits; then [slice] chunk sums
     __shared__ float shf[34];
     __shared__ int shi[8];
-    __shared__ int s_acc;
-    const int b = blockIdx.x, K = a.K, k = a.k, V = a.V;
+    __shared__ float4 slots[2][TR_CS * TR_WARPS];
+    __shared__ __align__(8) uint64_t full[TR_NP];
+    __shared__ float s_zp[8], s_zq[8], s_u[8];
+    const int K = a.K, k = a.k, V = a.V;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), b = blockIdx.x / cs;
+    const int nch = (V + TR_CH - 1) / TR_CH;
+    // block 0's slice is never empty; the last ones' may be
+    const int c_lo = min(nch, rank * slice_chunks);
+    const size_t rows = cached ? (size_t)slice_chunks * TR_CH : 0;
+    T *slice = (T *)dyn;
+    TrCtx<T> t{cluster, rank, cs, c_lo, min(nch, c_lo + slice_chunks), V, 0, 0, cached != 0,
+               (float *)(slice + 2 * rows), slice, slice + rows, slots, full, a.status};
+    if (threadIdx.x == 0) {
+        for (int p = 0; p < TR_NP; ++p) mbar_init(&full[p], 1);
+        mbar_fence_init();
+    }
     const size_t nrow = (size_t)(1 + K * k);
     const T *tp = (const T *)a.target + (size_t)b * nrow * V;
     const T *dq = GREEDY ? nullptr : (const T *)a.draft + (size_t)b * K * V;
@@ -278,17 +489,26 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
     int32_t *out = a.out_tokens + (size_t)b * (K + 1);
     uint8_t *fl = a.flags + (size_t)b * (K + 1);
     pdl_trigger();
+    __syncthreads();   // the barriers are ready
     pdl_wait();
+    if (!GREEDY && t.cached) tr_fill<T, VEC>(t, tp, dq);   // the root's rows, whatever the checks say
     // candidate ids outside [0, V): the sequence is reported and skipped
     bool ok = true;
     for (int i = threadIdx.x; i < K * k; i += TR_THREADS) ok &= cand[i] >= 0 && cand[i] < V;
     ok = __syncthreads_and(ok);
-    if (threadIdx.x <= K) {
+    const bool lead = rank == 0 && threadIdx.x == 0;
+    if (rank == 0 && threadIdx.x <= K) {
         out[threadIdx.x] = -1;
         fl[threadIdx.x] = 0;
     }
-    if (!ok) {
-        if (threadIdx.x == 0) {
+    // every block has started (its shared memory may be written), and the defaults
+    // above come before what other blocks of the cluster write over them
+    __threadfence();
+    cluster.sync();
+    if (!ok) {   // the same in every block
+        if (!GREEDY && VEC && t.cached)   // the copies under way land before the block can exit
+            for (int p = 0; p < TR_NP; ++p) mbar_wait(&full[p], 0);
+        if (lead) {
             set_status(a.status, OSPREY_ERR_INVALID_ARG);
             a.n_accepted[b] = 0;
             a.branch[b] = -1;
@@ -297,64 +517,71 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
     }
     const float invT = GREEDY ? 1.f : 1.f / a.temperature;
     int row = 0, nacc = 0, br = -1;
+    // the rows that the walk reads next if the chain candidate of depth i is
+    // accepted, on their way to L2 while this depth is decided
+    auto tr_next_rows = [&](int i) {
+        if (!VEC || GREEDY || threadIdx.x != 0) return;
+        const int e0 = t.c_lo * TR_CH, e1 = min(V, t.c_hi * TR_CH);
+        if (e1 <= e0) return;
+        const uint32_t bytes = (uint32_t)(e1 - e0) * sizeof(T);
+        tr_prefetch_l2(tp + (size_t)(1 + i * k) * V + e0, bytes);
+        if (i + 1 < K) tr_prefetch_l2(dq + (size_t)(i + 1) * V + e0, bytes);
+    };
     for (int i = 0; i < K; ++i) {
         const T *zp = tp + (size_t)row * V;
         if (GREEDY) {
-            const int y = tr_argmax<T, VEC>(zp, V, sha);
+            const int y = tr_argmax<T, VEC>(t, zp);
             int j = -1;
             for (int jj = 0; jj < k && j < 0; ++jj)
                 if (cand[i * k + jj] == y) j = jj;
-            if (threadIdx.x == 0) out[i] = y;
+            if (lead) out[i] = y;
             if (j < 0) break;
             ++nacc;
             br = j;
             row = 1 + i * k + j;
             if (j > 0 || i == K - 1) {
-                const int z = tr_argmax<T, VEC>(tp + (size_t)row * V, V, sha);
-                if (threadIdx.x == 0) out[i + 1] = z;
+                const int z = tr_argmax<T, VEC>(t, tp + (size_t)row * V);
+                if (lead) out[i + 1] = z;
                 break;
             }
             continue;
         }
         const T *zq = dq + (size_t)i * V;
+        if ((int)threadIdx.x < k) {   // the candidates' logits and uniforms, in flight with the rows
+            const int x = cand[i * k + threadIdx.x];
+            s_zp[threadIdx.x] = tr_at<T>(zp, x);
+            s_zq[threadIdx.x] = tr_at<T>(zq, x);
+            s_u[threadIdx.x] = a.u_accept[((size_t)b * K + i) * k + threadIdx.x];
+        }
         MS P, Q;
-        tr_stats<T, VEC>(zp, zq, V, invT, shm, P, Q);
-        TrNorm n{invT * TR_LOG2E, P.m * TR_LOG2E, 1.f / P.s, Q.m * TR_LOG2E, 1.f / Q.s};
+        tr_stats<T, VEC>(t, zp, zq, invT, P, Q);
+        tr_next_rows(i);
+        const TrNorm n = tr_norm(invT, P, Q);
         float c = 0.f, W = 1.f;
-        int flag = 0;
-        if (threadIdx.x == 0) s_acc = -1;
-        __syncthreads();
-        for (int j = 0; j < k; ++j) {
-            const int x = cand[i * k + j];
-            const float px = tr_ex2(tr_at<T>(zp, x) * n.c2 - n.mp) * n.isp;
-            const float qx = tr_ex2(tr_at<T>(zq, x) * n.c2 - n.mq) * n.isq;
+        int flag = 0, acc = -1;
+        for (int j = 0; j < k; ++j) {   // every thread of the cluster computes the same
+            const float px = tr_ex2(fmaf(s_zp[j], n.c2, -n.mp)) * n.isp;
+            const float qx = tr_ex2(fmaf(s_zq[j], n.c2, -n.mq)) * n.isq;
             const float r = fmaxf(0.f, px - c * qx) / W;
-            const float u = a.u_accept[((size_t)b * K + i) * k + j];
-            if (u < r / qx) {
-                if (threadIdx.x == 0) s_acc = j;
+            if (s_u[j] < r / qx) {
+                acc = j;
                 break;
             }
             // rejected: the next residual
             c += W;
-            W = tr_mass<T, VEC>(zp, zq, V, n, c, nullptr, shf);
+            W = tr_mass<T, VEC>(t, zp, zq, n, c);
             if (!(W > 0.f)) {   // no mass left in float32: sample p instead
                 c = 0.f;
                 W = 1.f;
                 flag |= 8;
             }
         }
-        __syncthreads();
-        const int acc = s_acc;
         if (acc < 0) {   // every candidate rejected: a draw from the residual
-            const int t = tr_draw<T, VEC>(zp, zq, V, n, c, a.u_sample[(size_t)b * (K + 1) + i], csum, shf, shi,
-                                          flag);
-            if (threadIdx.x == 0) {
-                out[i] = t;
-                fl[i] = (uint8_t)flag;
-            }
+            tr_draw<T, VEC>(t, zp, zq, n, c, a.u_sample[(size_t)b * (K + 1) + i], shf, shi, flag,
+                            out + i, fl + i);
             break;
         }
-        if (threadIdx.x == 0) {
+        if (lead) {
             out[i] = cand[i * k + acc];
             fl[i] = (uint8_t)flag;
         }
@@ -363,42 +590,60 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
         row = 1 + i * k + acc;
         if (acc > 0 || i == K - 1) {   // a leaf or the last depth: the next token from the node's row
             const T *zn = tp + (size_t)row * V;
+            __syncthreads();   // the slices are read no more
+            if (t.cached) tr_fill<T, VEC>(t, zn, (const T *)nullptr);
             MS Pn, Qn;
-            tr_stats<T, VEC>(zn, (const T *)nullptr, V, invT, shm, Pn, Qn);
-            TrNorm nn{invT * TR_LOG2E, Pn.m * TR_LOG2E, 1.f / Pn.s, 0.f, 0.f};
-            int f2 = 0;
-            const int t = tr_draw<T, VEC>(zn, (const T *)nullptr, V, nn, 0.f,
-                                          a.u_sample[(size_t)b * (K + 1) + i + 1], csum, shf, shi, f2);
-            if (threadIdx.x == 0) {
-                out[i + 1] = t;
-                fl[i + 1] = (uint8_t)f2;
-            }
+            tr_stats<T, VEC>(t, zn, (const T *)nullptr, invT, Pn, Qn);
+            const TrNorm nn = tr_norm(invT, Pn, MS{-INFINITY, 0.f});
+            tr_draw<T, VEC>(t, zn, (const T *)nullptr, nn, 0.f, a.u_sample[(size_t)b * (K + 1) + i + 1], shf, shi, 0,
+                            out + i + 1, fl + i + 1);
             break;
         }
+        __syncthreads();   // the slices and candidates are read no more
+        if (t.cached) tr_fill<T, VEC>(t, tp + (size_t)row * V, dq + (size_t)(i + 1) * V);
     }
-    if (threadIdx.x == 0) {
+    if (lead) {
         a.n_accepted[b] = nacc;
         a.branch[b] = br;
     }
 }
 
-template <typename T, bool VEC>
+template <typename T, bool VEC, bool GREEDY>
 static cudaError_t tree_launch(const VerifyTreeArgs &a, cudaStream_t s) {
-    const size_t smem = (size_t)((a.V + TR_CH - 1) / TR_CH) * sizeof(float);
+    auto *kernel = tree_verify_kernel<T, VEC, GREEDY>;
+    static std::atomic<int> done[kMaxDevices];
+    cudaError_t e = once_per_device(done, [&] { return allow_smem(kernel); });
+    if (e != cudaSuccess) return e;
+    const int nch = (a.V + TR_CH - 1) / TR_CH;
+    const int cs = TR_CS;
+    const int slice = (nch + cs - 1) / cs;
+    // two rows of a slice in shared memory; a vocabulary too large for that
+    // (V > 8 x 26k at 8 blocks) is read again by the later passes, from L2
+    size_t smem = (size_t)slice * (2 * TR_CH * sizeof(T) + sizeof(float));
+    const int cached = !GREEDY && smem <= TREE_SMEM_CAP;
+    if (!cached) smem = (size_t)slice * sizeof(float);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.B);
+    cfg.gridDim = dim3((unsigned)a.B * cs);
     cfg.blockDim = dim3(TR_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = a.temperature == 0.f ? cudaLaunchKernelEx(&cfg, tree_verify_kernel<T, VEC, true>, a)
-                                         : cudaLaunchKernelEx(&cfg, tree_verify_kernel<T, VEC, false>, a);
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, kernel, a, slice, cached);
     count_launch();
     return e;
+}
+
+template <typename T, bool VEC>
+static cudaError_t tree_launch(const VerifyTreeArgs &a, cudaStream_t s) {
+    return a.temperature == 0.f ? tree_launch<T, VEC, true>(a, s) : tree_launch<T, VEC, false>(a, s);
 }
 
 cudaError_t launch_verify_tree(const VerifyTreeArgs &a, cudaStream_t s) {
