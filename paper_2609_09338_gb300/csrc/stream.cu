@@ -785,7 +785,11 @@ StreamPlan stream_plan(GemvMode mode, const Dims &D, int sms) {
         p.stage_bytes = rows * row_bytes;
     }
     p.n_stages = (p.n_items + p.items - 1) / p.items;
-    const int bps = mode == G_LM ? OSP_SG_BLOCKS_PER_SM : OSP_SG_GEMV_BPS;
+    // a layer GEMV with rows so long that its ring leaves room for one block per SM
+    // gets one: twice as many ran as two waves, the second with nothing requested
+    // ahead (d 2560: down 20.4 us, QKV 18.2 us a launch)
+    const bool twice = 2 * (SG_NST * (size_t)p.stage_bytes + 4ull * Kd + 4096) <= 227 * 1024;
+    const int bps = mode == G_LM ? OSP_SG_BLOCKS_PER_SM : twice ? OSP_SG_GEMV_BPS : 1;
     p.blocks = p.n_stages < sms * bps ? p.n_stages : sms * bps;
     // LM head runs: the fewest stages per run that leave at most 32 runs a block
     const int maxloc = (p.n_stages + p.blocks - 1) / p.blocks;
