@@ -587,6 +587,17 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         // (one block per SM); beyond that the global-partials kernel keeps more
         // loads in flight
         const bool clu = ctx->attn_cs && (long long)R * D.Hkv * ctx->attn_cs <= ctx->sms;
+        // several rows a sequence share their keys: one pass over them for 16 queries
+        // (row, head) instead of one a row (96 x 8 rows: 356 us a launch against 592;
+        // 8 x 15 rows, 4 heads a group: 150 against 260).  Below one wave of the decode
+        // kernel's blocks, which then have every page in flight at once, it is the
+        // slower one (1 x 8 rows at 2048 keys: 51 us against 24).
+        const int mt = !clu && rows_per_seq > 1 && (long long)R * D.Hkv >= 2 * ctx->sms ? attn_rows_tiles(D, rows_per_seq) : 0;
+        auto attention = [&](AttnArgs &at) {
+            at.n_splits = clu ? ctx->attn_cs : mt ? attn_splits(B * mt, D.Hkv, max_ctx, ctx->sms) : ns;
+            at.split_len = attn_split_len(max_ctx, at.n_splits);
+            return clu ? launch_attn_cluster(at, ctx->attn_cs, s) : mt ? launch_attn_rows(at, B, mt, s) : launch_attn(at, s);
+        };
         // activation rows per launch: the streamed kernels serve one or two
         const bool streamed = R <= 2;
         StreamArgs sa{};
@@ -665,8 +676,6 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             at.dim = D;
             at.map = map;
             at.R = R;
-            at.n_splits = clu ? ctx->attn_cs : ns;
-            at.split_len = attn_split_len(max_ctx, at.n_splits);
             at.q = ws.q;
             at.k_pages = kp;
             at.v_pages = vp;
@@ -679,8 +688,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             at.ticket = ws.attn_ticket;
             at.status = dev_status;
             if ((e = attn_probe(step * D.L + l, true)) != cudaSuccess) return cuda_fail(e, "probe record");
-            e = clu ? launch_attn_cluster(at, ctx->attn_cs, s) : launch_attn(at, s);
-            if (e != cudaSuccess) return cuda_fail(e, "attention launch");
+            if ((e = attention(at)) != cudaSuccess) return cuda_fail(e, "attention launch");
             if ((e = attn_probe(step * D.L + l, false)) != cudaSuccess) return cuda_fail(e, "probe record");
             // x += W_o attn;  x += W_down (silu(W_g n) * W_u n),  n = RMSNorm(x)
             const int ha = D.Hq * D.hd;
@@ -763,8 +771,6 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             at.dim = D;
             at.map = map;
             at.R = R;
-            at.n_splits = clu ? ctx->attn_cs : ns;
-            at.split_len = attn_split_len(max_ctx, at.n_splits);
             at.q = ws.q;
             at.k_pages = g.k_pages;
             at.v_pages = g.v_pages;
@@ -775,8 +781,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             at.ticket = ws.attn_ticket;
             at.status = dev_status;
             if ((e = attn_probe(step * D.L + l, true)) != cudaSuccess) return cuda_fail(e, "probe record");
-            e = clu ? launch_attn_cluster(at, ctx->attn_cs, s) : launch_attn(at, s);
-            if (e != cudaSuccess) return cuda_fail(e, "attention launch");
+            if ((e = attention(at)) != cudaSuccess) return cuda_fail(e, "attention launch");
             if ((e = attn_probe(step * D.L + l, false)) != cudaSuccess) return cuda_fail(e, "probe record");
             if (streamed && R == 1 && ctx->fused_mlp) {
                 MlpArgs ma{};

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "common.cuh"
 #include "osprey.h"
 
 namespace osp {
@@ -106,6 +107,26 @@ struct AttnArgs {
     int *ticket;
     int32_t *status;
 };
+
+// Attention output element (row r, column col of the Hq hd heads): float32
+// into out, or the three bf16 planes x ~= q0 + q1 + q2 (q_i the bf16 rounding of
+// what the earlier planes leave) of the O projection's tensor-core operand.
+__device__ __forceinline__ void attn_store(const AttnArgs &a, int r, int col, float v) {
+    const int ha = a.dim.Hq * a.dim.hd;
+    if (!a.out_planes) {
+        a.out[(size_t)r * ha + col] = v;
+        return;
+    }
+    const size_t plane = (size_t)a.npad * ha;
+    uint16_t *p = a.out_planes + (size_t)r * ha + col;
+    float rem = v;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const uint16_t q = f_to_bf(rem);
+        p[i * plane] = q;
+        rem -= bf_to_f(q);
+    }
+}
 
 struct LmArgs {
     Dims dim;
@@ -237,6 +258,11 @@ cudaError_t launch_keep_hidden(const float *x, bool ext, int B, int K, int step,
                                const int *valid, const int *nnew, float *hidden, cudaStream_t s);
 cudaError_t launch_gemv(GemvMode mode, const GemvArgs &a, int rg, int sms, cudaStream_t s);
 cudaError_t launch_attn(const AttnArgs &a, cudaStream_t s);
+// Extend rows (map.rows_per_seq > 1): a sequence's new rows together, 16 (row,
+// head) queries a block, attn_rows_tiles blocks per sequence, KV head and range;
+// a.n_splits from attn_splits of B x tiles rows.
+int attn_rows_tiles(const Dims &D, int max_new);
+cudaError_t launch_attn_rows(const AttnArgs &a, int B, int mtiles, cudaStream_t s);
 // Cluster size (16 or 8) the on-chip-merge attention can run with on the
 // current device for this shape, 0 if clusters are not available.
 int attn_cluster_size(const Dims &D);
