@@ -1257,6 +1257,7 @@ extern "C" int osprey_verify_hidden(osprey_ctx *ctx, int B, int K, int logits_dt
         ta.K = D.d;
         ta.nout = V;
         ta.planes = TC_LM_PLANES;
+        ta.wide = true;
         ta.y = hw.z;
         ta.x = hw.z;
         ta.ldy = V;

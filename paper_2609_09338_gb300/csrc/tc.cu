@@ -31,6 +31,7 @@ namespace cg = cooperative_groups;
 constexpr int TC_THREADS = 192;
 constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
 constexpr int TC_MAXST = 8;
+constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
 #ifndef OSP_TC_CTAS_PER_SM
 #define OSP_TC_CTAS_PER_SM 2   // two CTAs per SM: two TMA producers and two MMA chains per SM
 #endif
@@ -63,6 +64,16 @@ __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, int x, i
         "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar))
         : "memory");
 }
+// The same to this CTA's and the other CTAs' shared memory of the cluster (mask),
+// counted at the same place's barrier in each.
+__device__ __forceinline__ void tma_2d_multicast(void *dst, const CUtensorMap *m, int x, int y, uint64_t *bar,
+                                                 uint16_t mask) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
+        "%3}], [%4], %5;" ::"r"(smem_u32(dst)),
+        "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
+        : "memory");
+}
 // Shared-memory matrix descriptor: K-major tile, rows 128 bytes apart inside
 // 8-row (1024-byte) swizzle atoms.
 __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
@@ -85,6 +96,17 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
 __device__ __forceinline__ void tc_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+// ... arriving at the same place's barrier in every CTA of the mask
+__device__ __forceinline__ void tc_commit_multicast(uint64_t *bar, uint16_t mask) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(mask)
+        : "memory");
+}
+__device__ __forceinline__ void tc_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -145,7 +167,10 @@ __device__ __forceinline__ void lm_combine(float &a1, int &i1, float &s1, float 
 // planes: one work item is NA adjacent tiles, accumulated side by side in TMEM.
 // Output features [0, nout_a) come from the weights of map wa, the rest from
 // wb (row f - nout_a): the SwiGLU gate and up projections run as one GEMM.
-template <int EPI, int NA>
+// CS > 1 (several row tiles): the CTAs of a cluster of CS take adjacent row tiles
+// of the same features and k-range, and each weight tile is loaded once, by the
+// CTAs in turn, and multicast.  A slot is free when every CTA's MMAs have read it.
+template <int EPI, int NA, int CS>
 __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     tc_kernel(const __grid_constant__ CUtensorMap wa, const __grid_constant__ CUtensorMap wb,
               const __grid_constant__ CUtensorMap xm, const TcArgs a, int nst) {
@@ -155,13 +180,15 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // work item = (NA output tiles of 128 features, row tile, k-range), the k-range
-    // fastest; items of a CTA are contiguous
+    // work item of a cluster = (NA output tiles of 128 features, CS row tiles,
+    // k-range), the k-range fastest; items of a cluster are contiguous
     const int segkb = a.segkb;
-    const int per_ft = a.nrt * a.nsplit;   // items of one feature tile
+    const int nrg = a.nrt / CS, per_ft = nrg * a.nsplit;   // items of one feature tile
     const int n_items = (a.nout + 128 * NA - 1) / (128 * NA) * per_ft;
-    const int i0 = (int)((long long)n_items * blockIdx.x / gridDim.x);
-    const int i1 = (int)((long long)n_items * (blockIdx.x + 1) / gridDim.x);
+    const int rank = CS > 1 ? (int)(blockIdx.x % CS) : 0, cl = blockIdx.x / CS, ncl = gridDim.x / CS;
+    const int i0 = (int)((long long)n_items * cl / ncl);
+    const int i1 = (int)((long long)n_items * (cl + 1) / ncl);
+    constexpr uint16_t all = (uint16_t)((1 << CS) - 1);
     const int nloc = i1 - i0, nkb = a.K / 64, npad = a.npad;
     auto krange = [&](int item, int &lo, int &hi) {
         const int sp = item % a.nsplit;
@@ -186,7 +213,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     if (threadIdx.x == 32) {
         for (int i = 0; i < nst; ++i) {
             mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
+            mbar_init(&empty[i], CS);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&accf[i], 1);
@@ -198,7 +225,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
         mbar_fence_init();
     }
     tc_fence_before();
-    __syncthreads();
+    if (CS > 1) tc_cluster_sync();   // every CTA's barriers are ready for the others' copies and commits
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     pdl_trigger();
@@ -210,10 +238,14 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     if (warp == 0) {
         if (lane == 0) {
             auto weights = [&](uint8_t *st, int y, int kb, uint64_t *bar) {
+                if (CS > 1 && kb % CS != rank) return;   // another CTA of the cluster brings them
 #pragma unroll
                 for (int t = 0; t < NA; ++t) {
                     const int f = y + 128 * t;   // tiles never straddle nout_a (a multiple of 128)
-                    tma_2d(st + t * TC_ABYTES, f < a.nout_a ? &wa : &wb, kb * 64, f < a.nout_a ? f : f - a.nout_a, bar);
+                    const CUtensorMap *w = f < a.nout_a ? &wa : &wb;
+                    const int r = f < a.nout_a ? f : f - a.nout_a;
+                    if constexpr (CS > 1) tma_2d_multicast(st + t * TC_ABYTES, w, kb * 64, r, bar, all);
+                    else tma_2d(st + t * TC_ABYTES, w, kb * 64, r, bar);
                 }
             };
             long long npre = 0;   // stages whose weights were requested before the wait
@@ -231,7 +263,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             bool stop = false;
             for (int it = 0; it < nloc && !stop; ++it) {
                 const int y = (i0 + it) / per_ft * 128 * NA;
-                const int row0 = (i0 + it) / a.nsplit % a.nrt * npad;   // of the operand planes
+                const int row0 = ((i0 + it) / a.nsplit % nrg * CS + rank) * npad;   // of the operand planes
                 int klo, khi;
                 krange(i0 + it, klo, khi);
                 for (int kb = klo; kb < khi; ++kb, ++g) {
@@ -325,7 +357,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                                 for (int kk = 0; kk < 4; ++kk)
                                     step(p, kk, d0, (kb != kb0) || kk || p != a.planes - 1);
                         }
-                        tc_commit(&empty[s]);
+                        if (CS > 1) tc_commit_multicast(&empty[s], all);
+                        else tc_commit(&empty[s]);
                     }
                     if (!stop) tc_commit(&accf[buf]);
                 }
@@ -407,7 +440,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             ft = (i0 + it) / per_ft;
             sp = (i0 + it) % a.nsplit;
             col0 = ft * 128 * NA + m;
-            row0 = (i0 + it) / a.nsplit % a.nrt * npad;
+            row0 = ((i0 + it) / a.nsplit % nrg * CS + rank) * npad;
             int klo, khi;
             krange(i0 + it, klo, khi);
             const int nseg = (khi - klo + segkb - 1) / segkb;
@@ -507,7 +540,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
         }
     }
     tc_fence_before();
-    __syncthreads();
+    if (CS > 1) tc_cluster_sync();   // the other CTAs write nothing more to this one's shared memory
+    else __syncthreads();
     tc_fence_after();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
@@ -1059,16 +1093,22 @@ size_t tc_smem_bytes(int npad, int planes, int na) {
     return (size_t)tc_stages(npad, planes, na) * stage + 1024;
 }
 
+template <int EPI, int NA, int CS>
+static cudaError_t tc_allow_smem() {
+    return cudaFuncSetAttribute(tc_kernel<EPI, NA, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_CAP);
+}
+
 cudaError_t tc_set_attributes() {
-    const int bytes = (int)TC_SMEM_CAP;
-    cudaError_t e = cudaFuncSetAttribute(tc_kernel<TC_STORE, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_kernel<TC_RESID, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(tc_kernel<TC_GLU, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(tc_kernel<TC_LM, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (e == cudaSuccess && OSP_TC_LM_NA > 1)
-        e = cudaFuncSetAttribute(tc_kernel<TC_LM, OSP_TC_LM_NA>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = tc_allow_smem<TC_STORE, 1, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_STORE, 1, TC_CS>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_STORE, OSP_TC_LM_NA, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_RESID, 1, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_RESID, 1, TC_CS>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_GLU, 1, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_GLU, 1, TC_CS>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, TC_CS>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, OSP_TC_LM_NA, 1>();
     if (e == cudaSuccess) e = allow_smem(lm_pick_kernel);
     return e;
 }
@@ -1086,6 +1126,29 @@ static cudaError_t pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t sme
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, k, args...);
+    count_launch();
+    return e;
+}
+
+template <int EPI, int NA, int CS>
+static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtensorMap &wa, const CUtensorMap &wb,
+                             const CUtensorMap &xm, const TcArgs &a, int nst) {
+    if (CS == 1) return pdl_launch(tc_kernel<EPI, NA, CS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CS;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_kernel<EPI, NA, CS>, wa, wb, xm, a, nst);
     count_launch();
     return e;
 }
@@ -1136,7 +1199,8 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     // reduction over d is short: one segment keeps its MMA chain at 4 d / 64 steps
     // per plane)
     int na = 1;
-    if (a.epi == TC_LM && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA) >= 2 &&
+    const bool wide = a.epi == TC_LM || (a.epi == TC_STORE && a.nsplit == 1 && a.wide);
+    if (wide && a.nrt == 1 && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA) >= 2 &&
         2 * OSP_TC_LM_NA * a.npad <= tmem_cols && a.kbps <= 32 && a.planes <= TC_LM_PLANES) {
         na = OSP_TC_LM_NA;
         a.segkb = a.kbps;
@@ -1144,22 +1208,30 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     const int nst = tc_stages(a.npad, a.planes, na);
     if (nst < 2) return cudaErrorInvalidValue;
     if ((na == 1 && a.sep ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
-    const int items = (a.nout + 128 * na - 1) / (128 * na) * a.nrt * a.nsplit;
-    const int grid = items < OSP_TC_CTAS_PER_SM * sms ? items : OSP_TC_CTAS_PER_SM * sms;
+    const int cs = a.nrt > 1 ? TC_CS : 1;   // several row tiles (an even number, tc_tiles) share the weights
+    if (a.nrt % cs || (cs > 1 && na > 1)) return cudaErrorInvalidValue;
+    const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / cs) * a.nsplit, slots = OSP_TC_CTAS_PER_SM * sms / cs;
+    const int grid = (items < slots ? items : slots) * cs;
     const size_t smem = tc_smem_bytes(a.npad, a.planes, na);
     cudaError_t e;
     switch (a.epi) {
     case TC_STORE:
-        e = pdl_launch(tc_kernel<TC_STORE, 1>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
+        e = cs > 1   ? tc_launch<TC_STORE, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
+            : na > 1 ? tc_launch<TC_STORE, OSP_TC_LM_NA, 1>(grid, smem, s, wa, wb, xm, a, nst)
+                     : tc_launch<TC_STORE, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
         break;
     case TC_RESID:
-        e = pdl_launch(tc_kernel<TC_RESID, 1>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
+        e = cs > 1 ? tc_launch<TC_RESID, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
+                   : tc_launch<TC_RESID, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
         break;
-    case TC_GLU: e = pdl_launch(tc_kernel<TC_GLU, 1>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst); break;
+    case TC_GLU:
+        e = cs > 1 ? tc_launch<TC_GLU, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
+                   : tc_launch<TC_GLU, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
+        break;
     default:
-        e = na > 1
-                ? pdl_launch(tc_kernel<TC_LM, OSP_TC_LM_NA>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst)
-                : pdl_launch(tc_kernel<TC_LM, 1>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
+        e = cs > 1   ? tc_launch<TC_LM, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
+            : na > 1 ? tc_launch<TC_LM, OSP_TC_LM_NA, 1>(grid, smem, s, wa, wb, xm, a, nst)
+                     : tc_launch<TC_LM, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
         break;
     }
     if (e != cudaSuccess || (a.nsplit == 1 && a.epi != TC_GLU)) return e;

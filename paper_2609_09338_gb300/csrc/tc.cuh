@@ -4,8 +4,8 @@
 //
 // Weights are the M = 128 operand, streamed tile by tile with 2-D TMA (128-byte
 // swizzle); the R activation rows are the N operand, in equal tiles of at most
-// 80 rows (padded to a multiple of 16).  The row tiles of one weight tile are
-// adjacent work items, so all but the first read the weights from L2.  The LM head multiplies two weight tiles against each stage's operand
+// 80 rows (padded to a multiple of 16).  Two row tiles at a time share each weight
+// tile: a cluster of two CTAs loads it once and multicasts it.  The LM head multiplies two weight tiles against each stage's operand
 // planes (twice the weight bytes in flight per byte of operand reloaded).  Activations are float32 between kernels; for the tensor cores each is
 // split into three bf16 planes, q0 = bf16(x), q1 = bf16(x - q0), q2 =
 // bf16(x - q0 - q1), and every k-step issues one MMA per plane into the same
@@ -57,6 +57,7 @@ inline TcTiles tc_tiles(long long rows) {
     TcTiles t;
     t.nrt = (int)((rows + TC_TILE_ROWS - 1) / TC_TILE_ROWS);
     if (t.nrt < 1) t.nrt = 1;
+    if (t.nrt > 1) t.nrt += t.nrt & 1;   // pairs of tiles share the weights they load
     t.npad = (int)(((rows + t.nrt - 1) / t.nrt + 15) / 16 * 16);
     return t;
 }
@@ -69,6 +70,7 @@ struct TcArgs {
     int nout;          // output features (tiles of 128, the last one may be partial)
     int nout_a;        // features [0, nout_a) from the first weight map, the rest from the second
     int planes;        // 1 (bf16 input) or TC_PLANES (split float32 input)
+    bool wide;         // TC_STORE of the LM head: the LM head's tiles, so the same sums bit for bit
     float *y;          // TC_STORE: [R][ldy] float32 output
     int ldy;
     float *x;          // TC_RESID: [R][ldy] float32, +=
