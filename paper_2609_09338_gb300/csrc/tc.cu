@@ -28,13 +28,14 @@ namespace osp {
 
 namespace cg = cooperative_groups;
 
-constexpr int TC_THREADS = 192;
-constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
-constexpr int TC_MAXST = 8;
-constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
 #ifndef OSP_TC_CTAS_PER_SM
 #define OSP_TC_CTAS_PER_SM 2   // two CTAs per SM: two TMA producers and two MMA chains per SM
 #endif
+constexpr int TC_THREADS = 192;
+constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
+constexpr int TC_MAXST = 8;
+constexpr int TC_TMEM_COLS = 512 / OSP_TC_CTAS_PER_SM;   // of one CTA
+constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
 constexpr size_t TC_SMEM_CAP = (OSP_TC_CTAS_PER_SM == 1 ? 200 : 100) * 1024;
 #ifndef OSP_TC_SEGKB
 #define OSP_TC_SEGKB 8   // k-blocks (64 wide) per accumulation segment
@@ -149,17 +150,11 @@ __device__ __forceinline__ void tc_split(float x, uint16_t (&q)[TC_PLANES]) {
     }
 }
 
-// Merges two (argmax logit a with its id i, sum s of exp((z - a) / T)) pairs
-// into the first: the larger logit wins (the lower id on ties) and the
-// other's sum is rescaled to it.
-__device__ __forceinline__ void lm_combine(float &a1, int &i1, float &s1, float a2, int i2, float s2, float invT) {
-    const bool two = a2 > a1 || (a2 == a1 && i2 < i1);
-    const float aw = two ? a2 : a1, al = two ? a1 : a2;
-    const float sw = two ? s2 : s1, sl = two ? s1 : s2;
-    const float f = al == -INFINITY ? 0.f : __expf((al - aw) * invT);
-    a1 = aw;
-    i1 = two ? i2 : i1;
-    s1 = sw + sl * f;
+// 2^x on the special-function unit (PTX ex2.approx, flush-to-zero)
+__device__ __forceinline__ float lm_ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 // ---------------------------------------------------------------- GEMM kernel
@@ -202,8 +197,11 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     // the first plane, so what their accumulator drops does not matter)
     const uint32_t acc_cols = NA * npad;
     const bool sep = NA == 1 && a.sep;
+    // an item of several segments is finished from columns of its own where they
+    // fit (tiles of up to 64 rows), so that its last segment's buffer is free at once
+    const bool own = NA == 1 && a.kbps > a.segkb && 4 * acc_cols <= TC_TMEM_COLS;
     uint32_t ncols = 32;
-    while (ncols < (sep ? 3 : 2) * acc_cols) ncols <<= 1;
+    while (ncols < (own ? 4 : sep ? 3 : 2) * acc_cols) ncols <<= 1;
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
@@ -379,20 +377,29 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             const int col = col0 + 128 * tile;
             const bool colok = col < a.nout;
             if constexpr (EPI == TC_LM) {
-                // per row: (argmax z, sum exp((z - max z) / T)) over this warp's 32
-                // ids, for the 16 rows c0.. at once: each butterfly round halves the
-                // rows a lane carries (it keeps one half and receives the partner's
-                // share of it), so after four rounds lane l holds row l / 2 over 16
-                // lanes and one more exchange completes it over all 32
+                // per row: (argmax z, sum exp((z - max z) / T)) over this warp's 32 ids,
+                // for the 16 rows c0.. at once: the maximum by a warp reduction, its
+                // first lane by a ballot, then the sums by a butterfly that halves the
+                // rows a lane carries each round (it keeps one half and receives the
+                // partner's share of it), so that lane l ends with row l / 2.  About 220
+                // instructions a chunk, independent across rows; merging (max, sum, id)
+                // triples through the butterfly took 500 in a chain, 2.8 us a chunk
                 const int sub = (int)(((long long)ft * 128 * NA + 128 * tile + lg) / TC_LM_GROUP);
-                float av[16], sv[16];
-                int ai[16];
+                const float c2 = a.lm_invT * 1.4426950408889634f;
+                float e[16], mine = -INFINITY;
+                int first = -1;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
-                    av[j] = colok ? v[j] : -INFINITY;
-                    ai[j] = colok ? col : 0x7fffffff;
-                    sv[j] = colok ? 1.f : 0.f;
                     if (a.y && colok && row0 + c0 + j < a.R) a.y[(size_t)(row0 + c0 + j) * a.ldy + col] = v[j];
+                    const float z = colok ? v[j] : -INFINITY;
+                    float mx;
+                    asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(mx) : "f"(z));
+                    const unsigned at = __ballot_sync(0xffffffffu, z == mx);
+                    e[j] = mx == -INFINITY ? 0.f : lm_ex2((z - mx) * c2);
+                    if ((lane >> 1) == j) {
+                        mine = mx;
+                        first = __ffs(at) - 1;
+                    }
                 }
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
@@ -400,27 +407,16 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                     const bool up = lane & off;
 #pragma unroll
                     for (int i = 0; i < w; ++i) {
-                        const float ra = __shfl_xor_sync(0xffffffffu, up ? av[i] : av[i + w], off);
-                        const int ri = __shfl_xor_sync(0xffffffffu, up ? ai[i] : ai[i + w], off);
-                        const float rs = __shfl_xor_sync(0xffffffffu, up ? sv[i] : sv[i + w], off);
-                        float ka = up ? av[i + w] : av[i], ks = up ? sv[i + w] : sv[i];
-                        int ki = up ? ai[i + w] : ai[i];
-                        lm_combine(ka, ki, ks, ra, ri, rs, a.lm_invT);
-                        av[i] = ka;
-                        ai[i] = ki;
-                        sv[i] = ks;
+                        const float got = __shfl_xor_sync(0xffffffffu, up ? e[i] : e[i + w], off);
+                        e[i] = (up ? e[i + w] : e[i]) + got;
                     }
                 }
-                {
-                    const float ra = __shfl_xor_sync(0xffffffffu, av[0], 1);
-                    const int ri = __shfl_xor_sync(0xffffffffu, ai[0], 1);
-                    const float rs = __shfl_xor_sync(0xffffffffu, sv[0], 1);
-                    lm_combine(av[0], ai[0], sv[0], ra, ri, rs, a.lm_invT);
-                }
+                e[0] += __shfl_xor_sync(0xffffffffu, e[0], 1);
                 const int n = row0 + c0 + (lane >> 1);
                 if (!(lane & 1) && n < a.R && sub < a.lm_nsub)
                     a.lm_part[(size_t)n * a.lm_nsub + sub] =
-                        make_float4(av[0] * a.lm_invT, sv[0], av[0], __int_as_float(ai[0]));
+                        make_float4(mine * a.lm_invT, e[0], mine,
+                                    __int_as_float(mine == -INFINITY ? 0x7fffffff : col - lane + first));
             } else {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -462,7 +458,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             if constexpr (NA == 1) {
                 // several segments: the running total is kept in registers, each segment
                 // added to it in float32 and its buffer freed at once, and is put back
-                // into the last segment's buffer, from which the loop below finishes it
+                // into TMEM, from which the loop below finishes it
                 // (a loop over chunks in TMEM: unrolled over registers, its code is five
                 // times as long, which cost each short launch 5 us of instruction fetches)
                 if (nseg > 1) {
@@ -504,9 +500,10 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&sepe);
                     }
+                    if (own) release();
 #pragma unroll
                     for (int c = 0; c < NCH; ++c)
-                        if (c < nch) tc_st16(lanes + (uint32_t)(u & 1) * acc_cols + 16u * c, tot[c]);
+                        if (c < nch) tc_st16(lanes + (own ? 3u : (uint32_t)(u & 1)) * acc_cols + 16u * c, tot[c]);
                     tc_st_wait();
                 } else if (!wait_acc()) {
                     break;
@@ -514,7 +511,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             } else if (!wait_acc()) {   // one segment an item
                 break;
             }
-            const uint32_t t0 = lanes + (uint32_t)(u & 1) * acc_cols;
+            const bool freed = own && nseg > 1;
+            const uint32_t t0 = lanes + (freed ? 3u : (uint32_t)(u & 1)) * acc_cols;
             for (int cc = 0; cc < NA * npad; cc += 16) {
                 // accumulator columns [t npad, (t + 1) npad) hold tile t's rows
                 const int tile = cc / npad;
@@ -534,8 +532,8 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                 }
                 finish(tile, cc - tile * npad, v);
             }
-            release();
-            if (sep && nseg == 1 && lane == 0) mbar_arrive(&sepe);   // after release()'s warp barrier
+            if (!freed) release();
+            if (sep && nseg == 1 && lane == 0) mbar_arrive(&sepe);   // (one segment: after release()'s warp barrier)
             ++u;
         }
     }
@@ -1193,7 +1191,7 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     a.kbps = (nkb + a.nsplit - 1) / a.nsplit;
     a.sep = a.planes > 1;   // (0.1 % of a call, for a third of the accumulators' error)
     a.segkb = a.fine ? OSP_TC_SEGKB_FINE : OSP_TC_SEGKB;
-    constexpr int tmem_cols = 512 / OSP_TC_CTAS_PER_SM;
+    constexpr int tmem_cols = TC_TMEM_COLS;
     // the LM head takes OSP_TC_LM_NA weight tiles per stage when two stages fit
     // and the double-buffered accumulators fit TMEM in one segment (the LM head's
     // reduction over d is short: one segment keeps its MMA chain at 4 d / 64 steps
