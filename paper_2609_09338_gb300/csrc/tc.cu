@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                     else tma_2d(st + t * TC_ABYTES, w, kb * 64, r, bar);
                 }
             };
-            long long npre = 0;   // stages whose weights were requested before the wait
+            int npre = 0;   // stages whose weights were requested before the wait
             for (int it = 0; it < nloc && npre < nst; ++it) {
                 const int y = (i0 + it) / per_ft * 128 * NA;
                 int klo, khi;
@@ -257,16 +257,22 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                 }
             }
             pdl_wait();
-            long long g = 0;
+            // slot and use of the ring advance by increments: a division by the runtime
+            // number of stages, twice a k-block, took longer than its MMAs
+            int g = 0, s = 0;          // k-block of the CTA, its slot
+            uint32_t ph = 1;           // parity of the slot's previous use
             bool stop = false;
             for (int it = 0; it < nloc && !stop; ++it) {
                 const int y = (i0 + it) / per_ft * 128 * NA;
                 const int row0 = ((i0 + it) / a.nsplit % nrg * CS + rank) * npad;   // of the operand planes
                 int klo, khi;
                 krange(i0 + it, klo, khi);
-                for (int kb = klo; kb < khi; ++kb, ++g) {
-                    const int s = (int)(g % nst);
-                    if (g >= nst && !mbar_wait(&empty[s], (uint32_t)((g / nst) - 1) & 1)) {
+                for (int kb = klo; kb < khi; ++kb, ++g, ++s) {
+                    if (s == nst) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                    if (g >= nst && !mbar_wait(&empty[s], ph)) {
                         set_status(a.status, OSPREY_ERR_TIMEOUT);
                         atomicExch(&s_abort, 1);
                         stop = true;
@@ -288,9 +294,9 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             if (stop) {   // let the copies this thread issued land before the CTA can exit
                 // stages whose weights were requested early but never armed: arrive, so
                 // that their phase completes when the weights land
-                for (long long q = g; q < npre; ++q) mbar_arrive(&full[q]);
-                const long long end = g > npre ? g : npre;
-                for (long long q = end - nst > 0 ? end - nst : 0; q < end; ++q)
+                for (int q = g; q < npre; ++q) mbar_arrive(&full[q]);
+                const int end = g > npre ? g : npre;
+                for (int q = end - nst > 0 ? end - nst : 0; q < end; ++q)
                     mbar_wait(&full[q % nst], (uint32_t)(q / nst) & 1, 200000000LL);
             }
         }
@@ -298,14 +304,15 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
         if (lane == 0) {
             // one accumulation unit = one segment of one tile, into buffer u & 1
             const uint32_t idesc = tc_idesc(128, npad);
-            long long g = 0, u = 0;
+            int u = 0, s = 0;          // accumulation unit, ring slot
+            uint32_t ph = 0;           // parity of the slot's current use
             bool stop = false;
             for (int it = 0; it < nloc && !stop; ++it) {
                 int klo, khi;
                 krange(i0 + it, klo, khi);
                 const int nseg = (khi - klo + segkb - 1) / segkb;
                 for (int sg = 0; sg < nseg && !stop; ++sg, ++u) {
-                    const int buf = (int)(u & 1);
+                    const int buf = u & 1;
                     if (u >= 2 && !mbar_wait(&acce[buf], (uint32_t)((u >> 1) - 1) & 1)) {
                         set_status(a.status, OSPREY_ERR_TIMEOUT);
                         atomicExch(&s_abort, 1);
@@ -315,9 +322,12 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                     tc_fence_after();
                     const uint32_t d0 = tmem + (uint32_t)buf * acc_cols;
                     const int kb0 = klo + sg * segkb, kb1 = min(khi, kb0 + segkb);
-                    for (int kb = kb0; kb < kb1; ++kb, ++g) {
-                        const int s = (int)(g % nst);
-                        if (!mbar_wait(&full[s], (uint32_t)(g / nst) & 1) || *(volatile int *)&s_abort) {
+                    for (int kb = kb0; kb < kb1; ++kb, ++s) {
+                        if (s == nst) {
+                            s = 0;
+                            ph ^= 1;
+                        }
+                        if (!mbar_wait(&full[s], ph) || *(volatile int *)&s_abort) {
                             set_status(a.status, OSPREY_ERR_TIMEOUT);
                             atomicExch(&s_abort, 1);
                             stop = true;
@@ -369,7 +379,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
         const int lg = (warp & 3) * 32;
         const int m = lg + lane;
         const uint32_t lanes = tmem + ((uint32_t)lg << 16);
-        long long u = 0;
+        int u = 0;
         bool stop = false;
         int ft = 0, sp = 0, col0 = 0, row0 = 0;
         // the finished sums v of rows row0 + c0 .. + 15, feature col0 + 128 tile
