@@ -94,6 +94,14 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
                  "l"(a), "l"(b), "r"(idesc), "r"(acc)
                  : "memory");
 }
+// One lane of a converged warp.  A role's loop runs under this predicate rather
+// than a test of the lane's number: the compiler then knows that a single thread
+// issues, and keeps descriptors and addresses in uniform registers.
+__device__ __forceinline__ bool tc_elect() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
 __device__ __forceinline__ void tc_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
@@ -234,7 +242,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     if (warp != 0) pdl_wait();
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (tc_elect()) {
             auto weights = [&](uint8_t *st, int y, int kb, uint64_t *bar) {
                 if (CS > 1 && kb % CS != rank) return;   // another CTA of the cluster brings them
 #pragma unroll
@@ -301,9 +309,9 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (tc_elect()) {
             // one accumulation unit = one segment of one tile, into buffer u & 1
-            const uint32_t idesc = tc_idesc(128, npad);
+            const uint32_t idesc = tc_idesc(128, npad), pstep = (uint32_t)npad * 128 >> 4;   // descriptor units a plane
             int u = 0, s = 0;          // accumulation unit, ring slot
             uint32_t ph = 0;           // parity of the slot's current use
             bool stop = false;
@@ -335,12 +343,12 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                         }
                         tc_fence_after();
                         const uint32_t st = smem_u32(sm + (size_t)s * stage);
+                        const uint64_t da = tc_desc(st), db0 = tc_desc(st + NA * TC_ABYTES);
                         auto step = [&](int p, int kk, uint32_t d, uint32_t acc) {
-                            const uint64_t db = tc_desc(st + NA * TC_ABYTES + (uint32_t)p * npad * 128);
+                            const uint64_t db = db0 + (uint64_t)(p * pstep) + 2 * kk;
 #pragma unroll
                             for (int t = 0; t < NA; ++t)
-                                tc_mma(d + (uint32_t)(t * npad), tc_desc(st + t * TC_ABYTES) + 2 * kk, db + 2 * kk,
-                                       idesc, acc);
+                                tc_mma(d + (uint32_t)(t * npad), da + t * (TC_ABYTES >> 4) + 2 * kk, db, idesc, acc);
                         };
                         if (sep) {
 #pragma unroll
