@@ -36,7 +36,11 @@ constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
 constexpr int TC_MAXST = 8;
 constexpr int TC_TMEM_COLS = 512 / OSP_TC_CTAS_PER_SM;   // of one CTA
 constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
-constexpr size_t TC_SMEM_CAP = (OSP_TC_CTAS_PER_SM == 1 ? 200 : 100) * 1024;
+constexpr long long TC_SHARE_BYTES = 40ll << 20;   // weights above which they do
+// two CTAs, the system's share and the static part fit 228 KB.  100 KB left the
+// third stage of 48 rows and the fifth of 16 out: 96 sequences 2945 us a call,
+// 16 sequences 1992; with it 2904 and 1970
+constexpr size_t TC_SMEM_CAP = (OSP_TC_CTAS_PER_SM == 1 ? 200 : 112) * 1024;
 #ifndef OSP_TC_SEGKB
 #define OSP_TC_SEGKB 8   // k-blocks (64 wide) per accumulation segment
 #endif
@@ -1224,7 +1228,11 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     const int nst = tc_stages(a.npad, a.planes, na);
     if (nst < 2) return cudaErrorInvalidValue;
     if ((na == 1 && a.sep ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
-    const int cs = a.nrt > 1 ? TC_CS : 1;   // several row tiles (an even number, tc_tiles) share the weights
+    // several row tiles (an even number, tc_tiles) share weights that the L2 does not
+    // keep from one tile to the next: d 4096 (100..235 MB a projection, 1.2 GB of LM
+    // head) 2136 us a call without, 2027 with.  Projections of 4..33 MB gain nothing
+    // and pay the clusters' start (d 1024, 96 rows: 1 us of 12..18 a launch)
+    const int cs = a.nrt > 1 && (long long)a.nout * a.K * 2 > TC_SHARE_BYTES ? TC_CS : 1;
     if (a.nrt % cs || (cs > 1 && na > 1)) return cudaErrorInvalidValue;
     const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / cs) * a.nsplit, slots = OSP_TC_CTAS_PER_SM * sms / cs;
     const int grid = (items < slots ? items : slots) * cs;
