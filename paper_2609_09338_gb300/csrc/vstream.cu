@@ -32,7 +32,7 @@
 // Logits-free form (HID): vs_stats reads the target rows only and the decision
 // takes q_i(x_i) and (M, log S) from the draft step; vs_sample takes a group's
 // draft rows from `zrec` (float32 whatever the target's type).  V 200064, B 64,
-// K 8, bf16: 176 us a call, of which the target's 230 MB take 45; with unstreamed
+// K 8, bf16: 165 us a call, of which the target's 230 MB take 55; with unstreamed
 // kernels for the rows and two launches for the decision rows' operand 238.
 // Both kernels are launched as programmatic dependents: barrier set-up overlaps
 // the previous kernel's tail, and every global read follows griddepcontrol.wait.
@@ -204,6 +204,15 @@ __device__ __forceinline__ void vs_mask(uint4 (&r)[VS_NV], int lane, int nel) {
         if ((lane + 32 * k) * L::VW >= nel) r[k] = make_uint4(L::NEG, L::NEG, L::NEG, L::NEG);
 }
 
+__device__ __forceinline__ uint64_t vs_pair(float lo, float hi) {
+    uint64_t p;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(lo), "f"(hi));
+    return p;
+}
+__device__ __forceinline__ void vs_unpair(uint64_t p, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+
 // Sum over the lane's vectors of exp((x - m) / T) = 2^((x - m) c), c = log2(e)/T.
 // SUB: the difference first, which is exact near the maximum; else as
 // 2^(x c - m c), one operation less, off by the rounding of m c (1e-6 where
@@ -212,17 +221,30 @@ template <typename T, bool SUB, int N>
 __device__ __forceinline__ float vs_sum_exp(const uint4 (&r)[N], float c, float m) {
     using L = VsT<T>;
     const float mc = m * c;
-    float s0 = 0.f, s1 = 0.f;
+    // two elements an instruction (f32x2), two sums
+    const uint64_t c2 = vs_pair(c, c), n2 = SUB ? vs_pair(-m, -m) : vs_pair(-mc, -mc);
+    uint64_t s = vs_pair(0.f, 0.f);
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         float f[L::VW];
         L::unpack(r[k], f);
 #pragma unroll
         for (int e = 0; e < L::VW; e += 2) {
-            s0 += vs_ex2(SUB ? (f[e] - m) * c : fmaf(f[e], c, -mc));
-            s1 += vs_ex2(SUB ? (f[e + 1] - m) * c : fmaf(f[e + 1], c, -mc));
+            const uint64_t x = vs_pair(f[e], f[e + 1]);
+            uint64_t y;
+            if (SUB) {
+                asm("add.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(x), "l"(n2));
+                asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(y), "l"(c2));
+            } else {
+                asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(y) : "l"(x), "l"(c2), "l"(n2));
+            }
+            float y0, y1;
+            vs_unpair(y, y0, y1);
+            asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(s), "l"(vs_pair(vs_ex2(y0), vs_ex2(y1))));
         }
     }
+    float s0, s1;
+    vs_unpair(s, s0, s1);
     return s0 + s1;
 }
 
