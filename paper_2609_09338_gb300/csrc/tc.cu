@@ -821,46 +821,61 @@ __global__ void __launch_bounds__(256) tc_reduce_rope_kernel(const TcArgs a, con
 }
 
 // ---------------------------------------------------------------- LM-head pick
-constexpr int PK_THREADS = 1024;   // each thread walks about V / 32 / 1024 partials
-
+constexpr int PK_THREADS = 1024, PK_WARPS = PK_THREADS / 32;
+constexpr int PK_CH = 8;     // partials a lane holds (a row of 32 x 8 x 32 groups, V 262144; beyond, they are read again)
 constexpr int PK_MAXK = 8;   // candidates per row at most
 
-// Recomputes the 32 logits of group g (ids 32 g ..): 8 warps x 4 ids, lanes
-// split the reduction over the row's operand in shared memory.
-__device__ __forceinline__ void pk_group_logits(const LmPickArgs &a, const float *hrow, int g, float *z) {
+// Recomputes the 32 logits of each of n groups (ids 32 g ..): warp w takes id w of
+// every group, two groups at a time, lanes split the reduction over the row's
+// operand in shared memory.
+__device__ __forceinline__ void pk_group_logits(const LmPickArgs &a, const float *hrow, const int *grp, int n, float *z) {
     const Dims &D = a.dim;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    constexpr int PER = TC_LM_GROUP / (PK_THREADS / 32);
-    for (int i = 0; i < PER; ++i) {
-        const int id = g * TC_LM_GROUP + warp * PER + i;
-        float acc = 0.f;
-        if (id < D.V) {
-            const uint16_t *wr = a.W + (size_t)id * D.d;
-            for (int k = lane * 8; k < D.d; k += 256) {
-                float wf[8];
-                unpack8(ld_stream(wr + k), wf);
+    static_assert(TC_LM_GROUP == PK_WARPS, "an id a warp");
+    for (int q = 0; q < n; q += 2) {
+        int id[2];
+        const uint16_t *wr[2];
+        float acc[2] = {0.f, 0.f};
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc = fmaf(wf[e], hrow[k + e], acc);
+        for (int e = 0; e < 2; ++e) {
+            id[e] = q + e < n && grp[q + e] >= 0 ? grp[q + e] * TC_LM_GROUP + warp : D.V;
+            wr[e] = a.W + (size_t)(id[e] < D.V ? id[e] : 0) * D.d + lane * 8;
+        }
+#pragma unroll 4
+        for (int k = 0; k < D.d; k += 256) {   // (d is a multiple of 256)
+            const uint4 w0 = ld_stream(wr[0] + k), w1 = q + 1 < n ? ld_stream(wr[1] + k) : make_uint4(0, 0, 0, 0);
+            float f0[8], f1[8];
+            unpack8(w0, f0);
+            unpack8(w1, f1);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float h = hrow[k + lane * 8 + e];
+                acc[0] = fmaf(f0[e], h, acc[0]);
+                acc[1] = fmaf(f1[e], h, acc[1]);
             }
         }
-        acc = warp_sum(acc);
-        if (lane == 0) z[warp * PER + i] = id < D.V ? acc : -INFINITY;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float v = warp_sum(acc[e]);
+            if (lane == 0 && q + e < n) z[(q + e) * TC_LM_GROUP + warp] = id[e] < D.V ? v : -INFINITY;
+        }
     }
 }
 
-// One block per row.  Level 1: the row's 32-id partials, a contiguous run per
-// thread, give M = max y, S = sum exp(y - M) and, per draw, the group holding
+// One block per row, bound by the latency of its steps: 64 rows of 6252 partials
+// 12 us a launch, 16 rows with four greedy candidates 25 (17 and 37 when a thread
+// walked a run of its own and every candidate cost passes over the partials).  Level 1: warp w holds the w-th contiguous range of the row's
+// 32-id partials, lanes side by side (coalesced, all loads in flight), which gives
+// M = max y, S = sum exp(y - M) and, per draw, the warp and then the group holding
 // u * S.  Level 2: that group's 32 logits, recomputed as dot products of the
 // LM-head rows with the row's operand (the sum of its bf16 planes), scanned in
 // ascending ids.  Greedy: the argmax from the partials; with topk > 1 the next
 // candidates come from the topk groups of largest maximum (the only groups
-// that can hold one of the topk largest logits), recomputed and ranked.
+// that can hold one of the topk largest logits), recomputed together and ranked.
 __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a) {
     extern __shared__ float hrow[];   // [d] the row's LM-head operand
-    __shared__ MS sm_ms[PK_THREADS / 32];
-    __shared__ AM sm_am[PK_THREADS / 32];
-    __shared__ float sh[34];
-    __shared__ int si[2];
+    __shared__ AM sm_am[2][PK_WARPS];
+    __shared__ float sm_m[PK_WARPS], sm_w[PK_WARPS], sh[PK_WARPS];
     __shared__ float s_z[PK_MAXK * TC_LM_GROUP];
     __shared__ int s_grp[PK_MAXK], s_tok[PK_MAXK];
     __shared__ float s_before, s_e[PK_MAXK];
@@ -873,103 +888,179 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
     const bool greedy = a.temperature == 0.f;
     const float invT = greedy ? 1.f : 1.f / a.temperature;
     const float4 *pp = a.part + (size_t)b * a.nsub;
-    const int per = (a.nsub + PK_THREADS - 1) / PK_THREADS;
-    const int j0 = min(a.nsub, t * per), j1 = min(a.nsub, j0 + per);
-    // one pass over the thread's run: its argmax and its (max, sum) rescaled online
-    float m = -INFINITY, sm = 0.f;
+    const int per = ((a.nsub + PK_WARPS - 1) / PK_WARPS + 31) / 32 * 32;   // partials of a warp
+    const int j0 = min(a.nsub, warp * per), j1 = min(a.nsub, j0 + per);
+    const int nch = (j1 - j0 + 31) / 32;                                   // of a lane
+    float px[PK_CH], py[PK_CH];
+    float m = -INFINITY;
     AM am{-INFINITY, 0x7fffffff};
-    for (int j = j0; j < j1; ++j) {
-        const float4 p = __ldcg(pp + j);
-        am = am_combine(am, AM{p.z, __float_as_int(p.w)});
-        if (p.x == -INFINITY) continue;
-        if (p.x > m) {
-            sm = (m == -INFINITY ? 0.f : sm * __expf(m - p.x)) + p.y;
-            m = p.x;
-        } else {
-            sm += p.y * __expf(p.x - m);
-        }
-    }
-    const MS tot = block_ms(MS{m, sm}, sm_ms);
-    const float M = tot.m, S = tot.s;
-    const float w = m == -INFINITY ? 0.f : sm * __expf(m - M);   // the run's weight
-    if (topk > 1 || !greedy) {
-        // the row's operand: the sum of its planes (the values the tensor cores multiplied)
-        const size_t plane = (size_t)a.npad * D.d;
-        const uint16_t *q = a.planes + (size_t)b * D.d;
-        for (int k = t; k < D.d; k += PK_THREADS) {
-            float h = 0.f;
+    {
+        float4 v[PK_CH];
 #pragma unroll
-            for (int i = 0; i < TC_PLANES; ++i)
-                if (i < a.npl) h += bf_to_f(q[i * plane + k]);
-            hrow[k] = h;
+        for (int i = 0; i < PK_CH; ++i) {
+            const int j = j0 + 32 * i + lane;
+            v[i] = j < j1 ? __ldcg(pp + j) : make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(0x7fffffff));
+        }
+        // meanwhile: the row's operand, the sum of its planes (the values the tensor
+        // cores multiplied), and the next chain row's context slot, x_L (Sec. 3.4)
+        if (topk > 1 || !greedy) {
+            const size_t plane = (size_t)a.npad * D.d;
+            const uint16_t *q = a.planes + (size_t)b * D.d;
+            for (int k = t; k < D.d; k += PK_THREADS) {
+                float h = 0.f;
+#pragma unroll
+                for (int i = 0; i < TC_PLANES; ++i)
+                    if (i < a.npl) h += bf_to_f(q[i * plane + k]);
+                hrow[k] = h;
+            }
+        }
+        if (a.step + 1 < a.K) {
+            const int src = a.src_is_ext ? b * a.max_new + a.nnew[b] - 1 : b;
+            const float *xl = a.x_in + (size_t)src * D.d;
+            const size_t ld = 2 * (size_t)D.d, plane = (size_t)a.qkv_npad * ld;
+            for (int k = t; k < D.d; k += PK_THREADS) {
+                const float x = xl[k];
+                a.s_chain[(size_t)b * D.d + k] = x;
+                if (a.qkv_planes) {
+                    uint16_t q[TC_PLANES];
+                    tc_split(x, q);
+#pragma unroll
+                    for (int i = 0; i < TC_PLANES; ++i) a.qkv_planes[(size_t)b * ld + i * plane + k] = q[i];
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < PK_CH; ++i) {
+            px[i] = v[i].x;
+            py[i] = v[i].y;
+            m = fmaxf(m, v[i].x);
+            am = am_combine(am, AM{v[i].z, __float_as_int(v[i].w)});
         }
     }
+    for (int i = PK_CH; i < nch; ++i) {
+        const int j = j0 + 32 * i + lane;
+        if (j >= j1) break;
+        const float4 p = __ldcg(pp + j);
+        m = fmaxf(m, p.x);
+        am = am_combine(am, AM{p.z, __float_as_int(p.w)});
+    }
+    m = warp_max(m);
+    if (greedy) am = warp_am(am);
+    if (lane == 0) {
+        sm_m[warp] = m;
+        sm_am[0][warp] = am;
+    }
+    __syncthreads();
+    const float M = warp_max(sm_m[lane]);
+    auto weight = [&](float x, float y) { return x == -INFINITY ? 0.f : y * __expf(x - M); };
+    // partial i of the lane: its weight (and for i >= PK_CH its place again from memory)
+    float mine = 0.f;
+#pragma unroll
+    for (int i = 0; i < PK_CH; ++i) {
+        py[i] = weight(px[i], py[i]);
+        mine += py[i];
+    }
+    auto far = [&](int i) {
+        const int j = j0 + 32 * i + lane;
+        const float4 p = j < j1 ? __ldcg(pp + j) : make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        return make_float2(p.x, weight(p.x, p.y));
+    };
+    for (int i = PK_CH; i < nch; ++i) mine += far(i).y;
+    mine = warp_sum(mine);
+    if (lane == 0) sm_w[warp] = mine;
+    __syncthreads();
+    const float wtot = sm_w[lane], wincl = warp_incl_scan(wtot);   // lane k: warp k's range
+    const float S = __shfl_sync(0xffffffffu, wincl, 31);
     if (greedy) {
-        const AM top = block_am(am, sm_am);   // candidate 0: the argmax of the tensor-core logits
+        const AM top = warp_am(sm_am[0][lane]);   // candidate 0: the argmax of the tensor-core logits
         if (t == 0) { s_tok[0] = top.i; s_e[0] = 1.f; }
         if (topk > 1) {
             // the topk groups of largest maximum, one block argmax per round
-            for (int r = 0; r < topk; ++r) {
+            int taken[PK_MAXK];
+#pragma unroll
+            for (int r = 0; r < PK_MAXK; ++r) {
+                if (r >= topk) break;
                 AM loc{-INFINITY, 0x7fffffff};
-                for (int j = j0; j < j1; ++j) {
-                    bool taken = false;
-                    for (int rr = 0; rr < r; ++rr) taken |= s_grp[rr] == j;
-                    const float4 p = __ldcg(pp + j);
-                    if (!taken) loc = am_combine(loc, AM{p.z, j});
-                }
-                const AM g = block_am(loc, sm_am);
-                if (t == 0) s_grp[r] = g.v == -INFINITY ? -1 : g.i;
+                auto offer = [&](float x, int j) {
+                    bool was = j >= j1;
+#pragma unroll
+                    for (int rr = 0; rr < r; ++rr) was |= taken[rr] == j;
+                    if (!was) loc = am_combine(loc, AM{x, j});
+                };
+#pragma unroll
+                for (int i = 0; i < PK_CH; ++i) offer(px[i], j0 + 32 * i + lane);
+                for (int i = PK_CH; i < nch; ++i) offer(far(i).x, j0 + 32 * i + lane);
+                loc = warp_am(loc);
+                AM *slot = sm_am[(r + 1) & 1];   // in turn: one barrier a round
+                if (lane == 0) slot[warp] = loc;
                 __syncthreads();
+                const AM g = warp_am(slot[lane]);
+                taken[r] = g.v == -INFINITY ? -1 : g.i;
+                if (t == 0) s_grp[r] = taken[r];
             }
             __syncthreads();
-            for (int r = 0; r < topk; ++r)
-                if (s_grp[r] >= 0) pk_group_logits(a, hrow, s_grp[r], s_z + r * TC_LM_GROUP);
-                else if (t < TC_LM_GROUP) s_z[r * TC_LM_GROUP + t] = -INFINITY;
+            pk_group_logits(a, hrow, s_grp, topk, s_z);
             __syncthreads();
             // rank: candidates 1.. are the largest recomputed logits other than candidate 0
-            for (int c = 1; c < topk; ++c) {
-                AM loc{-INFINITY, 0x7fffffff};
-                if (t < topk * TC_LM_GROUP) {
-                    const int r = t / TC_LM_GROUP, l = t - r * TC_LM_GROUP;
-                    const int id = s_grp[r] < 0 ? -1 : s_grp[r] * TC_LM_GROUP + l;
-                    bool taken = id < 0;
-                    for (int cc = 0; cc < c; ++cc) taken |= s_tok[cc] == id;
-                    if (!taken) loc = AM{s_z[t], id};
+            if (warp == 0) {
+                float z[PK_MAXK];
+#pragma unroll
+                for (int r = 0; r < PK_MAXK; ++r) z[r] = r < topk ? s_z[r * TC_LM_GROUP + lane] : -INFINITY;
+                int last = top.i;
+                for (int c = 1; c < topk; ++c) {
+                    AM loc{-INFINITY, 0x7fffffff};
+#pragma unroll
+                    for (int r = 0; r < PK_MAXK; ++r) {
+                        const int id = r < topk && s_grp[r] >= 0 ? s_grp[r] * TC_LM_GROUP + lane : -1;
+                        if (id < 0 || id == last) z[r] = -INFINITY;   // taken
+                        else loc = am_combine(loc, AM{z[r], id});
+                    }
+                    const AM best = warp_am(loc);
+                    // no finite logit left: candidate 0 again
+                    last = best.v == -INFINITY ? -1 : best.i;
+                    if (lane == 0) { s_tok[c] = best.v == -INFINITY ? top.i : best.i; s_e[c] = 1.f; }
                 }
-                const AM best = block_am(loc, sm_am);
-                if (t == 0) { s_tok[c] = best.i == 0x7fffffff ? s_tok[0] : best.i; s_e[c] = 1.f; }
-                __syncthreads();
             }
         }
         __syncthreads();
     } else {
-        // each draw: its group from the partials, then its id inside the recomputed group
-        float tot;
-        const float ex = block_excl_scan(w, sh, &tot);
+        // each draw: its warp and group from the partials, then its id inside the recomputed group
         for (int c = 0; c < topk; ++c) {
             const float target = a.u_draft[((size_t)b * a.K + a.step) * topk + c] * S;
-            if (t == 0) { si[0] = 0x7fffffff; si[1] = -1; }
-            __syncthreads();
-            if (w > 0.f && target < ex + w) atomicMin(&si[0], t);
-            if (w > 0.f) atomicMax(&si[1], t);
-            __syncthreads();
-            const int ct = si[0] != 0x7fffffff ? si[0] : (si[1] >= 0 ? si[1] : 0);
-            if (t == ct) {   // this thread's run holds the point: find its group
-                float cum = ex;
-                int grp = -1, lastg = -1;
-                float lastb = ex;
-                for (int j = j0; j < j1; ++j) {
-                    const float4 p = __ldcg(pp + j);
-                    const float wj = p.x != -INFINITY ? p.y * __expf(p.x - M) : 0.f;
-                    if (wj > 0.f) { lastg = j; lastb = cum; }
-                    if (wj > 0.f && target < cum + wj) { grp = j; break; }
-                    cum += wj;
+            const unsigned hits = __ballot_sync(0xffffffffu, wtot > 0.f && target < wincl);
+            const unsigned some = __ballot_sync(0xffffffffu, wtot > 0.f);
+            const int ct = hits ? __ffs(hits) - 1 : (some ? 31 - __clz(some) : 0);
+            const float before = __shfl_sync(0xffffffffu, wincl - wtot, ct);
+            if (warp == ct) {   // this warp's range holds the point: find its group
+                float run = before, bef = before;
+                int grp = -1, lastg = j0;
+                float lastb = before;
+                auto walk = [&](int i, float w) {   // warp-uniform but for w
+                    const float incl = warp_incl_scan(w);
+                    const unsigned h = __ballot_sync(0xffffffffu, w > 0.f && target < run + incl);
+                    const unsigned pos = __ballot_sync(0xffffffffu, w > 0.f);
+                    if (h) {
+                        const int l = __ffs(h) - 1;
+                        grp = j0 + 32 * i + l;
+                        bef = run + __shfl_sync(0xffffffffu, incl - w, l);
+                    } else if (pos) {
+                        const int l = 31 - __clz(pos);
+                        lastg = j0 + 32 * i + l;
+                        lastb = run + __shfl_sync(0xffffffffu, incl - w, l);
+                    }
+                    run += __shfl_sync(0xffffffffu, incl, 31);
+                };
+#pragma unroll
+                for (int i = 0; i < PK_CH; ++i)
+                    if (grp < 0) walk(i, py[i]);
+                for (int i = PK_CH; i < nch && grp < 0; ++i) walk(i, far(i).y);
+                if (lane == 0) {
+                    s_grp[c] = grp >= 0 ? grp : lastg;
+                    s_before = grp >= 0 ? bef : lastb;
                 }
-                s_grp[c] = grp >= 0 ? grp : (lastg >= 0 ? lastg : j0);
-                s_before = grp >= 0 ? cum : lastb;
             }
             __syncthreads();
-            pk_group_logits(a, hrow, s_grp[c], s_z);
+            pk_group_logits(a, hrow, s_grp + c, 1, s_z);
             __syncthreads();
             if (warp == 0) {
                 const int id = s_grp[c] * TC_LM_GROUP + lane;
@@ -994,37 +1085,24 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
     }
     const int token = s_tok[0];
     if (a.step + 1 < a.K) {
-        // next chain row: context slot <- x_L (Sec. 3.4), residual <- E[candidate 0]
-        const int src = a.src_is_ext ? b * a.max_new + a.nnew[b] - 1 : b;
-        const float *xl = a.x_in + (size_t)src * D.d;
+        // next chain row: residual <- E[candidate 0] (its context slot was written above;
+        // x_in may be x_chain, and every thread overwrites only what it has read)
         const uint16_t *er = a.embed + (size_t)token * D.d;
         float ss = 0.f;
         for (int k = t; k < D.d; k += PK_THREADS) {
             const float e = bf_to_f(er[k]);
-            a.s_chain[(size_t)b * D.d + k] = xl[k];
             a.x_chain[(size_t)b * D.d + k] = e;
             ss = fmaf(e, e, ss);
         }
-        if (a.qkv_planes) {   // and its first layer's operand, [s; RMSNorm(x)]
+        if (a.qkv_planes) {   // and its first layer's operand's second half, RMSNorm(x)
             ss = warp_sum(ss);
             if (lane == 0) sh[warp] = ss;
             __syncthreads();
-            if (t == 0) {
-                float tot = 0.f;
-                for (int w = 0; w < PK_THREADS / 32; ++w) tot += sh[w];
-                sh[33] = rsqrtf(tot / (float)D.d + a.eps);
-            }
-            __syncthreads();
-            const float inv = sh[33];
+            const float inv = rsqrtf(warp_sum(sh[lane]) / (float)D.d + a.eps);
             const size_t ld = 2 * (size_t)D.d, plane = (size_t)a.qkv_npad * ld;
             uint16_t *p0 = a.qkv_planes + (size_t)b * ld;
             for (int k = t; k < D.d; k += PK_THREADS) {
-                // the s half from this thread's own copy in s_chain: x_in may be x_chain,
-                // whose row b now holds the embedding
                 uint16_t q[TC_PLANES];
-                tc_split(a.s_chain[(size_t)b * D.d + k], q);
-#pragma unroll
-                for (int i = 0; i < TC_PLANES; ++i) p0[i * plane + k] = q[i];
                 tc_split(bf_to_f(er[k]) * inv * bf_to_f(a.qkv_gain[k]), q);
 #pragma unroll
                 for (int i = 0; i < TC_PLANES; ++i) p0[i * plane + D.d + k] = q[i];
