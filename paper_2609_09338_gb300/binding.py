@@ -125,8 +125,11 @@ def _check(code: int):
         raise OspreyError(code, osprey_last_error())
 
 
+# A small call is bound by this module (its kernels take a few microseconds), so
+# the helpers below make no objects that the call does not need: addresses go to
+# ctypes as integers, and the stream's handle is read without a Stream around it.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _need(t, dtype, shape=None, name="tensor", device=True):
@@ -138,15 +141,15 @@ def _need(t, dtype, shape=None, name="tensor", device=True):
         raise ValueError(f"{name} must be a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:   # both tuples
         raise ValueError(f"{name}: shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t
 
 
 def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 # ---------------------------------------------------------------------------- context
@@ -173,7 +176,7 @@ class Ctx:
         for name, shp in shapes.items():
             arr = getattr(w, name)
             for l in range(shape.n_layers):
-                arr[l] = _ptr(_need(weights[name][l], bf, shp, f"{name}[{l}]")).value
+                arr[l] = _ptr(_need(weights[name][l], bf, shp, f"{name}[{l}]"))
         self._cfg, self._w = cfg, w
         h = _vp()
         _check(_c_create(ctypes.byref(cfg), ctypes.byref(w), ctypes.byref(h)))
