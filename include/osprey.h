@@ -109,7 +109,7 @@ const char *osprey_last_error(void);
 /* Validate the shape and weight pointers and make a context (host memory only).
  * The context picks the kernels a draft call uses:
  *   rows <= 2 per chain step: TMA-streamed GEMVs (weights read once per step);
- *   3..4096 rows: tcgen05 tensor-core GEMMs in tiles of up to 80 rows, float32
+ *   3..4096 rows: tcgen05 tensor-core GEMMs in tiles of up to 128 rows, float32
  *     activations split into three bf16 planes (24 mantissa bits) so results
  *     match the GEMV path's (the LM head's operand of up to 80 sequences into
  *     two planes, 16 bits: its logits differ from the GEMV path's by rounding

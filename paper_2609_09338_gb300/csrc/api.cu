@@ -1,4 +1,5 @@
 // C ABI: argument validation, workspace layout and launch sequencing.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdlib>
@@ -263,21 +264,22 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     // tensor-core path: bf16 operand planes, QKV output, row-sampler partials
     // (a step of more than TC_MAX_ROWS rows runs on the CUDA cores and needs none)
     const long long re = R_ext <= TC_MAX_ROWS ? R_ext : 0, rc = B <= TC_MAX_ROWS ? B : 0;
-    const long long np = std::max(tc_tiles(re).rows(), tc_tiles(rc).rows());
+    auto plane_rows = [](long long r) { return std::max(tc_tiles(r, 1).rows(), tc_tiles(r, TC_BIG_K).rows()); };
+    const long long np = std::max(plane_rows(re), plane_rows(rc));
+    const long long npl = std::max({np, (long long)tc_tiles_lm(re).rows(), (long long)tc_tiles_lm(rc).rows()});
     const long long nqkv = (long long)(D.Hq + 2 * D.Hkv) * D.hd;
     const bool tcw = ctx->tc;
     size_t o_xq = take(tcw ? 2ull * TC_PLANES * np * 2 * D.d : 0), o_yq = take(tcw ? 4ull * np * nqkv : 0);
     size_t o_xo = take(tcw ? 2ull * TC_PLANES * np * D.Hq * D.hd : 0), o_xg = take(tcw ? 2ull * TC_PLANES * np * D.d : 0);
-    size_t o_xh = take(tcw ? 2ull * TC_PLANES * np * D.F : 0), o_xl = take(tcw ? 2ull * TC_PLANES * np * D.d : 0);
+    size_t o_xh = take(tcw ? 2ull * TC_PLANES * np * D.F : 0), o_xl = take(tcw ? 2ull * TC_PLANES * npl * D.d : 0);
     const long long lm_nsub = (D.V + TC_LM_GROUP - 1) / TC_LM_GROUP;
     size_t o_rp = take(tcw && R_lm <= TC_MAX_ROWS ? 16ull * R_lm * lm_nsub : 0);
     // split-K partials: the largest nsplit x rows x outputs of the call's projections
     long long part = 0;
     if (tcw) {
         for (const long long rows : {re, rc}) {
-            const int nrt = tc_tiles(rows).nrt;
             auto need = [&](int nout, int K_, bool always = false) {
-                const int ns = tc_nsplit(nout, K_, nrt, ctx->sms);
+                const int ns = tc_nsplit(nout, K_, tc_tiles(rows, K_), ctx->sms);
                 if (ns > 1 || always) part = std::max(part, (long long)ns * rows * nout);
             };
             need(D.d, D.feat);
@@ -437,7 +439,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     for (int i = 0; i < D.hd / 2; ++i) g.inv_freq[i] = ctx->inv_freq[i];
     // tensor-core path for 3..TC_MAX_ROWS activation rows
     auto tc_rows = [&](int rows) { return ctx->tc && rows >= 3 && rows <= TC_MAX_ROWS; };
-    auto npad_of = [](int rows) { return tc_tiles(rows).rows(); };   // rows of an operand plane
+    auto npad_of = [](int rows, int K_) { return tc_tiles(rows, K_).rows(); };   // rows of an operand plane
+    auto npad_lm = [](int rows) { return tc_tiles_lm(rows).rows(); };   // ... of the LM head's
     // the LM head's operand planes: three for batches beyond one tile of rows
     const int lm_npl = block || B <= TC_TILE_ROWS ? TC_LM_PLANES : TC_PLANES;
     // the next GEMM's operand planes, written by a residual GEMM's reduction when it has one
@@ -450,7 +453,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
                        const void *xbuf, bool in_place_rows, float *y, int ldy, uint16_t *h,
                        const char *what, const CUtensorMap *wb = nullptr, const NextPlanes *nxt = nullptr,
                        bool *nxt_done = nullptr, const QkvPostArgs *rope = nullptr) -> int {
-        const TcTiles tt = tc_tiles(rows);
+        const TcTiles tt = tc_tiles(rows, K_);
         CUtensorMap xm;
         const bool ok = in_place_rows ? tc_encode_rows(&xm, xbuf, rows, tt.npad, K_)
                                       : tc_encode_operand(&xm, xbuf, planes, tt, K_);
@@ -460,7 +463,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         ta.R = rows;
         ta.npad = tt.npad;
         ta.nrt = tt.nrt;
-        ta.fine = tt.nrt > 1 && !block;
+        ta.bps = tt.bps;
+        ta.fine = rows > TC_TILE_ROWS && !block;
         ta.K = K_;
         ta.nout = nout;
         ta.planes = planes;
@@ -468,6 +472,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         ta.x = y;
         ta.ldy = ldy;
         ta.h = h;
+        ta.h_rows = h ? npad_of(rows, D.F) : 0;
         ta.status = dev_status;
         ta.part = ws.tc_part;
         ta.part_cap = ws.tc_part_cap;
@@ -493,7 +498,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     // sampling partials in its epilogue (logits stored only into z, when given),
     // then one pick block per row
     auto tc_lm = [&](int rows, float *z, long long ldz, const LmPickArgs &pick_in) -> int {
-        const TcTiles tt = tc_tiles(rows);
+        const TcTiles tt = tc_tiles_lm(rows);
         CUtensorMap xm;
         if (!tc_encode_operand(&xm, ws.tc_xl, lm_npl, tt, D.d))
             return fail(OSPREY_ERR_INVALID_ARG, "lm head: tensor map encoding failed");
@@ -502,7 +507,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         ta.R = rows;
         ta.npad = tt.npad;
         ta.nrt = tt.nrt;
-        ta.fine = tt.nrt > 1 && !block;
+        ta.bps = tt.bps;
+        ta.fine = rows > TC_TILE_ROWS && !block;
         ta.K = D.d;
         ta.nout = D.V;
         ta.planes = lm_npl;
@@ -530,7 +536,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     };
     auto planes = [&](const float *src, const uint16_t *gain, int d_, int rows, int ld, int col0, uint16_t *dst,
                       int rows_per_seq, bool last_of_seq, const char *what, int npl = TC_PLANES,
-                      const float *src2 = nullptr, int col2 = 0) -> int {
+                      const float *src2 = nullptr, int col2 = 0, bool lm = false) -> int {
         PlaneArgs pl{};
         pl.npl = npl;
         pl.src2 = src2;
@@ -540,7 +546,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         pl.eps = D.eps;
         pl.d = d_;
         pl.R = rows;
-        pl.npad = npad_of(rows);
+        pl.npad = lm ? npad_lm(rows) : npad_of(rows, ld);
         pl.ld = ld;
         pl.col0 = col0;
         pl.dst = dst;
@@ -684,7 +690,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             at.part = ws.attn_part;
             at.out = ws.attn_out;
             at.out_planes = ws.tc_xo;   // the O projection's operand, written by attention itself
-            at.npad = npad_of(R);
+            at.npad = npad_of(R, D.Hq * D.hd);
             at.ticket = ws.attn_ticket;
             at.status = dev_status;
             if ((e = attn_probe(step * D.L + l, true)) != cudaSuccess) return cuda_fail(e, "probe record");
@@ -693,7 +699,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             // x += W_o attn;  x += W_down (silu(W_g n) * W_u n),  n = RMSNorm(x)
             const int ha = D.Hq * D.hd;
             const NextPlanes ffn{ws.tc_xg, (const uint16_t *)W.ffn_norm[l], D.d, 0, TC_PLANES, 0, rows_per_seq,
-                                 npad_of(R)};
+                                 npad_of(R, D.d)};
             bool ffn_ready = false;
             if ((rc = tc_gemm(TC_RESID, R, ha, D.d, TC_PLANES, ctx->tm_o[l], ws.tc_xo, false, x, D.d, nullptr,
                               "o-proj launch", nullptr, &ffn, &ffn_ready)) != OSPREY_OK ||
@@ -708,12 +714,12 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             const NextPlanes *nxtp = nullptr;
             if (l + 1 < D.L) {
                 nxt = NextPlanes{ws.tc_xq, (const uint16_t *)W.attn_norm[l + 1], 2 * D.d, D.d, TC_PLANES, 0,
-                                 rows_per_seq, npad_of(R)};
+                                 rows_per_seq, npad_of(R, 2 * D.d)};
                 nxtp = &nxt;
             } else if (lm_tc) {
                 const bool last_rows = ext && !block;   // one LM row per sequence: its last new row
                 nxt = NextPlanes{ws.tc_xl, (const uint16_t *)W.final_norm, D.d, 0, lm_npl, last_rows ? 1 : 0,
-                                 rows_per_seq, npad_of(last_rows ? B : R)};
+                                 rows_per_seq, npad_lm(last_rows ? B : R)};
                 nxtp = &nxt;
             }
             bool nxt_ready = false;
@@ -827,7 +833,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             const int rows = B * max_new;
             int rc;
             if (!xl_ready && (rc = planes(x, (const uint16_t *)W.final_norm, D.d, rows, D.d, 0, ws.tc_xl, max_new, false,
-                                          "lm operand", lm_npl)) != OSPREY_OK)
+                                          "lm operand", lm_npl, nullptr, 0, true)) != OSPREY_OK)
                 return rc;
             LmPickArgs pk{};
             pk.B = rows;
@@ -868,7 +874,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             // (topk candidates per row when drafting a tree)
             int rc;
             if (!xl_ready && (rc = planes(x, (const uint16_t *)W.final_norm, D.d, B, D.d, 0, ws.tc_xl, 1, ext,
-                                          "lm operand", lm_npl)) != OSPREY_OK)
+                                          "lm operand", lm_npl, nullptr, 0, true)) != OSPREY_OK)
                 return rc;
             LmPickArgs pk{};
             pk.B = B;
@@ -889,7 +895,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
                 pk.qkv_planes = ws.tc_xq;
                 pk.qkv_gain = (const uint16_t *)W.attn_norm[0];
                 pk.eps = D.eps;
-                pk.qkv_npad = npad_of(B);
+                pk.qkv_npad = npad_of(B, 2 * D.d);
                 xq_next = true;
             }
             if ((rc = tc_lm(B, draft_logits ? draft_logits + (size_t)step * D.V : nullptr, (long long)K * D.V, pk)) !=

@@ -32,7 +32,7 @@ struct DraftWs {
     float4 *lm_stats;                      // [B][lm_warps]
     float2 *lm_sup;                        // [B][blocks][nsup] run statistics of the streamed LM head
     float4 *lm_cta_stats;                  // [B][sms]
-    // tensor-core path (rows padded to np <= 80): bf16 operand planes [TC_PLANES][np][...]
+    // tensor-core path (np: the rows of a plane, TcTiles::rows): bf16 operand planes [TC_PLANES][np][...]
     uint16_t *tc_xq;                       // [P][np][2d]    [s; RMSNorm(x)] for QKV
     float *tc_yq;                          // [np][(Hq+2Hkv)hd] QKV output before RoPE
     uint16_t *tc_xo;                       // [P][np][Hq*hd] attention output

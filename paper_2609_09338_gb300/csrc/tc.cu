@@ -2,17 +2,20 @@
 // the projections of Sec. 3.3 (Eq. 1-3, MLP, LM head), operand preparation,
 // RoPE + paged K/V write, and per-row sampling of the draft token (Sec. 3.1).
 //
-// tc_kernel: persistent, two CTAs per SM, 6 warps.
+// tc_kernel: persistent, two CTAs per SM (one for large calls), 6 warps.
 //   warp 0     issues 2-D TMA copies of one 128-row weight tile and the
 //              activation planes per 64-wide k-block into
 //              an nst-slot shared-memory ring (128-byte swizzle);
 //   warp 1     issues tcgen05.mma (M 128, N npad, K 16, bf16 in, float32
 //              accumulate in TMEM) per k-block and plane, then commits the
-//              k-block to the slot's "empty" barrier and the tile to the
-//              accumulator's "full" barrier;
+//              k-block to the slot's "empty" barrier and each accumulation
+//              segment to its accumulator's "full" barrier;
 //   warps 2-5  read the accumulator (tcgen05.ld, TMEM lane group = warp % 4)
-//              and run the epilogue while the next tile accumulates into the
-//              other TMEM buffer.
+//              and run the epilogue while the next segment accumulates into
+//              the other TMEM buffer.
+// What bounds it: in the decode shapes the weights' way from HBM (the LM head of 64
+// rows, 410 MB: 77 us, 5.3 TB/s); with more rows shared memory, from which an MMA
+// reads its weights (measured 44 cycles an MMA of 64 rows), and the ring's depth.
 // Every wait is bounded; on expiry the CTA records OSPREY_ERR_TIMEOUT, stops
 // issuing, lets its copies and MMAs land and frees its TMEM.
 #include <cooperative_groups.h>
@@ -28,19 +31,20 @@ namespace osp {
 
 namespace cg = cooperative_groups;
 
-#ifndef OSP_TC_CTAS_PER_SM
-#define OSP_TC_CTAS_PER_SM 2   // two CTAs per SM: two TMA producers and two MMA chains per SM
-#endif
 constexpr int TC_THREADS = 192;
 constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
 constexpr int TC_MAXST = 8;
-constexpr int TC_TMEM_COLS = 512 / OSP_TC_CTAS_PER_SM;   // of one CTA
 constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
 constexpr long long TC_SHARE_BYTES = 40ll << 20;   // weights above which they do
-// two CTAs, the system's share and the static part fit 228 KB.  100 KB left the
-// third stage of 48 rows and the fifth of 16 out: 96 sequences 2945 us a call,
-// 16 sequences 1992; with it 2904 and 1970
-constexpr size_t TC_SMEM_CAP = (OSP_TC_CTAS_PER_SM == 1 ? 200 : 112) * 1024;
+// Two CTAs per SM are two TMA producers, MMA chains and epilogues; one has all of
+// TMEM and shared memory, and tiles of up to TC_BIG_ROWS rows (tc_tiles).  An MMA reads its 4 KB of weights from shared memory however
+// many rows it multiplies (32 cycles; 16 rows more take 4), so 128 rows at once
+// cost two thirds of twice 64.
+// Two CTAs, the system's share and the static part fit 228 KB: 100 KB left the
+// third stage of 48 rows and the fifth of 16 out (16 sequences, 2 layers of d
+// 2048: 1992 us a call, with it 1970).
+__host__ __device__ constexpr size_t tc_smem_cap(int bps) { return (size_t)(bps == 1 ? 225 : 112) * 1024; }
+__host__ __device__ constexpr uint32_t tc_tmem_cols(int bps) { return 512 / bps; }   // of one CTA
 #ifndef OSP_TC_SEGKB
 #define OSP_TC_SEGKB 8   // k-blocks (64 wide) per accumulation segment
 #endif
@@ -177,8 +181,9 @@ __device__ __forceinline__ float lm_ex2(float x) {
 // CS > 1 (several row tiles): the CTAs of a cluster of CS take adjacent row tiles
 // of the same features and k-range, and each weight tile is loaded once, by the
 // CTAs in turn, and multicast.  A slot is free when every CTA's MMAs have read it.
-template <int EPI, int NA, int CS>
-__global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
+// BPS: CTAs per SM.
+template <int EPI, int NA, int CS, int BPS>
+__global__ void __launch_bounds__(TC_THREADS, BPS)
     tc_kernel(const __grid_constant__ CUtensorMap wa, const __grid_constant__ CUtensorMap wb,
               const __grid_constant__ CUtensorMap xm, const TcArgs a, int nst) {
     extern __shared__ uint8_t raw[];
@@ -211,7 +216,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
     const bool sep = NA == 1 && a.sep;
     // an item of several segments is finished from columns of its own where they
     // fit (tiles of up to 64 rows), so that its last segment's buffer is free at once
-    const bool own = NA == 1 && a.kbps > a.segkb && 4 * acc_cols <= TC_TMEM_COLS;
+    const bool own = NA == 1 && a.kbps > a.segkb && 4 * acc_cols <= tc_tmem_cols(BPS);
     uint32_t ncols = 32;
     while (ncols < (own ? 4 : sep ? 3 : 2) * acc_cols) ncols <<= 1;
 
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
                 // (a loop over chunks in TMEM: unrolled over registers, its code is five
                 // times as long, which cost each short launch 5 us of instruction fetches)
                 if (nseg > 1) {
-                    constexpr int NCH = TC_TILE_ROWS / 16;
+                    constexpr int NCH = (BPS == 1 ? TC_BIG_ROWS : TC_TILE_ROWS) / 16;
                     const int nch = npad / 16;
                     float tot[NCH][16];
                     auto add = [&](uint32_t t0) {   // two chunks' loads in flight at a time
@@ -569,7 +574,7 @@ __global__ void __launch_bounds__(TC_THREADS, OSP_TC_CTAS_PER_SM)
 // ---------------------------------------------------------------- split-K reduction
 // out[n][col] = sum over the k-ranges (in order) of the partials, then the
 // GEMM's epilogue.  TC_GLU: gate = output col, up = output nout_a + col, and
-// the planes of h = silu(gate) * up go to h [TC_PLANES][nrt npad][nout_a].
+// the planes of h = silu(gate) * up go to h [TC_PLANES][h_rows][nout_a].
 template <int EPI>
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const TcArgs a) {
     pdl_trigger();
@@ -591,7 +596,7 @@ __global__ void __launch_bounds__(256) tc_reduce_kernel(const TcArgs a) {
         uint16_t q[TC_PLANES];
         tc_split(h, q);
 #pragma unroll
-        for (int i = 0; i < TC_PLANES; ++i) a.h[((size_t)i * a.nrt * a.npad + n) * w + col] = q[i];
+        for (int i = 0; i < TC_PLANES; ++i) a.h[((size_t)i * a.h_rows + n) * w + col] = q[i];
     }
 }
 
@@ -1083,7 +1088,7 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
         a.stats[o * 2 + 0] = M;
         a.stats[o * 2 + 1] = logf(S);
     }
-    const int token = s_tok[0];
+    const int token = min(max(s_tok[0], 0), D.V - 1);   // a row of NaN has no argmax
     if (a.step + 1 < a.K) {
         // next chain row: residual <- E[candidate 0] (its context slot was written above;
         // x_in may be x_chain, and every thread overwrites only what it has read)
@@ -1181,32 +1186,39 @@ bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, const TcTiles 
     return encode2d(m, x, K, (uint64_t)planes * t.rows(), t.npad);
 }
 
-static int tc_stages(int npad, int planes, int na) {
+static int tc_stages(int npad, int planes, int na, int bps) {
     const size_t stage = (size_t)na * TC_ABYTES + (size_t)planes * npad * 128;
-    int n = (int)((TC_SMEM_CAP - 1024) / stage);
+    int n = (int)((tc_smem_cap(bps) - 1024) / stage);
     return n > TC_MAXST ? TC_MAXST : n;
 }
-size_t tc_smem_bytes(int npad, int planes, int na) {
+static size_t tc_smem_bytes(int npad, int planes, int na, int bps) {
     const size_t stage = (size_t)na * TC_ABYTES + (size_t)planes * npad * 128;
-    return (size_t)tc_stages(npad, planes, na) * stage + 1024;
+    return (size_t)tc_stages(npad, planes, na, bps) * stage + 1024;
 }
 
-template <int EPI, int NA, int CS>
+template <int EPI, int NA, int CS, int BPS>
 static cudaError_t tc_allow_smem() {
-    return cudaFuncSetAttribute(tc_kernel<EPI, NA, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM_CAP);
+    return cudaFuncSetAttribute(tc_kernel<EPI, NA, CS, BPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tc_smem_cap(BPS));
+}
+// an epilogue's kernels: small calls, large ones, large ones whose row tiles share weights
+template <int EPI>
+static cudaError_t tc_allow_smem_all() {
+    cudaError_t e = tc_allow_smem<EPI, 1, 1, 2>();
+    if (e == cudaSuccess) e = tc_allow_smem<EPI, 1, 1, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<EPI, 1, TC_CS, 1>();
+    if (e == cudaSuccess) e = tc_allow_smem<EPI, 1, TC_CS, 2>();
+    return e;
 }
 
 cudaError_t tc_set_attributes() {
-    cudaError_t e = tc_allow_smem<TC_STORE, 1, 1>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_STORE, 1, TC_CS>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_STORE, OSP_TC_LM_NA, 1>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_RESID, 1, 1>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_RESID, 1, TC_CS>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_GLU, 1, 1>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_GLU, 1, TC_CS>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, 1>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, TC_CS>();
-    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, OSP_TC_LM_NA, 1>();
+    cudaError_t e = tc_allow_smem_all<TC_STORE>();
+    if (e == cudaSuccess) e = tc_allow_smem_all<TC_RESID>();
+    if (e == cudaSuccess) e = tc_allow_smem_all<TC_GLU>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, 1, 2>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, 1, TC_CS, 2>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_STORE, OSP_TC_LM_NA, 1, 2>();
+    if (e == cudaSuccess) e = tc_allow_smem<TC_LM, OSP_TC_LM_NA, 1, 2>();
     if (e == cudaSuccess) e = allow_smem(lm_pick_kernel);
     return e;
 }
@@ -1228,10 +1240,10 @@ static cudaError_t pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t sme
     return e;
 }
 
-template <int EPI, int NA, int CS>
+template <int EPI, int NA, int CS, int BPS>
 static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtensorMap &wa, const CUtensorMap &wb,
                              const CUtensorMap &xm, const TcArgs &a, int nst) {
-    if (CS == 1) return pdl_launch(tc_kernel<EPI, NA, CS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
+    if (CS == 1) return pdl_launch(tc_kernel<EPI, NA, CS, BPS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(TC_THREADS);
@@ -1246,7 +1258,7 @@ static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtens
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_kernel<EPI, NA, CS>, wa, wb, xm, a, nst);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_kernel<EPI, NA, CS, BPS>, wa, wb, xm, a, nst);
     count_launch();
     return e;
 }
@@ -1256,11 +1268,11 @@ static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtens
 #ifndef OSP_TC_MIN_KB
 #define OSP_TC_MIN_KB 1   // k-blocks (of 64) per range at least: fewer, longer ranges write fewer partials
 #endif
-int tc_nsplit(int nout, int K, int nrt, int sms) {
-    const int tiles = (nout + 127) / 128 * nrt, nkb = K / 64;
+int tc_nsplit(int nout, int K, const TcTiles &t, int sms) {
+    const int tiles = (nout + 127) / 128 * t.nrt, nkb = K / 64;
     // at most one item per CTA slot: one item more than the slots would take two
     // item times for barely more than one wave of work
-    int want = OSP_TC_CTAS_PER_SM * sms / tiles;
+    int want = t.bps * sms / tiles;
     if (want < 1) want = 1;
     if (want > nkb / OSP_TC_MIN_KB) want = nkb / OSP_TC_MIN_KB > 1 ? nkb / OSP_TC_MIN_KB : 1;
     const int kbps = (nkb + want - 1) / want;
@@ -1278,64 +1290,58 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     TcArgs a = a_in;
     if (planes_done) *planes_done = false;
     if (a.nrt < 1) a.nrt = 1;
-    if (a.npad % 16 || a.npad < 16 || a.npad > TC_TILE_ROWS || a.K % 64 || a.R > (long long)a.nrt * a.npad)
+    if (a.bps != 1) a.bps = 2;
+    if (a.bps == 1 && a.epi == TC_LM) return cudaErrorInvalidValue;
+    if (a.npad % 16 || a.npad < 16 || a.npad > (a.bps == 1 ? TC_BIG_ROWS : TC_TILE_ROWS) || a.K % 64 || a.R > (long long)a.nrt * a.npad)
         return cudaErrorInvalidValue;
     if (a.nout_a < 1 || a.nout_a > a.nout || (a.nout_a < a.nout && a.nout_a % 128)) return cudaErrorInvalidValue;
-    if (a.epi == TC_GLU && (a.nout != 2 * a.nout_a || !a.part || !a.h)) return cudaErrorInvalidValue;
+    if (a.epi == TC_GLU && (a.nout != 2 * a.nout_a || !a.part || !a.h || a.h_rows < a.R)) return cudaErrorInvalidValue;
     const int nkb = a.K / 64;
     if (a.epi == TC_LM && (!a.lm_part || a.lm_nsub != (a.nout + TC_LM_GROUP - 1) / TC_LM_GROUP))
         return cudaErrorInvalidValue;
-    a.nsplit = a.part && a.epi != TC_LM ? tc_nsplit(a.nout, a.K, a.nrt, sms) : 1;   // the LM epilogue needs whole sums
+    a.nsplit = a.part && a.epi != TC_LM ? tc_nsplit(a.nout, a.K, TcTiles{a.nrt, a.npad, a.bps}, sms) : 1;   // the LM epilogue needs whole sums
     if ((long long)a.nsplit * a.R * a.nout > a.part_cap) a.nsplit = 1;
     if (a.epi == TC_GLU && (long long)a.nsplit * a.R * a.nout > a.part_cap) return cudaErrorInvalidValue;
     a.kbps = (nkb + a.nsplit - 1) / a.nsplit;
     a.sep = a.planes > 1;   // (0.1 % of a call, for a third of the accumulators' error)
     a.segkb = a.fine ? OSP_TC_SEGKB_FINE : OSP_TC_SEGKB;
-    constexpr int tmem_cols = TC_TMEM_COLS;
+    const int bps = a.bps, tmem_cols = tc_tmem_cols(bps);
     // the LM head takes OSP_TC_LM_NA weight tiles per stage when two stages fit
     // and the double-buffered accumulators fit TMEM in one segment (the LM head's
     // reduction over d is short: one segment keeps its MMA chain at 4 d / 64 steps
     // per plane)
     int na = 1;
     const bool wide = a.epi == TC_LM || (a.epi == TC_STORE && a.nsplit == 1 && a.wide);
-    if (wide && a.nrt == 1 && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA) >= 2 &&
+    if (wide && a.nrt == 1 && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA, bps) >= 2 &&
         2 * OSP_TC_LM_NA * a.npad <= tmem_cols && a.kbps <= 32 && a.planes <= TC_LM_PLANES) {
         na = OSP_TC_LM_NA;
         a.segkb = a.kbps;
     }
-    const int nst = tc_stages(a.npad, a.planes, na);
+    const int nst = tc_stages(a.npad, a.planes, na, bps);
     if (nst < 2) return cudaErrorInvalidValue;
     if ((na == 1 && a.sep ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
-    // several row tiles (an even number, tc_tiles) share weights that the L2 does not
-    // keep from one tile to the next: d 4096 (100..235 MB a projection, 1.2 GB of LM
-    // head) 2136 us a call without, 2027 with.  Projections of 4..33 MB gain nothing
-    // and pay the clusters' start (d 1024, 96 rows: 1 us of 12..18 a launch)
-    const int cs = a.nrt > 1 && (long long)a.nout * a.K * 2 > TC_SHARE_BYTES ? TC_CS : 1;
+    // pairs of row tiles share weights that the L2 does not keep from one tile to the
+    // next
+    const int cs = a.nrt % TC_CS == 0 && (long long)a.nout * a.K * 2 > TC_SHARE_BYTES ? TC_CS : 1;
     if (a.nrt % cs || (cs > 1 && na > 1)) return cudaErrorInvalidValue;
-    const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / cs) * a.nsplit, slots = OSP_TC_CTAS_PER_SM * sms / cs;
+    const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / cs) * a.nsplit, slots = bps * sms / cs;
     const int grid = (items < slots ? items : slots) * cs;
-    const size_t smem = tc_smem_bytes(a.npad, a.planes, na);
+    const size_t smem = tc_smem_bytes(a.npad, a.planes, na, bps);
     cudaError_t e;
+#define OSP_TC_GO(EPI, NA_, CS_, BPS_) tc_launch<EPI, NA_, CS_, BPS_>(grid, smem, s, wa, wb, xm, a, nst)
+#define OSP_TC_ROWS(EPI)                                                          \
+    (bps == 1 ? (cs > 1 ? OSP_TC_GO(EPI, 1, TC_CS, 1) : OSP_TC_GO(EPI, 1, 1, 1)) \
+              : (cs > 1 ? OSP_TC_GO(EPI, 1, TC_CS, 2) : OSP_TC_GO(EPI, 1, 1, 2)))
     switch (a.epi) {
-    case TC_STORE:
-        e = cs > 1   ? tc_launch<TC_STORE, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
-            : na > 1 ? tc_launch<TC_STORE, OSP_TC_LM_NA, 1>(grid, smem, s, wa, wb, xm, a, nst)
-                     : tc_launch<TC_STORE, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
-        break;
-    case TC_RESID:
-        e = cs > 1 ? tc_launch<TC_RESID, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
-                   : tc_launch<TC_RESID, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
-        break;
-    case TC_GLU:
-        e = cs > 1 ? tc_launch<TC_GLU, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
-                   : tc_launch<TC_GLU, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
-        break;
+    case TC_STORE: e = na > 1 ? OSP_TC_GO(TC_STORE, OSP_TC_LM_NA, 1, 2) : OSP_TC_ROWS(TC_STORE); break;
+    case TC_RESID: e = OSP_TC_ROWS(TC_RESID); break;
+    case TC_GLU: e = OSP_TC_ROWS(TC_GLU); break;
     default:
-        e = cs > 1   ? tc_launch<TC_LM, 1, TC_CS>(grid, smem, s, wa, wb, xm, a, nst)
-            : na > 1 ? tc_launch<TC_LM, OSP_TC_LM_NA, 1>(grid, smem, s, wa, wb, xm, a, nst)
-                     : tc_launch<TC_LM, 1, 1>(grid, smem, s, wa, wb, xm, a, nst);
+        e = na > 1 ? OSP_TC_GO(TC_LM, OSP_TC_LM_NA, 1, 2) : cs > 1 ? OSP_TC_GO(TC_LM, 1, TC_CS, 2) : OSP_TC_GO(TC_LM, 1, 1, 2);
         break;
     }
+#undef OSP_TC_ROWS
+#undef OSP_TC_GO
     if (e != cudaSuccess || (a.nsplit == 1 && a.epi != TC_GLU)) return e;
     if (a.epi == TC_RESID && a.pl_dst && a.nout <= RP_CS * 256 * RP_VPT) {
         cudaLaunchConfig_t cfg = {};

@@ -3,19 +3,22 @@
 // swap-AB GEMMs, Y[R x Nout] = X[R x K] . W[Nout x K]^T, for 3..4096 rows.
 //
 // Weights are the M = 128 operand, streamed tile by tile with 2-D TMA (128-byte
-// swizzle); the R activation rows are the N operand, in equal tiles of at most
-// 80 rows (padded to a multiple of 16).  Two row tiles at a time share each weight
-// tile: a cluster of two CTAs loads it once and multicasts it.  The LM head multiplies two weight tiles against each stage's operand
-// planes (twice the weight bytes in flight per byte of operand reloaded).  Activations are float32 between kernels; for the tensor cores each is
-// split into three bf16 planes, q0 = bf16(x), q1 = bf16(x - q0), q2 =
-// bf16(x - q0 - q1), and every k-step issues one MMA per plane into the same
-// float32 accumulator, so the product keeps the 24 mantissa bits of x (bf16
-// inputs such as the target features use a single plane).  Two planes (16
-// bits) were not enough: attention over thousands of cached keys turns a 1e-5
-// relative error in q into logit errors two orders above the float32 path's.  The reduction is accumulated in segments of
-// 512 (a fresh TMEM accumulator each) whose float32 sum the epilogue keeps, so
-// no accumulation chain in the tensor core is longer than 32 MMA steps per
-// plane (a long chain loses precision against a float32 tree sum).
+// swizzle); the R activation rows are the N operand, in equal tiles (tc_tiles).
+// Pairs of row tiles share weights that are read from HBM each time: a cluster of
+// two CTAs loads a tile once and multicasts it.  The LM head of one row tile
+// multiplies two weight tiles against each stage's operand planes (twice the
+// weight bytes in flight per byte of operand reloaded).
+//
+// Activations are float32 between kernels; for the tensor cores each is split into
+// three bf16 planes, q0 = bf16(x), q1 = bf16(x - q0), q2 = bf16(x - q0 - q1), one
+// MMA per plane and k-step, so the product keeps the 24 mantissa bits of x (bf16
+// inputs such as the target features use a single plane).  Two planes (16 bits)
+// were not enough: attention over thousands of cached keys turns a 1e-5 relative
+// error in q into logit errors two orders above the float32 path's.  A reduction
+// is accumulated in segments (a fresh TMEM accumulator each, of 8 k-blocks, or 2
+// where the rows were float32 dot products before) whose float32 sum the epilogue
+// keeps, and the planes after the first have an accumulator of their own: a
+// tensor-core accumulator truncates at every step.
 #pragma once
 
 #include <cuda.h>
@@ -42,30 +45,47 @@ constexpr int TC_LM_PLANES = 2;
 // planes would put q(token) 1e-4 off at logits of 40 (three: 1e-6).
 
 constexpr int TC_TILE_ROWS = 80;   // activation rows per tile: three accumulators fit a CTA's 256 TMEM columns
+constexpr int TC_BIG_ROWS = 128;   // rows per tile of a larger GEMM ...
+constexpr int TC_BIG_K = 4096;     // ... whose reduction is at least this long
 constexpr int TC_MAX_ROWS = 4096;  // rows of a call on the tensor cores (beyond: the CUDA-core GEMV, whose workspace is smaller)
 constexpr int TC_GROUP_ROWS = 512; // rows of one pass of block drafting
 constexpr int TC_PLANES = 3;       // bf16 planes of a float32 operand
 
-// A call's rows as equal tiles of at most TC_TILE_ROWS (the MMA's N, a multiple
-// of 16).  80 rows a tile keep two CTAs per SM (two accumulators of 80 columns
-// and a running total in 256 TMEM columns, two stages of three planes in 100 KB).
+// A GEMM's rows as equal tiles (the MMA's N, a multiple of 16).  Up to TC_TILE_ROWS
+// keep two CTAs per SM (two accumulators of 80 columns and one of the small planes
+// in 256 TMEM columns, two stages of three planes in 112 KB).  More rows: with a
+// reduction of TC_BIG_K or more, tiles of up to TC_BIG_ROWS and one CTA per SM
+// (four accumulators of 128 columns, three stages): 120 rows at d 4096, gate and up
+// 110 -> 88 us, the O and down projections 39 -> 34; with a shorter one, an even
+// number of the small tiles: start and epilogue weigh more there, and two CTAs
+// overlap them (96 rows, d 1024: 11.7 us a launch against 12.7).
 struct TcTiles {
     int nrt, npad;     // row tiles, rows per tile
+    int bps;           // CTAs per SM
     __host__ __device__ int rows() const { return nrt * npad; }   // rows of an operand plane
 };
-inline TcTiles tc_tiles(long long rows) {
+inline TcTiles tc_tiles_of(long long rows, int most, int even, int bps) {
     TcTiles t;
-    t.nrt = (int)((rows + TC_TILE_ROWS - 1) / TC_TILE_ROWS);
-    if (t.nrt < 1) t.nrt = 1;
-    if (t.nrt > 1) t.nrt += t.nrt & 1;   // pairs of tiles share the weights they load
+    t.nrt = rows <= most ? 1 : (int)((rows + most - 1) / most + even - 1) / even * even;
     t.npad = (int)(((rows + t.nrt - 1) / t.nrt + 15) / 16 * 16);
+    t.bps = bps;
     return t;
 }
+inline TcTiles tc_tiles(long long rows, int K) {
+    return rows > TC_TILE_ROWS && K >= TC_BIG_K ? tc_tiles_of(rows, TC_BIG_ROWS, 1, 1)
+                                                : tc_tiles_of(rows, TC_TILE_ROWS, 2, 2);
+}
+// The LM head keeps two CTAs per SM at any number of rows, whose epilogues (the
+// sampling partials are most of an item's time) run beside each other's MMAs:
+// 96 rows, V 151936, d 1024, in two tiles of 48 132 us, in one of 96 161.  An even
+// number of tiles: pairs share the weights that they load.
+inline TcTiles tc_tiles_lm(long long rows) { return tc_tiles_of(rows, TC_TILE_ROWS, 2, 2); }
 
 struct TcArgs {
     int epi;           // TcEpi
     int R;             // rows
     int npad, nrt;     // rows per tile (a multiple of 16), row tiles; an operand plane has nrt * npad rows
+    int bps;           // CTAs per SM
     int K;             // reduction length (multiple of 64)
     int nout;          // output features (tiles of 128, the last one may be partial)
     int nout_a;        // features [0, nout_a) from the first weight map, the rest from the second
@@ -74,7 +94,8 @@ struct TcArgs {
     float *y;          // TC_STORE: [R][ldy] float32 output
     int ldy;
     float *x;          // TC_RESID: [R][ldy] float32, +=
-    uint16_t *h;       // TC_GLU: [TC_PLANES][nrt npad][nout_a] bf16 planes of silu(gate) * up
+    uint16_t *h;       // TC_GLU: [TC_PLANES][h_rows][nout_a] bf16 planes of silu(gate) * up
+    int h_rows;        // plane rows of the GEMM that reads h
     int32_t *status;
     // TC_LM: partials [R][lm_nsub] (lm_nsub = ceil(nout / 32)), 1/T (1 for greedy)
     float4 *lm_part;
@@ -115,7 +136,7 @@ cudaError_t tc_set_attributes();
 // silu(gate) * up.  Outputs narrower than the CTA slots are split along K
 // (tc_nsplit ranges per 128-feature, npad-row tile); the float32 partials are then summed
 // in range order by a reduction kernel that applies the epilogue.
-int tc_nsplit(int nout, int K, int nrt, int sms);
+int tc_nsplit(int nout, int K, const TcTiles &t, int sms);
 cudaError_t launch_tc(const TcArgs &a, const CUtensorMap &wa, const CUtensorMap &xm, int sms, cudaStream_t s);
 // *planes_done (when given) tells whether the reduction did the follow-up work:
 // wrote the pl_* planes (TC_RESID), or RoPE and the K/V write of `rope`

@@ -1,8 +1,10 @@
-"""Draft calls of more than 80 rows: the tensor-core projections and the LM head run in tiles of up to 80 rows.
+"""Draft calls of more than 80 rows: the tensor-core projections and the LM head run in tiles of rows.
 
 Sizes at the edges of the tiling (one row past a tile, a last tile that is nearly empty, several tiles, ragged extend
 rows), against the oracle with the tolerances of the other draft tests.
 """
+from dataclasses import replace
+
 import numpy as np
 import pytest
 
@@ -21,6 +23,17 @@ def test_more_rows_than_a_tile(B, max_new, T):
     n_new = rng.integers(1, max_new + 1, size=B)
     pick = sorted({0, B // 2, B - 1, min(79, B - 1), min(80, B - 1)})
     check_case(run_case(TINY, ctx, 3, T, 50 + B, n_new=n_new, max_new=max_new, peaked=T > 0, sample_seqs=pick))
+
+
+@pytest.mark.parametrize("B,max_new", [(81, 1), (129, 1), (27, 8)])
+def test_long_reductions(B, max_new):
+    """Reductions of 4096 take the larger tiles (one CTA per SM), their neighbours of a layer the small ones: the operand
+    planes between them have either's rows."""
+    shape = replace(TINY, ffn_dim=4096, feat_dim=4096, n_layers=2)
+    rng = np.random.default_rng(B)
+    n_new = rng.integers(1, max_new + 1, size=B)
+    pick = sorted({0, B // 2, B - 1, min(80, B - 1)})
+    check_case(run_case(shape, rng.integers(0, 30, size=B), 2, 0.0, 30 + B, n_new=n_new, max_new=max_new, sample_seqs=pick))
 
 
 def test_block_rows_beyond_a_tile():
