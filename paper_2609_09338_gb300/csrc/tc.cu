@@ -691,7 +691,13 @@ __global__ void __launch_bounds__(256) tc_resid_planes_kernel(const TcArgs a) {
 }
 
 // ---------------------------------------------------------------- operand planes
-__global__ void __launch_bounds__(256) planes_kernel(const PlaneArgs a) {
+// A block a row, and few rows: what bounds these kernels is the latency of a
+// thread's chain of loads, so a row of d elements gets the width that leaves a
+// thread four to eight of them.  With 256 threads at every d, a block drafter's
+// call (d 4096, 120 rows) took 1902 us instead of 1884, a tree of 2048 wide
+// rows 1905 instead of 1900; below d 2048 the width is what it was.
+static int row_threads(int d) { return d >= 4096 ? 1024 : d >= 2048 ? 512 : 256; }
+__global__ void __launch_bounds__(1024) planes_kernel(const PlaneArgs a) {
     __shared__ float red[33];
     const int r = blockIdx.x;
     pdl_trigger();
@@ -1123,7 +1129,7 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
 }
 
 // ---------------------------------------------------------------- embedding rows
-__global__ void __launch_bounds__(256) embed_rows_kernel(const EmbedArgs a) {
+__global__ void __launch_bounds__(1024) embed_rows_kernel(const EmbedArgs a) {
     const int r = blockIdx.x, b = r / a.max_new, j = r - b * a.max_new;
     pdl_trigger();
     pdl_wait();
@@ -1384,7 +1390,7 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
 }
 
 cudaError_t launch_planes(const PlaneArgs &a, cudaStream_t s) {
-    return pdl_launch(planes_kernel, dim3(a.R), dim3(256), 0, s, a);
+    return pdl_launch(planes_kernel, dim3(a.R), dim3(row_threads(a.d)), 0, s, a);
 }
 
 cudaError_t launch_qkv_post(const QkvPostArgs &a, cudaStream_t s) {
@@ -1393,7 +1399,7 @@ cudaError_t launch_qkv_post(const QkvPostArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_embed_rows(const EmbedArgs &a, cudaStream_t s) {
-    return pdl_launch(embed_rows_kernel, dim3(a.R), dim3(256), 0, s, a);
+    return pdl_launch(embed_rows_kernel, dim3(a.R), dim3(row_threads(a.d)), 0, s, a);
 }
 
 cudaError_t launch_lm_pick(const LmPickArgs &a, cudaStream_t s) {

@@ -36,6 +36,15 @@ def test_long_reductions(B, max_new):
     check_case(run_case(shape, rng.integers(0, 30, size=B), 2, 0.0, 30 + B, n_new=n_new, max_new=max_new, sample_seqs=pick))
 
 
+@pytest.mark.parametrize("d", [1792, 2048, 2304, 3840, 4096])
+def test_wide_rows(d):
+    """The blocks that normalise and gather rows are wider from d 2048 and from d 4096: both sides of each edge, a last
+    pass that is partly filled, ragged extend rows."""
+    shape = replace(TINY, d_model=d)
+    n_new = np.array([1, 3, 2, 3])
+    check_case(run_case(shape, np.array([5, 0, 17, 30]), 2, 0.0, 90 + d, n_new=n_new, max_new=3))
+
+
 def test_block_rows_beyond_a_tile():
     """Ten blocks of 11 positions (100 rows, two row tiles in one group) give what each gives in a call of its own."""
     from paper_2609_09338_gb300.binding import to_device_bf16
