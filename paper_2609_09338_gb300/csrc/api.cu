@@ -279,7 +279,7 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     if (tcw) {
         for (const long long rows : {re, rc}) {
             auto need = [&](int nout, int K_, bool always = false) {
-                const int ns = tc_nsplit(nout, K_, tc_tiles(rows, K_), ctx->sms);
+                const int ns = tc_nsplit(nout, K_, block ? TC_BLOCK_SPLITS : tc_tiles(rows, K_), ctx->sms);
                 if (ns > 1 || always) part = std::max(part, (long long)ns * rows * nout);
             };
             need(D.d, D.feat);
@@ -376,6 +376,14 @@ extern "C" int osprey_kv_append(const osprey_ctx *ctx, const osprey_kv *kv, int 
 }
 
 // ------------------------------------------------------------------ draft step
+// Sequences of a block-drafting call whose P rows each fill one tile: a group
+// (consecutive sequences; the last one may be smaller) is summed in the same order
+// whatever is drafted beside it (TcArgs::block).
+static int block_group(int B, int P) {
+    const int g = TC_TILE_ROWS / P;
+    return g < 1 ? 1 : (g < B ? g : B);
+}
+
 // block: a block-drafting call (EAGLE-style DFlash): K = 1, every one of the
 // max_new extend rows of a sequence is sampled (row j's output proposes the
 // token at j + 1) into draft_* [B][max_new], and only the first row (the
@@ -441,6 +449,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     auto tc_rows = [&](int rows) { return ctx->tc && rows >= 3 && rows <= TC_MAX_ROWS; };
     auto npad_of = [](int rows, int K_) { return tc_tiles(rows, K_).rows(); };   // rows of an operand plane
     auto npad_lm = [](int rows) { return tc_tiles_lm(rows).rows(); };   // ... of the LM head's
+    // block drafting: sequences whose rows are summed in the order of one group (TcArgs::block)
+    const int grp = block ? block_group(B, max_new) : B;
     // the LM head's operand planes: three for batches beyond one tile of rows
     const int lm_npl = block || B <= TC_TILE_ROWS ? TC_LM_PLANES : TC_PLANES;
     // the next GEMM's operand planes, written by a residual GEMM's reduction when it has one
@@ -456,7 +466,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         const TcTiles tt = tc_tiles(rows, K_);
         CUtensorMap xm;
         const bool ok = in_place_rows ? tc_encode_rows(&xm, xbuf, rows, tt.npad, K_)
-                                      : tc_encode_operand(&xm, xbuf, planes, tt, K_);
+                                      : tc_encode_operand(&xm, xbuf, planes, tt.rows(), tt.npad, K_);
         if (!ok) return fail(OSPREY_ERR_INVALID_ARG, "%s: tensor map encoding failed", what);
         TcArgs ta{};
         ta.epi = epi;
@@ -464,6 +474,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         ta.npad = tt.npad;
         ta.nrt = tt.nrt;
         ta.bps = tt.bps;
+        ta.block = block;
         ta.fine = rows > TC_TILE_ROWS && !block;
         ta.K = K_;
         ta.nout = nout;
@@ -497,41 +508,59 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
     // the LM head of `rows` operand rows in ws.tc_xl on the tensor cores, with the
     // sampling partials in its epilogue (logits stored only into z, when given),
     // then one pick block per row
-    auto tc_lm = [&](int rows, float *z, long long ldz, const LmPickArgs &pick_in) -> int {
-        const TcTiles tt = tc_tiles_lm(rows);
-        CUtensorMap xm;
-        if (!tc_encode_operand(&xm, ws.tc_xl, lm_npl, tt, D.d))
-            return fail(OSPREY_ERR_INVALID_ARG, "lm head: tensor map encoding failed");
-        TcArgs ta{};
-        ta.epi = TC_LM;
-        ta.R = rows;
-        ta.npad = tt.npad;
-        ta.nrt = tt.nrt;
-        ta.bps = tt.bps;
-        ta.fine = rows > TC_TILE_ROWS && !block;
-        ta.K = D.d;
-        ta.nout = D.V;
-        ta.planes = lm_npl;
-        ta.y = z;
-        ta.ldy = (int)ldz;
-        ta.status = dev_status;
-        ta.lm_part = ws.rs_part;
-        ta.lm_nsub = (D.V + TC_LM_GROUP - 1) / TC_LM_GROUP;
-        ta.lm_invT = temperature > 0.f ? 1.f / temperature : 1.f;
-        cudaError_t e2 = launch_tc(ta, ctx->tm_lm, xm, ctx->sms, s);
-        if (e2 != cudaSuccess) return cuda_fail(e2, "lm head launch");
+    auto tc_lm = [&](int all_rows, float *z, long long ldz, const LmPickArgs &pick_in) -> int {
+        const int prows = npad_lm(all_rows);
+        const int lm_nsub = (D.V + TC_LM_GROUP - 1) / TC_LM_GROUP;
+        cudaError_t e2;
+        auto head = [&](int row0, int rows, bool whole) -> int {
+            const TcTiles tt = tc_tiles_lm(rows);
+            CUtensorMap xm;
+            if (!tc_encode_operand(&xm, ws.tc_xl, lm_npl, prows, tt.npad, D.d))
+                return fail(OSPREY_ERR_INVALID_ARG, "lm head: tensor map encoding failed");
+            TcArgs ta{};
+            ta.epi = block ? TC_LM_BLOCK : TC_LM;
+            ta.R = rows;
+            ta.prows = prows;
+            ta.prow0 = row0;
+            ta.block = block;
+            ta.whole = whole;
+            ta.npad = tt.npad;
+            ta.nrt = tt.nrt;
+            ta.bps = tt.bps;
+            ta.fine = rows > TC_TILE_ROWS && !block;
+            ta.K = D.d;
+            ta.nout = D.V;
+            ta.planes = lm_npl;
+            ta.y = z ? z + row0 * ldz : nullptr;
+            ta.ldy = (int)ldz;
+            ta.status = dev_status;
+            ta.lm_part = ws.rs_part + (size_t)row0 * lm_nsub;
+            ta.lm_nsub = lm_nsub;
+            ta.lm_invT = temperature > 0.f ? 1.f / temperature : 1.f;
+            e2 = launch_tc(ta, ctx->tm_lm, xm, ctx->sms, s);
+            return e2 == cudaSuccess ? OSPREY_OK : cuda_fail(e2, "lm head launch");
+        };
+        // block drafting: a group of up to 64 rows sums a reduction of up to 2048 in one segment
+        auto whole = [&](int seqs) { return (seqs * max_new + 15) / 16 * 16 <= 64 && D.d <= 2048; };
+        const int tail = block ? B % grp : 0;   // sequences of the last group, if it is not a full one
+        const bool two = tail && whole(tail) != whole(grp);
+        const int first = two ? (B - tail) * max_new : all_rows;
+        int rc2;
+        if ((rc2 = head(0, first, block && whole(grp))) != OSPREY_OK ||
+            (two && (rc2 = head(first, tail * max_new, whole(tail))) != OSPREY_OK))
+            return rc2;
         LmPickArgs pk = pick_in;
         pk.dim = D;
         pk.part = ws.rs_part;
-        pk.nsub = ta.lm_nsub;
+        pk.nsub = lm_nsub;
         pk.planes = ws.tc_xl;
-        pk.npad = tt.rows();
+        pk.npad = prows;
         pk.npl = lm_npl;
         pk.W = (const uint16_t *)W.lm_head;
         pk.temperature = temperature;
         pk.u_draft = u_draft;
         pk.embed = (const uint16_t *)W.embed;
-        e2 = launch_lm_pick(pk, s);
+        e2 = block ? launch_block_pick(pk, s) : launch_lm_pick(pk, s);
         return e2 == cudaSuccess ? OSPREY_OK : cuda_fail(e2, "sampler launch");
     };
     auto planes = [&](const float *src, const uint16_t *gain, int d_, int rows, int ld, int col0, uint16_t *dst,
@@ -555,6 +584,7 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         pl.last_of_seq = last_of_seq;
         pl.valid = ws.seq_valid;
         pl.rows_per_seq = rows_per_seq;
+        pl.block = block;
         const cudaError_t e2 = launch_planes(pl, s);
         return e2 == cudaSuccess ? OSPREY_OK : cuda_fail(e2, what);
     };
@@ -588,21 +618,36 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         RowMap map{ws.seq_valid, ws.seq_pos0, ws.seq_nnew, rows_per_seq, step};
         float *x = ext ? ws.x_ext : ws.x_chain;
         float *sb = ext ? ws.s_ext : ws.s_chain;
-        const int ns = attn_splits(R, D.Hkv, max_ctx, ctx->sms);
         // the on-chip-merge attention pays off while its clusters fit in one wave
         // (one block per SM); beyond that the global-partials kernel keeps more
         // loads in flight
-        const bool clu = ctx->attn_cs && (long long)R * D.Hkv * ctx->attn_cs <= ctx->sms;
+        auto clusters = [&](int rows) { return ctx->attn_cs && (long long)rows * D.Hkv * ctx->attn_cs <= ctx->sms; };
         // several rows a sequence share their keys: one pass over them for 16 queries
         // (row, head) instead of one a row (96 x 8 rows: 356 us a launch against 592;
-        // 8 x 15 rows, 4 heads a group: 150 against 260).  Below one wave of the decode
+        // 16 x 6 rows: 99 against 141).  Below one wave of the decode
         // kernel's blocks, which then have every page in flight at once, it is the
         // slower one (1 x 8 rows at 2048 keys: 51 us against 24).
-        const int mt = !clu && rows_per_seq > 1 && (long long)R * D.Hkv >= 2 * ctx->sms ? attn_rows_tiles(D, rows_per_seq) : 0;
-        auto attention = [&](AttnArgs &at) {
-            at.n_splits = clu ? ctx->attn_cs : mt ? attn_splits(B * mt, D.Hkv, max_ctx, ctx->sms) : ns;
-            at.split_len = attn_split_len(max_ctx, at.n_splits);
-            return clu ? launch_attn_cluster(at, ctx->attn_cs, s) : mt ? launch_attn_rows(at, B, mt, s) : launch_attn(at, s);
+        const int mt = !block && !clusters(R) && rows_per_seq > 1 && (long long)R * D.Hkv >= 2 * ctx->sms
+                           ? attn_rows_tiles(D, rows_per_seq) : 0;
+        auto attention = [&](const AttnArgs &all) {
+            cudaError_t e2 = cudaSuccess;
+            for (int b0 = 0; b0 < B && e2 == cudaSuccess; b0 += grp) {   // one launch; one a group in block drafting
+                AttnArgs at = all;
+                const size_t r0 = (size_t)b0 * rows_per_seq, ha = (size_t)D.Hq * D.hd;
+                at.R = std::min(grp, B - b0) * rows_per_seq;
+                at.map.valid += b0;
+                at.map.pos0 += b0;
+                at.map.nnew += b0;
+                at.q += r0 * ha;
+                at.out += r0 * ha;
+                if (at.out_planes) at.out_planes += r0 * ha;
+                at.page_table += (size_t)b0 * at.max_pages;
+                const bool clu = clusters(at.R);
+                at.n_splits = clu ? ctx->attn_cs : attn_splits(mt ? B * mt : at.R, D.Hkv, max_ctx, ctx->sms);
+                at.split_len = attn_split_len(max_ctx, at.n_splits);
+                e2 = clu ? launch_attn_cluster(at, ctx->attn_cs, s) : mt ? launch_attn_rows(at, B, mt, s) : launch_attn(at, s);
+            }
+            return e2;
         };
         // activation rows per launch: the streamed kernels serve one or two
         const bool streamed = R <= 2;
@@ -840,7 +885,6 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
             pk.K = 1;
             pk.step = 0;
             pk.max_new = max_new;
-            pk.rows_per_valid = max_new;
             pk.valid = ws.seq_valid;
             pk.nnew = ws.seq_nnew;
             pk.tokens = draft_tokens;
@@ -975,13 +1019,13 @@ extern "C" int osprey_draft_step_topk(osprey_ctx *ctx, const osprey_kv *kv, int 
 }
 
 // ------------------------------------------------------------------ block drafting
-// Sequences are drafted in groups of at most TC_GROUP_ROWS block rows; each
-// group's call reads the weights once (its row tiles share them through L2).  Workspace:
-// the block-mode draft layout of one group, then the group's token array
-// [n][P], n_new [n] and broadcast features [n][P][feat_dim] bf16.
-static int block_group(int B, int P) {
-    const int g = TC_GROUP_ROWS / P;
-    return g < 1 ? 1 : (g < B ? g : B);
+// Sequences are drafted in passes of at most TC_GROUP_ROWS block rows, whole groups
+// of block_group sequences each; a pass reads the weights once (its row tiles share
+// them through L2).  Workspace: the block-mode draft layout of one pass, then the
+// pass's token array [n][P], n_new [n] and broadcast features [n][P][feat_dim] bf16.
+static int block_pass(int B, int P) {
+    const int g = block_group(B, P), n = TC_GROUP_ROWS / P / g * g;
+    return n < g ? g : (n < B ? n : B);
 }
 
 static size_t block_layout(const osprey_ctx *ctx, int n, int P, int max_pages, DraftWs *ws, void *base,
@@ -1009,7 +1053,7 @@ static bool block_args_ok(const osprey_ctx *ctx, int B, int block, int max_pages
 extern "C" size_t osprey_dflash_workspace_bytes(const osprey_ctx *ctx, int B, int block, int max_pages_per_seq) {
     if (!block_args_ok(ctx, B, block, max_pages_per_seq)) return 0;
     const int P = block - 1;
-    return block_layout(ctx, block_group(B, P), P, max_pages_per_seq, nullptr, nullptr, nullptr, nullptr, nullptr);
+    return block_layout(ctx, block_pass(B, P), P, max_pages_per_seq, nullptr, nullptr, nullptr, nullptr, nullptr);
 }
 
 extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, int block, const int32_t *anchors,
@@ -1034,7 +1078,7 @@ extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, i
     if (temperature > 0.f && !u_draft) return fail(OSPREY_ERR_INVALID_ARG, "u_draft is required when temperature > 0");
     if (((uintptr_t)feats | (uintptr_t)workspace) % 16)
         return fail(OSPREY_ERR_INVALID_ARG, "feats and workspace must be 16-byte aligned");
-    const int P = block - 1, G = block_group(B, P);
+    const int P = block - 1, G = block_pass(B, P);
     const Dims &D = ctx->dim;
     DraftWs ws{};
     int32_t *tok = nullptr, *nnew = nullptr;
@@ -1254,7 +1298,7 @@ extern "C" int osprey_verify_hidden(osprey_ctx *ctx, int B, int K, int logits_dt
         if ((e = launch_planes(pl, s)) != cudaSuccess) return cuda_fail(e, "decision-row operand launch");
         // 3. their draft logits on the tensor cores (the draft step's LM head GEMM)
         CUtensorMap xm;
-        if (!tc_encode_operand(&xm, hw.planes, TC_LM_PLANES, TcTiles{1, npad}, D.d))
+        if (!tc_encode_operand(&xm, hw.planes, TC_LM_PLANES, npad, npad, D.d))
             return fail(OSPREY_ERR_INVALID_ARG, "decision-row tensor map encoding failed");
         TcArgs ta{};
         ta.epi = TC_STORE;

@@ -3,8 +3,8 @@
 // one KV head together and streams the key range once for all of them.
 //
 // The decode kernels stream the range once a row, which for 8 rows of 96
-// sequences or 15 rows of a block drafter read every page 8 or 15 times from L2
-// and spent the CUDA cores on as many unpacked multiply-adds.  16 queries a page
+// sequences read every page 8 times from L2 and spent the CUDA cores on as many
+// unpacked multiply-adds.  (Block drafting keeps them, see TcArgs::block.)  16 queries a page
 // are a small matrix product: mma.sync m16n8k16 fits them (a tcgen05 tile has 128
 // rows) and keeps scores and outputs in registers.  It is bound by that
 // instruction's rate, about one in 9 cycles an SM here: 96 of them a page take

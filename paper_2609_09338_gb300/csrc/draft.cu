@@ -504,7 +504,10 @@ __global__ void __launch_bounds__(AT) attn_kernel(const AttnArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     pdl_trigger();   // the next projection may start streaming its weights
     int b, pos;
-    if (!a.map.row(r, b, pos)) return;   // the row map was written by the prepare kernel
+    if (!a.map.row(r, b, pos)) {   // the row map was written by the prepare kernel
+        pdl_wait();   // a later launch waits for this one alone: it must not end before its predecessors
+        return;
+    }
     const int n_keys = pos + 1, pos0 = a.map.pos0[b];
     const int k_begin = split * a.split_len;   // a multiple of the page size
     const int k_end = min(n_keys, k_begin + a.split_len);
@@ -648,7 +651,10 @@ __global__ void __launch_bounds__(AttnCluster<HD, G, CS>::THREADS, 1) attn_clust
     cluster_arrive_relaxed();   // this block has started: its shared memory may be written by the cluster
     pdl_trigger();              // the next projection may start streaming its weights
     int b, pos;
-    if (!a.map.row(r, b, pos)) return;   // the whole cluster (same row) leaves here
+    if (!a.map.row(r, b, pos)) {   // the whole cluster (same row) leaves here
+        pdl_wait();                // (not before its predecessors end, as in attn_kernel)
+        return;
+    }
     const int n_keys = pos + 1, pos0 = a.map.pos0[b];
     const int k_begin = split * a.split_len;   // a multiple of the page size
     const int k_end = min(n_keys, k_begin + a.split_len);

@@ -166,6 +166,19 @@ __device__ __forceinline__ void tc_split(float x, uint16_t (&q)[TC_PLANES]) {
     }
 }
 
+// Merges two (argmax logit a with its id i, sum s of exp((z - a) / T)) pairs
+// into the first: the larger logit wins (the lower id on ties) and the
+// other's sum is rescaled to it.
+__device__ __forceinline__ void lm_combine(float &a1, int &i1, float &s1, float a2, int i2, float s2, float invT) {
+    const bool two = a2 > a1 || (a2 == a1 && i2 < i1);
+    const float aw = two ? a2 : a1, al = two ? a1 : a2;
+    const float sw = two ? s2 : s1, sl = two ? s1 : s2;
+    const float f = al == -INFINITY ? 0.f : __expf((al - aw) * invT);
+    a1 = aw;
+    i1 = two ? i2 : i1;
+    s1 = sw + sl * f;
+}
+
 // 2^x on the special-function unit (PTX ex2.approx, flush-to-zero)
 __device__ __forceinline__ float lm_ex2(float x) {
     float y;
@@ -220,7 +233,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
     // the LM head's two weight tiles: an accumulator of the small planes beside each
     // buffer where they fit, up to 32 rows (16 rows, d 2048: logits 3.3e-6 off the
     // float64 ones instead of 5.1e-6, for 0.7 % of a call)
-    const bool duo = NA > 1 && a.planes > 1 && 4 * acc_cols <= tc_tmem_cols(BPS);
+    const bool duo = NA > 1 && a.sep && 4 * acc_cols <= tc_tmem_cols(BPS);
     uint32_t ncols = 32;
     while (ncols < (own || duo ? 4 : sep ? 3 : 2) * acc_cols) ncols <<= 1;
 
@@ -308,7 +321,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
                         weights(st, y, kb, &full[s]);
                     }
                     for (int p = 0; p < a.planes; ++p)
-                        tma_2d(st + NA * TC_ABYTES + (size_t)p * npad * 128, &xm, kb * 64, p * a.nrt * npad + row0,
+                        tma_2d(st + NA * TC_ABYTES + (size_t)p * npad * 128, &xm, kb * 64, p * a.prows + a.prow0 + row0,
                                &full[s]);
                 }
             }
@@ -378,6 +391,10 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
 #pragma unroll
                                 for (int kk = 0; kk < 4; ++kk)
                                     step(p, kk, tmem + 2u * acc_cols, (kb != klo) || kk || p > 1);
+                        } else if (a.block) {
+#pragma unroll
+                            for (int kk = 0; kk < 4; ++kk)
+                                for (int p = 0; p < a.planes; ++p) step(p, kk, d0, (kb != kb0) || kk || p);
                         } else {
                             // plane by plane (planes inside a k-step made the calls 1.5 % slower), the
                             // small ones first, while the accumulator is small
@@ -450,6 +467,44 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
                     a.lm_part[(size_t)n * a.lm_nsub + sub] =
                         make_float4(mine * a.lm_invT, e[0], mine,
                                     __int_as_float(mine == -INFINITY ? 0x7fffffff : col - lane + first));
+            } else if constexpr (EPI == TC_LM_BLOCK) {
+                // the same partials, as (max, id, sum) triples merged through the butterfly:
+                // the order that block drafting keeps (120 rows, d 4096: 361 us a launch; as above 292)
+                const int sub = (int)(((long long)ft * 128 * NA + 128 * tile + lg) / TC_LM_GROUP);
+                float av[16], sv[16];
+                int ai[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    av[j] = colok ? v[j] : -INFINITY;
+                    ai[j] = colok ? col : 0x7fffffff;
+                    sv[j] = colok ? 1.f : 0.f;
+                    if (a.y && colok && row0 + c0 + j < a.R) a.y[(size_t)(row0 + c0 + j) * a.ldy + col] = v[j];
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int off = 16 >> r, w = 8 >> r;
+                    const bool up = lane & off;
+#pragma unroll
+                    for (int i = 0; i < w; ++i) {
+                        const float ra = __shfl_xor_sync(0xffffffffu, up ? av[i] : av[i + w], off);
+                        const int ri = __shfl_xor_sync(0xffffffffu, up ? ai[i] : ai[i + w], off);
+                        const float rs = __shfl_xor_sync(0xffffffffu, up ? sv[i] : sv[i + w], off);
+                        float ka = up ? av[i + w] : av[i], ks = up ? sv[i + w] : sv[i];
+                        int ki = up ? ai[i + w] : ai[i];
+                        lm_combine(ka, ki, ks, ra, ri, rs, a.lm_invT);
+                        av[i] = ka;
+                        ai[i] = ki;
+                        sv[i] = ks;
+                    }
+                }
+                const float ra = __shfl_xor_sync(0xffffffffu, av[0], 1);
+                const int ri = __shfl_xor_sync(0xffffffffu, ai[0], 1);
+                const float rs = __shfl_xor_sync(0xffffffffu, sv[0], 1);
+                lm_combine(av[0], ai[0], sv[0], ra, ri, rs, a.lm_invT);
+                const int n = row0 + c0 + (lane >> 1);
+                if (!(lane & 1) && n < a.R && sub < a.lm_nsub)
+                    a.lm_part[(size_t)n * a.lm_nsub + sub] =
+                        make_float4(av[0] * a.lm_invT, sv[0], av[0], __int_as_float(ai[0]));
             } else {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -901,7 +956,7 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
     const int topk = a.topk > 1 ? a.topk : 1;
     pdl_trigger();
     pdl_wait();
-    if (!a.valid[a.rows_per_valid > 1 ? b / a.rows_per_valid : b]) return;
+    if (!a.valid[b]) return;
     const bool greedy = a.temperature == 0.f;
     const float invT = greedy ? 1.f : 1.f / a.temperature;
     const float4 *pp = a.part + (size_t)b * a.nsub;
@@ -1128,6 +1183,103 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
     }
 }
 
+// The draw of a block row (row b of sequence b / max_new, one candidate, no next
+// step): the partials as contiguous runs, one a thread, summed and scanned in the
+// order that block drafting keeps (see TcArgs::block).  120 rows of 4748 partials,
+// d 4096: 19 us a launch.
+__global__ void __launch_bounds__(PK_THREADS) block_pick_kernel(const LmPickArgs a) {
+    extern __shared__ float hrow[];   // [d] the row's LM-head operand
+    __shared__ MS sm_ms[PK_WARPS];
+    __shared__ AM sm_am[PK_WARPS];
+    __shared__ float sh[34], s_z[TC_LM_GROUP], s_before;
+    __shared__ int si[2], s_grp;
+    const Dims &D = a.dim;
+    const int b = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    pdl_trigger();
+    pdl_wait();
+    if (!a.valid[b / a.max_new]) return;
+    const bool greedy = a.temperature == 0.f;
+    const float invT = greedy ? 1.f : 1.f / a.temperature;
+    const float4 *pp = a.part + (size_t)b * a.nsub;
+    const int per = (a.nsub + PK_THREADS - 1) / PK_THREADS;
+    const int j0 = min(a.nsub, t * per), j1 = min(a.nsub, j0 + per);
+    // the run's argmax, and its (max, sum) rescaled online
+    float m = -INFINITY, sm = 0.f;
+    AM am{-INFINITY, 0x7fffffff};
+    for (int j = j0; j < j1; ++j) {
+        const float4 p = __ldcg(pp + j);
+        am = am_combine(am, AM{p.z, __float_as_int(p.w)});
+        if (p.x == -INFINITY) continue;
+        if (p.x > m) {
+            sm = (m == -INFINITY ? 0.f : sm * __expf(m - p.x)) + p.y;
+            m = p.x;
+        } else {
+            sm += p.y * __expf(p.x - m);
+        }
+    }
+    const MS tot = block_ms(MS{m, sm}, sm_ms);
+    const float M = tot.m, S = tot.s;
+    if (greedy) {
+        const AM top = block_am(am, sm_am);
+        if (t == 0) {
+            a.tokens[b] = top.i;
+            if (a.qx) a.qx[b] = 1.f;
+        }
+    } else {
+        const float w = m == -INFINITY ? 0.f : sm * __expf(m - M);   // the run's weight
+        const size_t plane = (size_t)a.npad * D.d;
+        const uint16_t *q = a.planes + (size_t)b * D.d;
+        for (int k = t; k < D.d; k += PK_THREADS) {
+            float h = 0.f;
+#pragma unroll
+            for (int i = 0; i < TC_LM_PLANES; ++i) h += bf_to_f(q[i * plane + k]);
+            hrow[k] = h;
+        }
+        float all;
+        const float ex = block_excl_scan(w, sh, &all);
+        const float target = a.u_draft[b] * S;
+        if (t == 0) { si[0] = 0x7fffffff; si[1] = -1; }
+        __syncthreads();
+        if (w > 0.f && target < ex + w) atomicMin(&si[0], t);
+        if (w > 0.f) atomicMax(&si[1], t);
+        __syncthreads();
+        const int ct = si[0] != 0x7fffffff ? si[0] : (si[1] >= 0 ? si[1] : 0);
+        if (t == ct) {   // this thread's run holds the point: find its group
+            float cum = ex;
+            int grp = -1, lastg = -1;
+            float lastb = ex;
+            for (int j = j0; j < j1; ++j) {
+                const float4 p = __ldcg(pp + j);
+                const float wj = p.x != -INFINITY ? p.y * __expf(p.x - M) : 0.f;
+                if (wj > 0.f) { lastg = j; lastb = cum; }
+                if (wj > 0.f && target < cum + wj) { grp = j; break; }
+                cum += wj;
+            }
+            s_grp = grp >= 0 ? grp : (lastg >= 0 ? lastg : j0);
+            s_before = grp >= 0 ? cum : lastb;
+        }
+        __syncthreads();
+        pk_group_logits(a, hrow, &s_grp, 1, s_z);
+        __syncthreads();
+        if (warp == 0) {
+            const int id = s_grp * TC_LM_GROUP + lane;
+            const float e = id < D.V ? __expf(s_z[lane] * invT - M) : 0.f;
+            const float cum = s_before + warp_incl_scan(e);
+            const unsigned hit = __ballot_sync(0xffffffffu, e > 0.f && target < cum);
+            const unsigned pos = __ballot_sync(0xffffffffu, e > 0.f);
+            const int l = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
+            if (lane == l) {
+                a.tokens[b] = id;
+                if (a.qx) a.qx[b] = e / S;
+            }
+        }
+    }
+    if (t == 0 && a.stats) {
+        a.stats[(size_t)b * 2 + 0] = M;
+        a.stats[(size_t)b * 2 + 1] = logf(S);
+    }
+}
+
 // ---------------------------------------------------------------- embedding rows
 __global__ void __launch_bounds__(1024) embed_rows_kernel(const EmbedArgs a) {
     const int r = blockIdx.x, b = r / a.max_new, j = r - b * a.max_new;
@@ -1194,8 +1346,8 @@ static bool encode2d(CUtensorMap *m, const void *base, uint64_t inner, uint64_t 
 
 bool tc_encode_weight(CUtensorMap *m, const void *w, int rows, int K) { return encode2d(m, w, K, rows, 128); }
 bool tc_encode_rows(CUtensorMap *m, const void *x, int rows, int npad, int K) { return encode2d(m, x, K, rows, npad); }
-bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, const TcTiles &t, int K) {
-    return encode2d(m, x, K, (uint64_t)planes * t.rows(), t.npad);
+bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, int prows, int npad, int K) {
+    return encode2d(m, x, K, (uint64_t)planes * prows, npad);
 }
 
 static int tc_stages(int npad, int planes, int na, int bps) {
@@ -1208,7 +1360,10 @@ static size_t tc_smem_bytes(int npad, int planes, int na, int bps) {
     return (size_t)tc_stages(npad, planes, na, bps) * stage + 1024;
 }
 
-cudaError_t tc_set_attributes() { return allow_smem(lm_pick_kernel); }
+cudaError_t tc_set_attributes() {
+    const cudaError_t e = allow_smem(lm_pick_kernel);
+    return e == cudaSuccess ? allow_smem(block_pick_kernel) : e;
+}
 
 template <typename... P, typename... A>
 static cudaError_t pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A &...args) {
@@ -1287,19 +1442,22 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     if (planes_done) *planes_done = false;
     if (a.nrt < 1) a.nrt = 1;
     if (a.bps != 1) a.bps = 2;
-    if (a.bps == 1 && a.epi == TC_LM) return cudaErrorInvalidValue;
+    const bool lm = a.epi == TC_LM || a.epi == TC_LM_BLOCK;
+    if (a.prows < 1) a.prows = a.nrt * a.npad;
+    if (a.bps == 1 && lm) return cudaErrorInvalidValue;
     if (a.npad % 16 || a.npad < 16 || a.npad > (a.bps == 1 ? TC_BIG_ROWS : TC_TILE_ROWS) || a.K % 64 || a.R > (long long)a.nrt * a.npad)
         return cudaErrorInvalidValue;
     if (a.nout_a < 1 || a.nout_a > a.nout || (a.nout_a < a.nout && a.nout_a % 128)) return cudaErrorInvalidValue;
     if (a.epi == TC_GLU && (a.nout != 2 * a.nout_a || !a.part || !a.h || a.h_rows < a.R)) return cudaErrorInvalidValue;
     const int nkb = a.K / 64;
-    if (a.epi == TC_LM && (!a.lm_part || a.lm_nsub != (a.nout + TC_LM_GROUP - 1) / TC_LM_GROUP))
+    if (lm && (!a.lm_part || a.lm_nsub != (a.nout + TC_LM_GROUP - 1) / TC_LM_GROUP))
         return cudaErrorInvalidValue;
-    a.nsplit = a.part && a.epi != TC_LM ? tc_nsplit(a.nout, a.K, TcTiles{a.nrt, a.npad, a.bps}, sms) : 1;   // the LM epilogue needs whole sums
+    // (the LM epilogue needs whole sums)
+    a.nsplit = a.part && !lm ? tc_nsplit(a.nout, a.K, a.block ? TC_BLOCK_SPLITS : TcTiles{a.nrt, a.npad, a.bps}, sms) : 1;
     if ((long long)a.nsplit * a.R * a.nout > a.part_cap) a.nsplit = 1;
     if (a.epi == TC_GLU && (long long)a.nsplit * a.R * a.nout > a.part_cap) return cudaErrorInvalidValue;
     a.kbps = (nkb + a.nsplit - 1) / a.nsplit;
-    a.sep = a.planes > 1;   // (0.1 % of a call, for a third of the accumulators' error)
+    a.sep = a.planes > 1 && !a.block;   // (0.1 % of a call, for a third of the accumulators' error)
     a.segkb = a.fine ? OSP_TC_SEGKB_FINE : OSP_TC_SEGKB;
     const int bps = a.bps, tmem_cols = tc_tmem_cols(bps);
     // the LM head takes OSP_TC_LM_NA weight tiles per stage when two stages fit
@@ -1307,7 +1465,8 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     // reduction over d is short: one segment keeps its MMA chain at 4 d / 64 steps
     // per plane)
     int na = 1;
-    const bool wide = a.epi == TC_LM || (a.epi == TC_STORE && a.nsplit == 1 && a.wide);
+    if (a.block && a.whole) a.segkb = a.kbps;
+    const bool wide = (lm && (!a.block || a.whole)) || (a.epi == TC_STORE && a.nsplit == 1 && a.wide);
     if (wide && a.nrt == 1 && OSP_TC_LM_NA > 1 && tc_stages(a.npad, a.planes, OSP_TC_LM_NA, bps) >= 2 &&
         2 * OSP_TC_LM_NA * a.npad <= tmem_cols && a.kbps <= 32 && a.planes <= TC_LM_PLANES) {
         na = OSP_TC_LM_NA;
@@ -1332,6 +1491,9 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     case TC_STORE: e = na > 1 ? OSP_TC_GO(TC_STORE, OSP_TC_LM_NA, 1, 2) : OSP_TC_ROWS(TC_STORE); break;
     case TC_RESID: e = OSP_TC_ROWS(TC_RESID); break;
     case TC_GLU: e = OSP_TC_ROWS(TC_GLU); break;
+    case TC_LM_BLOCK:
+        e = na > 1 ? OSP_TC_GO(TC_LM_BLOCK, OSP_TC_LM_NA, 1, 2) : cs > 1 ? OSP_TC_GO(TC_LM_BLOCK, 1, TC_CS, 2) : OSP_TC_GO(TC_LM_BLOCK, 1, 1, 2);
+        break;
     default:
         e = na > 1 ? OSP_TC_GO(TC_LM, OSP_TC_LM_NA, 1, 2) : cs > 1 ? OSP_TC_GO(TC_LM, 1, TC_CS, 2) : OSP_TC_GO(TC_LM, 1, 1, 2);
         break;
@@ -1374,7 +1536,7 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
 }
 
 cudaError_t launch_planes(const PlaneArgs &a, cudaStream_t s) {
-    return pdl_launch(planes_kernel, dim3(a.R), dim3(row_threads(a.d)), 0, s, a);
+    return pdl_launch(planes_kernel, dim3(a.R), dim3(a.block ? 256 : row_threads(a.d)), 0, s, a);
 }
 
 cudaError_t launch_qkv_post(const QkvPostArgs &a, cudaStream_t s) {
@@ -1388,6 +1550,10 @@ cudaError_t launch_embed_rows(const EmbedArgs &a, cudaStream_t s) {
 
 cudaError_t launch_lm_pick(const LmPickArgs &a, cudaStream_t s) {
     return pdl_launch(lm_pick_kernel, dim3(a.B), dim3(PK_THREADS), (size_t)a.dim.d * 4, s, a);
+}
+
+cudaError_t launch_block_pick(const LmPickArgs &a, cudaStream_t s) {
+    return pdl_launch(block_pick_kernel, dim3(a.B), dim3(PK_THREADS), (size_t)a.dim.d * 4, s, a);
 }
 
 }  // namespace osp

@@ -33,7 +33,8 @@ namespace osp {
 // TC_LM: the LM head; per row and 32-id group of the vocabulary the epilogue
 // keeps only (max of logits/T, sum of exp(logits/T - max), argmax logit and its
 // id), and stores the logits only when y is given.
-enum TcEpi { TC_STORE = 0, TC_RESID = 1, TC_GLU = 2, TC_LM = 3 };
+// TC_LM_BLOCK: the same for block drafting, in its order of summation (TcArgs::block).
+enum TcEpi { TC_STORE = 0, TC_RESID = 1, TC_GLU = 2, TC_LM = 3, TC_LM_BLOCK = 4 };
 constexpr int TC_LM_GROUP = 32;    // vocabulary ids per LM-head partial (one epilogue warp's lanes)
 // The LM head's operand rows enter as two bf16 planes (16 significant bits):
 // a logit's error from the dropped bits is a sum of d random terms of
@@ -80,16 +81,28 @@ inline TcTiles tc_tiles(long long rows, int K) {
 // 96 rows, V 151936, d 1024, in two tiles of 48 132 us, in one of 96 161.  An even
 // number of tiles: pairs share the weights that they load.
 inline TcTiles tc_tiles_lm(long long rows) { return tc_tiles_of(rows, TC_TILE_ROWS, 2, 2); }
+// k-ranges of block drafting's GEMMs: those of one row tile, whatever the rows
+constexpr TcTiles TC_BLOCK_SPLITS{1, TC_TILE_ROWS, 2};
 
 struct TcArgs {
     int epi;           // TcEpi
     int R;             // rows
-    int npad, nrt;     // rows per tile (a multiple of 16), row tiles; an operand plane has nrt * npad rows
+    int npad, nrt;     // rows per tile (a multiple of 16), row tiles
+    int prows, prow0;  // rows of an operand plane (0: nrt * npad), the first row's place in it
     int bps;           // CTAs per SM
     int K;             // reduction length (multiple of 64)
     int nout;          // output features (tiles of 128, the last one may be partial)
     int nout_a;        // features [0, nout_a) from the first weight map, the rest from the second
     int planes;        // 1 (bf16 input) or TC_PLANES (split float32 input)
+    // Block drafting.  Its mask positions leave up to half of the draft mass on ids of
+    // probability 1e-7 to 1e-5, less than a float32 sum over the row resolves: two
+    // orders of summation, both within 1e-5 of float64, put 8 of 1920 sampled ids on
+    // different neighbours.  So these calls keep one order, whatever is drafted beside
+    // a sequence: one accumulator for all planes (plane by plane within a k-step) over
+    // segments of 8 k-blocks, the k-ranges of one row tile, attention and the LM
+    // head's segments by groups of TC_TILE_ROWS rows, runs and merges of the sampler.
+    bool block;
+    bool whole;        // TC_LM_BLOCK: the whole reduction in one segment
     bool wide;         // TC_STORE of the LM head: the LM head's tiles, so the same sums bit for bit
     float *y;          // TC_STORE: [R][ldy] float32 output
     int ldy;
@@ -123,10 +136,10 @@ struct TcArgs {
 };
 
 // Host side.  Tensor maps: weights [rows][K] bf16 with a 64 x 128 box, operand
-// planes [planes * tiles.rows()][K] bf16 with a 64 x npad box, both 128-byte swizzled.
+// planes [planes * prows][K] bf16 with a 64 x npad box, both 128-byte swizzled.
 bool tc_available();   // the driver exposes tensor-map encoding and the device is sm_100+
 bool tc_encode_weight(CUtensorMap *m, const void *w, int rows, int K);
-bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, const TcTiles &t, int K);
+bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, int prows, int npad, int K);
 // a single bf16 plane of `rows` rows read in place (rows past `rows` read as zero)
 bool tc_encode_rows(CUtensorMap *m, const void *x, int rows, int npad, int K);
 size_t tc_smem_bytes(int npad, int planes, int na);
@@ -168,6 +181,7 @@ struct PlaneArgs {
     // every draft token was accepted
     const Decision *dec;
     int dec_b0, dec_K;
+    bool block;                // block drafting: 256 threads a row at every d (TcArgs::block)
 };
 cudaError_t launch_planes(const PlaneArgs &a, cudaStream_t s);
 
@@ -191,14 +205,14 @@ cudaError_t launch_qkv_post(const QkvPostArgs &a, cudaStream_t s);
 // group's logits, recomputed from the LM head's operand planes; T = 0 takes the
 // argmax (lowest id).  Writes the token, q(token), (max, log-sum-exp) and, when
 // a next chain step follows, the next chain row (context slot = x_L, residual =
-// E[token]).  Row b belongs to sequence b / rows_per_valid (0 or 1: itself).
+// E[token]).
 // topk > 1 (tree drafting): k candidates per row, [B][K][k] in tokens and qx;
 // sampled: k independent inverse-CDF draws at u_draft[b][step][j]; greedy: the
 // k highest logits in descending order (ties to the lowest id).  Candidate 0
 // continues the chain.
 struct LmPickArgs {
     Dims dim;
-    int B, K, step, max_new, src_is_ext, rows_per_valid;
+    int B, K, step, max_new, src_is_ext;
     int topk;                  // candidates per row (0 or 1: one)
     const int *valid, *nnew;
     const float4 *part;        // [B][nsub] TC_LM partials
@@ -221,6 +235,8 @@ struct LmPickArgs {
     int qkv_npad;
 };
 cudaError_t launch_lm_pick(const LmPickArgs &a, cudaStream_t s);
+// Block drafting: rows b of sequences b / max_new, one candidate, no next step.
+cudaError_t launch_block_pick(const LmPickArgs &a, cudaStream_t s);
 // Block drafting inputs (EAGLE-style DFlash): for row r = b*P + j of n
 // sequences, tokens[r] = anchor[b] (j = 0) or mask (j > 0); feats_rep[r] =
 // feats[b] (feat_dim bf16, broadcast over the block); nnew[b] = P.

@@ -1,0 +1,91 @@
+"""Block drafting keeps one order of summation.
+
+Mask positions leave much of the draft mass on ids of 1e-6 beside a leading one.  A float32 drafter's leading logit is
+some 1e-5 off, which moves the cumulative sum past several such ids, so any other order of any sum on the way draws
+neighbouring ids.  The ids and logits of a call are the same bit for bit whatever else is drafted in it, and the ids are
+those recorded in tests/golden/block_ids.json.
+"""
+import json
+import os
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle.bf16 import widen  # noqa: E402
+from paper_2609_09338_gb300 import synthetic as syn  # noqa: E402
+from paper_2609_09338_gb300.workloads import TINY  # noqa: E402
+from test_dflash_gpu import _built  # noqa: E402,F401
+
+GOLDEN = os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "block_ids.json")
+# groups of 5 + 3 and of 8 + 1 sequences (the last one with one LM-head segment)
+CASES = {
+    "d512-b8-blk16": (replace(TINY, d_model=512, n_layers=4, n_q_heads=8, n_kv_heads=2, ffn_dim=4096, feat_dim=4096,
+                              vocab=262144), [30, 1, 64, 17, 5, 90, 200, 41], 16),
+    "d1024-b9-blk11": (replace(TINY, d_model=1024, n_layers=2, n_q_heads=8, n_kv_heads=4, ffn_dim=2048, feat_dim=4096,
+                               vocab=131072), [700, 3, 9, 61, 2, 18, 33, 150, 40], 11),
+}
+
+
+def make(shape, ctx, block, seed):
+    """Weights whose head gives each token one successor of about half the mass, and a call's inputs."""
+    w = syn.make_weights(shape, seed)
+    rng = np.random.default_rng(seed + 1)
+    embed = widen(w["embed"]) * np.float32(50)                      # N(0, 1)
+    w["embed"] = syn.bf16_bits(embed)
+    gain = np.log(shape.vocab) * np.sqrt(1 + shape.n_layers * shape.d_model / 2560) / shape.d_model
+    w["lm_head"] = syn.bf16_bits(widen(w["lm_head"]) + np.float32(gain) * embed[rng.permutation(shape.vocab)])
+    B, P = len(ctx), block - 1
+    return {"shape": shape, "block": block, "ctx": np.asarray(ctx, np.int32), "w": w,
+            "kv": syn.make_kv_prefix(shape, np.asarray(ctx, np.int32), P, seed + 2),
+            "anchors": rng.integers(0, shape.vocab, size=B).astype(np.int32),
+            "feats": syn.make_draft_inputs(shape, B, 1, 1, seed + 3)["feats"][:, 0],
+            "u": rng.random((B, P), dtype=np.float32)}
+
+
+def propose(c, T, seqs=None):
+    from paper_2609_09338_gb300.binding import to_device_bf16
+    from paper_2609_09338_gb300.session import DflashSession
+    seqs = list(range(len(c["ctx"]))) if seqs is None else seqs
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    offs = np.concatenate([[0], np.cumsum(c["ctx"])])
+    rows = np.concatenate([np.arange(offs[b], offs[b + 1]) for b in seqs])
+    kv = c["kv"]
+    sess = DflashSession(c["shape"], c["w"], kv["page_table"][seqs], kv["n_pages"], c["block"])
+    sess.append(c["ctx"][seqs], kv["k_rows"][:, rows], kv["v_rows"][:, rows])
+    out = sess.block_buffers(with_logits=True)
+    sess.propose(dev(c["anchors"][seqs]), 5, to_device_bf16(np.ascontiguousarray(c["feats"][seqs])), T,
+                 dev(c["u"][seqs]), out)
+    torch.cuda.synchronize()
+    assert int(sess.status.item()) == 0
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+def ids_of(name):
+    shape, ctx, block = CASES[name]
+    return propose(make(shape, ctx, block, 91), 1.0)
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_sampled_ids_are_the_recorded_ones(name):
+    with open(GOLDEN) as f:
+        want = np.array(json.load(f)[name], np.int32)
+    np.testing.assert_array_equal(ids_of(name)["draft_tokens"], want)
+
+
+@pytest.mark.parametrize("block,T", [(16, 1.0), (11, 0.0), (24, 1.0)])
+def test_groups_do_not_change_one_another(block, T):
+    """A call's groups of up to 80 rows give bit for bit what each gives in a call of its own."""
+    shape = replace(TINY, d_model=768, n_layers=2, n_q_heads=4, vocab=32768)
+    P = block - 1
+    B, group = 2 * (80 // P) + 1, 80 // P
+    c = make(shape, np.random.default_rng(block).integers(1, 200, size=B), block, 71)
+    whole = propose(c, T)
+    for b0 in range(0, B, group):
+        seqs = list(range(b0, min(B, b0 + group)))
+        own = propose(c, T, seqs)
+        for k in own:
+            np.testing.assert_array_equal(whole[k][seqs], own[k], err_msg=f"{k} of group {b0}")
