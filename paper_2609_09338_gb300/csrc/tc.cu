@@ -34,8 +34,6 @@ namespace cg = cooperative_groups;
 constexpr int TC_THREADS = 192;
 constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
 constexpr int TC_MAXST = 8;
-constexpr int TC_CS = 2;      // CTAs of a cluster that share weight tiles
-constexpr long long TC_SHARE_BYTES = 40ll << 20;   // weights above which they do
 // Two CTAs per SM are two TMA producers, MMA chains and epilogues; one has all of
 // TMEM and shared memory, and tiles of up to TC_BIG_ROWS rows (tc_tiles).  An MMA reads its 4 KB of weights from shared memory however
 // many rows it multiplies (32 cycles; 16 rows more take 4), so 128 rows at once
@@ -73,16 +71,6 @@ __device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, int x, i
         "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar))
         : "memory");
 }
-// The same to this CTA's and the other CTAs' shared memory of the cluster (mask),
-// counted at the same place's barrier in each.
-__device__ __forceinline__ void tma_2d_multicast(void *dst, const CUtensorMap *m, int x, int y, uint64_t *bar,
-                                                 uint16_t mask) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-        "%3}], [%4], %5;" ::"r"(smem_u32(dst)),
-        "l"(m), "r"(x), "r"(y), "r"(smem_u32(bar)), "h"(mask)
-        : "memory");
-}
 // Shared-memory matrix descriptor: K-major tile, rows 128 bytes apart inside
 // 8-row (1024-byte) swizzle atoms.
 __device__ __forceinline__ uint64_t tc_desc(uint32_t saddr) {
@@ -113,17 +101,6 @@ __device__ __forceinline__ bool tc_elect() {
 __device__ __forceinline__ void tc_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
-}
-// ... arriving at the same place's barrier in every CTA of the mask
-__device__ __forceinline__ void tc_commit_multicast(uint64_t *bar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
-        "h"(mask)
-        : "memory");
-}
-__device__ __forceinline__ void tc_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -191,11 +168,10 @@ __device__ __forceinline__ float lm_ex2(float x) {
 // planes: one work item is NA adjacent tiles, accumulated side by side in TMEM.
 // Output features [0, nout_a) come from the weights of map wa, the rest from
 // wb (row f - nout_a): the SwiGLU gate and up projections run as one GEMM.
-// CS > 1 (several row tiles): the CTAs of a cluster of CS take adjacent row tiles
-// of the same features and k-range, and each weight tile is loaded once, by the
-// CTAs in turn, and multicast.  A slot is free when every CTA's MMAs have read it.
+// a.pair CTAs next to one another take adjacent row tiles of the same features and
+// k-range at the same time: the second one's weight tiles come from L2.
 // BPS: CTAs per SM.
-template <int EPI, int NA, int CS, int BPS>
+template <int EPI, int NA, int BPS>
 __global__ void __launch_bounds__(TC_THREADS, BPS)
     tc_kernel(const __grid_constant__ CUtensorMap wa, const __grid_constant__ CUtensorMap wb,
               const __grid_constant__ CUtensorMap xm, const TcArgs a, int nst) {
@@ -205,15 +181,14 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // work item of a cluster = (NA output tiles of 128 features, CS row tiles,
-    // k-range), the k-range fastest; items of a cluster are contiguous
+    // work item of a pair = (NA output tiles of 128 features, a.pair row tiles,
+    // k-range), the k-range fastest; items of a pair are contiguous
     const int segkb = a.segkb;
-    const int nrg = a.nrt / CS, per_ft = nrg * a.nsplit;   // items of one feature tile
+    const int pair = a.pair, nrg = a.nrt / pair, per_ft = nrg * a.nsplit;   // items of one feature tile
     const int n_items = (a.nout + 128 * NA - 1) / (128 * NA) * per_ft;
-    const int rank = CS > 1 ? (int)(blockIdx.x % CS) : 0, cl = blockIdx.x / CS, ncl = gridDim.x / CS;
-    const int i0 = (int)((long long)n_items * cl / ncl);
-    const int i1 = (int)((long long)n_items * (cl + 1) / ncl);
-    constexpr uint16_t all = (uint16_t)((1 << CS) - 1);
+    const int rank = blockIdx.x % pair, at = blockIdx.x / pair, of = gridDim.x / pair;
+    const int i0 = (int)((long long)n_items * at / of);
+    const int i1 = (int)((long long)n_items * (at + 1) / of);
     const int nloc = i1 - i0, nkb = a.K / 64, npad = a.npad;
     auto krange = [&](int item, int &lo, int &hi) {
         const int sp = item % a.nsplit;
@@ -245,7 +220,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
     if (threadIdx.x == 32) {
         for (int i = 0; i < nst; ++i) {
             mbar_init(&full[i], 1);
-            mbar_init(&empty[i], CS);
+            mbar_init(&empty[i], 1);
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&accf[i], 1);
@@ -257,8 +232,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
         mbar_fence_init();
     }
     tc_fence_before();
-    if (CS > 1) tc_cluster_sync();   // every CTA's barriers are ready for the others' copies and commits
-    else __syncthreads();
+    __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
     pdl_trigger();
@@ -270,14 +244,10 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
     if (warp == 0) {
         if (tc_elect()) {
             auto weights = [&](uint8_t *st, int y, int kb, uint64_t *bar) {
-                if (CS > 1 && kb % CS != rank) return;   // another CTA of the cluster brings them
 #pragma unroll
                 for (int t = 0; t < NA; ++t) {
                     const int f = y + 128 * t;   // tiles never straddle nout_a (a multiple of 128)
-                    const CUtensorMap *w = f < a.nout_a ? &wa : &wb;
-                    const int r = f < a.nout_a ? f : f - a.nout_a;
-                    if constexpr (CS > 1) tma_2d_multicast(st + t * TC_ABYTES, w, kb * 64, r, bar, all);
-                    else tma_2d(st + t * TC_ABYTES, w, kb * 64, r, bar);
+                    tma_2d(st + t * TC_ABYTES, f < a.nout_a ? &wa : &wb, kb * 64, f < a.nout_a ? f : f - a.nout_a, bar);
                 }
             };
             int npre = 0;   // stages whose weights were requested before the wait
@@ -298,7 +268,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
             bool stop = false;
             for (int it = 0; it < nloc && !stop; ++it) {
                 const int y = (i0 + it) / per_ft * 128 * NA;
-                const int row0 = ((i0 + it) / a.nsplit % nrg * CS + rank) * npad;   // of the operand planes
+                const int row0 = ((i0 + it) / a.nsplit % nrg * pair + rank) * npad;   // of the operand planes
                 int klo, khi;
                 krange(i0 + it, klo, khi);
                 for (int kb = klo; kb < khi; ++kb, ++g, ++s) {
@@ -405,8 +375,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
                                 for (int kk = 0; kk < 4; ++kk) step(p, kk, d, !first || kk);
                             }
                         }
-                        if (CS > 1) tc_commit_multicast(&empty[s], all);
-                        else tc_commit(&empty[s]);
+                        tc_commit(&empty[s]);
                     }
                     if (!stop) tc_commit(&accf[buf]);
                 }
@@ -524,7 +493,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
             ft = (i0 + it) / per_ft;
             sp = (i0 + it) % a.nsplit;
             col0 = ft * 128 * NA + m;
-            row0 = ((i0 + it) / a.nsplit % nrg * CS + rank) * npad;
+            row0 = ((i0 + it) / a.nsplit % nrg * pair + rank) * npad;
             int klo, khi;
             krange(i0 + it, klo, khi);
             const int nseg = (khi - klo + segkb - 1) / segkb;
@@ -626,8 +595,7 @@ __global__ void __launch_bounds__(TC_THREADS, BPS)
         }
     }
     tc_fence_before();
-    if (CS > 1) tc_cluster_sync();   // the other CTAs write nothing more to this one's shared memory
-    else __syncthreads();
+    __syncthreads();
     tc_fence_after();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
@@ -1382,7 +1350,7 @@ static cudaError_t pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t sme
     return e;
 }
 
-template <int EPI, int NA, int CS, int BPS>
+template <int EPI, int NA, int BPS>
 static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtensorMap &wa, const CUtensorMap &wb,
                              const CUtensorMap &xm, const TcArgs &a, int nst) {
     // opted into its shared memory, and so loaded, at its first launch: with every
@@ -1390,28 +1358,11 @@ static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtens
     // in L2) took 679 us instead of 672
     static std::atomic<int> done[kMaxDevices];
     const cudaError_t es = once_per_device(done, [] {
-        return cudaFuncSetAttribute(tc_kernel<EPI, NA, CS, BPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        return cudaFuncSetAttribute(tc_kernel<EPI, NA, BPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)tc_smem_cap(BPS));
     });
     if (es != cudaSuccess) return es;
-    if (CS == 1) return pdl_launch(tc_kernel<EPI, NA, CS, BPS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = CS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, tc_kernel<EPI, NA, CS, BPS>, wa, wb, xm, a, nst);
-    count_launch();
-    return e;
+    return pdl_launch(tc_kernel<EPI, NA, BPS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
 }
 
 // k-ranges per output tile so that tiles x ranges fill the CTA slots (few
@@ -1475,28 +1426,22 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     const int nst = tc_stages(a.npad, a.planes, na, bps);
     if (nst < 2) return cudaErrorInvalidValue;
     if ((na == 1 && a.sep ? 3 : 2) * na * a.npad > tmem_cols) return cudaErrorInvalidValue;   // TMEM columns
-    // pairs of row tiles share weights that the L2 does not keep from one tile to the
-    // next
-    const int cs = a.nrt % TC_CS == 0 && (long long)a.nout * a.K * 2 > TC_SHARE_BYTES ? TC_CS : 1;
-    if (a.nrt % cs || (cs > 1 && na > 1)) return cudaErrorInvalidValue;
-    const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / cs) * a.nsplit, slots = bps * sms / cs;
-    const int grid = (items < slots ? items : slots) * cs;
+    // an even number of row tiles goes in pairs: the weights of the second one come from
+    // L2 also where a tile's next one would find them gone (120 rows, d 4096: 2496 us a
+    // call, one row tile after the other 2570; 96 rows, d 1024: 2864, 2884)
+    a.pair = a.nrt % 2 == 0 ? 2 : 1;
+    const int items = (a.nout + 128 * na - 1) / (128 * na) * (a.nrt / a.pair) * a.nsplit, slots = bps * sms / a.pair;
+    const int grid = (items < slots ? items : slots) * a.pair;
     const size_t smem = tc_smem_bytes(a.npad, a.planes, na, bps);
     cudaError_t e;
-#define OSP_TC_GO(EPI, NA_, CS_, BPS_) tc_launch<EPI, NA_, CS_, BPS_>(grid, smem, s, wa, wb, xm, a, nst)
-#define OSP_TC_ROWS(EPI)                                                          \
-    (bps == 1 ? (cs > 1 ? OSP_TC_GO(EPI, 1, TC_CS, 1) : OSP_TC_GO(EPI, 1, 1, 1)) \
-              : (cs > 1 ? OSP_TC_GO(EPI, 1, TC_CS, 2) : OSP_TC_GO(EPI, 1, 1, 2)))
+#define OSP_TC_GO(EPI, NA_, BPS_) tc_launch<EPI, NA_, BPS_>(grid, smem, s, wa, wb, xm, a, nst)
+#define OSP_TC_ROWS(EPI) (bps == 1 ? OSP_TC_GO(EPI, 1, 1) : OSP_TC_GO(EPI, 1, 2))
     switch (a.epi) {
-    case TC_STORE: e = na > 1 ? OSP_TC_GO(TC_STORE, OSP_TC_LM_NA, 1, 2) : OSP_TC_ROWS(TC_STORE); break;
+    case TC_STORE: e = na > 1 ? OSP_TC_GO(TC_STORE, OSP_TC_LM_NA, 2) : OSP_TC_ROWS(TC_STORE); break;
     case TC_RESID: e = OSP_TC_ROWS(TC_RESID); break;
     case TC_GLU: e = OSP_TC_ROWS(TC_GLU); break;
-    case TC_LM_BLOCK:
-        e = na > 1 ? OSP_TC_GO(TC_LM_BLOCK, OSP_TC_LM_NA, 1, 2) : cs > 1 ? OSP_TC_GO(TC_LM_BLOCK, 1, TC_CS, 2) : OSP_TC_GO(TC_LM_BLOCK, 1, 1, 2);
-        break;
-    default:
-        e = na > 1 ? OSP_TC_GO(TC_LM, OSP_TC_LM_NA, 1, 2) : cs > 1 ? OSP_TC_GO(TC_LM, 1, TC_CS, 2) : OSP_TC_GO(TC_LM, 1, 1, 2);
-        break;
+    case TC_LM_BLOCK: e = na > 1 ? OSP_TC_GO(TC_LM_BLOCK, OSP_TC_LM_NA, 2) : OSP_TC_GO(TC_LM_BLOCK, 1, 2); break;
+    default: e = na > 1 ? OSP_TC_GO(TC_LM, OSP_TC_LM_NA, 2) : OSP_TC_GO(TC_LM, 1, 2); break;
     }
 #undef OSP_TC_ROWS
 #undef OSP_TC_GO

@@ -4,8 +4,8 @@
 //
 // Weights are the M = 128 operand, streamed tile by tile with 2-D TMA (128-byte
 // swizzle); the R activation rows are the N operand, in equal tiles (tc_tiles).
-// Pairs of row tiles share weights that are read from HBM each time: a cluster of
-// two CTAs loads a tile once and multicasts it.  The LM head of one row tile
+// Row tiles share the weights through L2: CTAs next to one another take two of them
+// at the same time.  The LM head of one row tile
 // multiplies two weight tiles against each stage's operand planes (twice the
 // weight bytes in flight per byte of operand reloaded).
 //
@@ -130,6 +130,7 @@ struct TcArgs {
     float *part;
     long long part_cap;   // floats available in part
     int nsplit, kbps;     // set by launch_tc
+    int pair;             // CTAs next to one another on adjacent row tiles (1 or 2), set by launch_tc
     int segkb;            // k-blocks per accumulation segment, set by launch_tc
     bool fine;            // short accumulation segments (calls of more rows than a tile, block drafting aside)
     bool sep;             // planes after the first accumulate by themselves, set by launch_tc
