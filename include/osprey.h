@@ -130,7 +130,8 @@ void osprey_destroy(osprey_ctx *ctx);
 
 /* Bytes of workspace osprey_draft_step needs for a batch of B sequences, chains
  * of K tokens, up to max_new extend rows per sequence and page tables of
- * max_pages_per_seq pages.  0 on bad arguments. */
+ * max_pages_per_seq pages.  It never falls as B grows: a workspace for B sequences
+ * serves smaller calls too.  0 on bad arguments. */
 size_t osprey_draft_workspace_bytes(const osprey_ctx *ctx, int B, int K, int max_new,
                                     int max_pages_per_seq);
 
@@ -237,7 +238,8 @@ int osprey_verify_tree(int B, int K, int topk, int V, int logits_dtype, const vo
                        const float *u_sample, int32_t *out_tokens, int32_t *n_accepted, int32_t *branch,
                        uint8_t *flags, int32_t *dev_status, void *stream);
 
-/* Bytes of workspace osprey_dflash_step needs.  0 on bad arguments. */
+/* Bytes of workspace osprey_dflash_step needs; it never falls as B grows.  0 on
+ * bad arguments. */
 size_t osprey_dflash_workspace_bytes(const osprey_ctx *ctx, int B, int block, int max_pages_per_seq);
 
 /* Block drafting with the EAGLE-style DFlash interface (Appendix, "EAGLE-Style

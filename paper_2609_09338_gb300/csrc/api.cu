@@ -239,8 +239,8 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     const long long R_ext = (long long)B * max_new;
     const long long R_lm = block ? R_ext : B;
     const int max_ctx = max_pages * D.P;
-    const int ns = std::max(attn_splits((int)R_ext, D.Hkv, max_ctx, ctx->sms),
-                            attn_splits(B, D.Hkv, max_ctx, ctx->sms));
+    // extend rows take at most the ranges of as many chain rows as there are sequences
+    const long long ranges = max_new * attn_ranges(B, D.Hkv, max_ctx, ctx->sms);
     const int lm_warps = lm_blocks(D.V, ctx->sms) * 8;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align256(off + bytes); return o; };
@@ -254,7 +254,7 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     size_t o_xe = take(4ull * R_ext * D.d), o_se = take(4ull * R_ext * D.d);
     size_t o_xc = take(4ull * B * D.d), o_sc = take(4ull * B * D.d);
     size_t o_q = take(4ull * R_ext * D.Hq * D.hd);
-    size_t o_ap = take(4ull * R_ext * D.Hq * ns * (D.hd + 2));
+    size_t o_ap = take(4ull * ranges * D.Hq * (D.hd + 2));
     size_t o_ao = take(4ull * R_ext * D.Hq * D.hd);
     size_t o_fh = take(4ull * R_ext * D.F);
     size_t o_ls = take(16ull * B * lm_warps);
@@ -262,32 +262,27 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
     size_t o_lsup = take(8ull * B * lmp.blocks * lmp.nsup);   // the streamed LM head's run statistics (rows <= 2)
     size_t o_lc = take(16ull * B * lmp.blocks);
     // tensor-core path: bf16 operand planes, QKV output, row-sampler partials
-    // (a step of more than TC_MAX_ROWS rows runs on the CUDA cores and needs none)
-    const long long re = R_ext <= TC_MAX_ROWS ? R_ext : 0, rc = B <= TC_MAX_ROWS ? B : 0;
-    auto plane_rows = [](long long r) { return std::max(tc_tiles(r, 1).rows(), tc_tiles(r, TC_BIG_K).rows()); };
-    const long long np = std::max(plane_rows(re), plane_rows(rc));
-    const long long npl = std::max({np, (long long)tc_tiles_lm(re).rows(), (long long)tc_tiles_lm(rc).rows()});
+    // (a step of more than TC_MAX_ROWS rows runs on the CUDA cores, its smaller calls do not)
+    const long long rt = std::min<long long>(R_ext, TC_MAX_ROWS);
+    const long long np = tc_plane_rows(rt), npl = std::max<long long>(np, tc_tiles_lm(rt).rows());
     const long long nqkv = (long long)(D.Hq + 2 * D.Hkv) * D.hd;
     const bool tcw = ctx->tc;
     size_t o_xq = take(tcw ? 2ull * TC_PLANES * np * 2 * D.d : 0), o_yq = take(tcw ? 4ull * np * nqkv : 0);
     size_t o_xo = take(tcw ? 2ull * TC_PLANES * np * D.Hq * D.hd : 0), o_xg = take(tcw ? 2ull * TC_PLANES * np * D.d : 0);
     size_t o_xh = take(tcw ? 2ull * TC_PLANES * np * D.F : 0), o_xl = take(tcw ? 2ull * TC_PLANES * npl * D.d : 0);
     const long long lm_nsub = (D.V + TC_LM_GROUP - 1) / TC_LM_GROUP;
-    size_t o_rp = take(tcw && R_lm <= TC_MAX_ROWS ? 16ull * R_lm * lm_nsub : 0);
-    // split-K partials: the largest nsplit x rows x outputs of the call's projections
+    size_t o_rp = take(tcw ? 16ull * std::min<long long>(R_lm, TC_MAX_ROWS) * lm_nsub : 0);
+    // split-K partials: the largest of the call's projections
     long long part = 0;
     if (tcw) {
-        for (const long long rows : {re, rc}) {
-            auto need = [&](int nout, int K_, bool always = false) {
-                const int ns = tc_nsplit(nout, K_, block ? TC_BLOCK_SPLITS : tc_tiles(rows, K_), ctx->sms);
-                if (ns > 1 || always) part = std::max(part, (long long)ns * rows * nout);
-            };
-            need(D.d, D.feat);
-            need((D.Hq + 2 * D.Hkv) * D.hd, 2 * D.d);
-            need(D.d, D.Hq * D.hd);
-            need(2 * D.F, D.d, true);   // gate/up: one GEMM whose partials always go through the buffer
-            need(D.d, D.F);
-        }
+        auto need = [&](int nout, int K_, bool always = false) {
+            part = std::max(part, tc_part_floats(nout, K_, rt, ctx->sms, block, always));
+        };
+        need(D.d, D.feat);
+        need((D.Hq + 2 * D.Hkv) * D.hd, 2 * D.d);
+        need(D.d, D.Hq * D.hd);
+        need(2 * D.F, D.d, true);   // gate/up: one GEMM whose partials always go through the buffer
+        need(D.d, D.F);
     }
     size_t o_tp = take(4ull * part);
     if (ws && base) {
@@ -321,7 +316,6 @@ static size_t draft_layout(const osprey_ctx *ctx, int B, int K, int max_new, int
         ws->n_counters = (int)n_counters;
         ws->tc_part = (float *)(p + o_tp);
         ws->tc_part_cap = part;
-        ws->n_splits_max = ns;
         ws->lm_warps_max = lm_warps;
     }
     (void)K;
@@ -1021,28 +1015,27 @@ extern "C" int osprey_draft_step_topk(osprey_ctx *ctx, const osprey_kv *kv, int 
 // ------------------------------------------------------------------ block drafting
 // Sequences are drafted in passes of at most TC_GROUP_ROWS block rows, whole groups
 // of block_group sequences each; a pass reads the weights once (its row tiles share
-// them through L2).  Workspace: the block-mode draft layout of one pass, then the
-// pass's token array [n][P], n_new [n] and broadcast features [n][P][feat_dim] bf16.
+// them through L2).  Workspace: a full pass's token array [n][P], n_new [n] and
+// broadcast features [n][P][feat_dim] bf16, then the block-mode draft layout, which a
+// smaller pass lays out anew inside a full one's.
 static int block_pass(int B, int P) {
     const int g = block_group(B, P), n = TC_GROUP_ROWS / P / g * g;
     return n < g ? g : (n < B ? n : B);
 }
 
-static size_t block_layout(const osprey_ctx *ctx, int n, int P, int max_pages, DraftWs *ws, void *base,
-                           int32_t **tok, int32_t **nnew, uint16_t **feats) {
-    size_t off = align256(draft_layout(ctx, n, 1, P, max_pages, ws, base, true));
-    const size_t o_t = off;
-    off = align256(off + 4ull * n * P);
-    const size_t o_n = off;
-    off = align256(off + 4ull * n);
-    const size_t o_f = off;
-    off = align256(off + 2ull * n * P * ctx->dim.feat);
-    if (base) {
-        *tok = (int32_t *)((char *)base + o_t);
-        *nnew = (int32_t *)((char *)base + o_n);
-        *feats = (uint16_t *)((char *)base + o_f);
-    }
-    return off;
+struct BlockIn {
+    size_t tok, nnew, feats, draft;   // offsets
+};
+static BlockIn block_inputs(const osprey_ctx *ctx, int n, int P) {
+    BlockIn o;
+    o.tok = 0;
+    o.nnew = align256(4ull * n * P);
+    o.feats = align256(o.nnew + 4ull * n);
+    o.draft = align256(o.feats + 2ull * n * P * ctx->dim.feat);
+    return o;
+}
+static size_t block_bytes(const osprey_ctx *ctx, int n, int P, int max_pages) {
+    return align256(block_inputs(ctx, n, P).draft + draft_layout(ctx, n, 1, P, max_pages, nullptr, nullptr, true));
 }
 
 static bool block_args_ok(const osprey_ctx *ctx, int B, int block, int max_pages) {
@@ -1053,7 +1046,7 @@ static bool block_args_ok(const osprey_ctx *ctx, int B, int block, int max_pages
 extern "C" size_t osprey_dflash_workspace_bytes(const osprey_ctx *ctx, int B, int block, int max_pages_per_seq) {
     if (!block_args_ok(ctx, B, block, max_pages_per_seq)) return 0;
     const int P = block - 1;
-    return block_layout(ctx, block_pass(B, P), P, max_pages_per_seq, nullptr, nullptr, nullptr, nullptr, nullptr);
+    return block_bytes(ctx, block_pass(B, P), P, max_pages_per_seq);
 }
 
 extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, int block, const int32_t *anchors,
@@ -1080,12 +1073,12 @@ extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, i
         return fail(OSPREY_ERR_INVALID_ARG, "feats and workspace must be 16-byte aligned");
     const int P = block - 1, G = block_pass(B, P);
     const Dims &D = ctx->dim;
-    DraftWs ws{};
-    int32_t *tok = nullptr, *nnew = nullptr;
-    uint16_t *frep = nullptr;
-    const size_t need = block_layout(ctx, G, P, kv->max_pages_per_seq, &ws, workspace, &tok, &nnew, &frep);
+    const size_t need = block_bytes(ctx, G, P, kv->max_pages_per_seq);
     if (workspace_bytes < need)
         return fail(OSPREY_ERR_CAPACITY, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
+    const BlockIn in = block_inputs(ctx, G, P);
+    int32_t *tok = (int32_t *)((char *)workspace + in.tok), *nnew = (int32_t *)((char *)workspace + in.nnew);
+    uint16_t *frep = (uint16_t *)((char *)workspace + in.feats);
     cudaStream_t s = (cudaStream_t)stream;
     for (int b0 = 0; b0 < B; b0 += G) {
         const int n = B - b0 < G ? B - b0 : G;
@@ -1100,8 +1093,9 @@ extern "C" int osprey_dflash_step(osprey_ctx *ctx, const osprey_kv *kv, int B, i
         const int rc = draft_step_impl(ctx, &kg, n, 1, P, nnew, tok, frep, temperature, u_draft ? u_draft + o : nullptr,
                                        draft_tokens + o, draft_qx ? draft_qx + o : nullptr,
                                        draft_stats ? draft_stats + 2 * o : nullptr,
-                                       draft_logits ? draft_logits + o * D.V : nullptr, nullptr, workspace,
-                                       workspace_bytes, dev_status, stream, true);
+                                       draft_logits ? draft_logits + o * D.V : nullptr, nullptr,
+                                       (char *)workspace + in.draft, workspace_bytes - in.draft, dev_status, stream,
+                                       true);
         if (rc != OSPREY_OK) return rc;
     }
     return OSPREY_OK;

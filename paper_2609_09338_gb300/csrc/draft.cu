@@ -27,7 +27,6 @@ namespace osp {
 constexpr int GT = 256;          // threads per GEMV / LM-head block
 constexpr int GW = GT / 32;      // warps per block
 constexpr int AT = 128;          // threads per attention block
-constexpr int ATTN_MAX_SPLITS = 128;
 
 // ---------------------------------------------------------------------------
 // One warp computes TR dot products of length Kd (bf16 weights streamed from
@@ -943,17 +942,6 @@ __global__ void __launch_bounds__(128) prepare_kernel(const PrepArgs a) {
 
 // Splits per (row, KV head): about four blocks per SM over the whole grid, at
 // most 1024 keys per block, at least 64 keys (one page per warp) per block.
-int attn_splits(int R, int Hkv, int max_ctx, int sms) {
-    auto cdiv = [](long long x, long long y) { return (int)((x + y - 1) / y); };
-    int want = cdiv(4LL * sms, (long long)R * Hkv);
-    int by_len = cdiv(max_ctx, 1024);
-    int s = want > by_len ? want : by_len;
-    int cap = cdiv(max_ctx, 64);
-    if (s > cap) s = cap;
-    if (s > ATTN_MAX_SPLITS) s = ATTN_MAX_SPLITS;
-    return s < 1 ? 1 : s;
-}
-
 int attn_split_len(int max_ctx, int n_splits) {
     int len = (max_ctx + n_splits - 1) / n_splits;
     return (len + 15) / 16 * 16;

@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "osprey.h"
+#include "sizes.h"
 
 namespace osp {
 
@@ -45,7 +46,7 @@ struct DraftWs {
     int *rs_ticket;                        // [B]
     int *counters;                         // attn_ticket .. rs_ticket: one contiguous block
     int n_counters;
-    int n_splits_max, lm_warps_max;
+    int lm_warps_max;
 };
 
 // Which rows a launch works on: extend rows (step 0, rows_per_seq = max_new,
@@ -268,7 +269,6 @@ cudaError_t launch_attn_rows(const AttnArgs &a, int B, int mtiles, cudaStream_t 
 int attn_cluster_size(const Dims &D);
 cudaError_t launch_attn_cluster(const AttnArgs &a, int cs, cudaStream_t s);
 cudaError_t launch_lm(const LmArgs &a, int rg, int blocks, cudaStream_t s);
-int attn_splits(int R, int Hkv, int max_ctx, int sms);
 int attn_split_len(int max_ctx, int n_splits);
 int lm_blocks(int V, int sms);
 size_t gemv_smem(GemvMode mode, const Dims &d, int rg);

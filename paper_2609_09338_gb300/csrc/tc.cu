@@ -1365,22 +1365,6 @@ static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtens
     return pdl_launch(tc_kernel<EPI, NA, BPS>, dim3(grid), dim3(TC_THREADS), smem, s, wa, wb, xm, a, nst);
 }
 
-// k-ranges per output tile so that tiles x ranges fill the CTA slots (few
-// output tiles, long K: the layer projections); 1 for wide outputs.
-#ifndef OSP_TC_MIN_KB
-#define OSP_TC_MIN_KB 1   // k-blocks (of 64) per range at least: fewer, longer ranges write fewer partials
-#endif
-int tc_nsplit(int nout, int K, const TcTiles &t, int sms) {
-    const int tiles = (nout + 127) / 128 * t.nrt, nkb = K / 64;
-    // at most one item per CTA slot: one item more than the slots would take two
-    // item times for barely more than one wave of work
-    int want = t.bps * sms / tiles;
-    if (want < 1) want = 1;
-    if (want > nkb / OSP_TC_MIN_KB) want = nkb / OSP_TC_MIN_KB > 1 ? nkb / OSP_TC_MIN_KB : 1;
-    const int kbps = (nkb + want - 1) / want;
-    return (nkb + kbps - 1) / kbps;
-}
-
 cudaError_t launch_tc(const TcArgs &a_in, const CUtensorMap &wa, const CUtensorMap &xm, int sms, cudaStream_t s) {
     TcArgs a = a_in;
     a.nout_a = a.nout;

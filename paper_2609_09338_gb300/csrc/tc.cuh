@@ -27,6 +27,7 @@
 
 #include "draft.cuh"
 #include "internal.h"
+#include "sizes.h"
 
 namespace osp {
 
@@ -45,44 +46,7 @@ constexpr int TC_LM_PLANES = 2;
 // logits were float32 dot products before they ran on the tensor cores, and two
 // planes would put q(token) 1e-4 off at logits of 40 (three: 1e-6).
 
-constexpr int TC_TILE_ROWS = 80;   // activation rows per tile: three accumulators fit a CTA's 256 TMEM columns
-constexpr int TC_BIG_ROWS = 128;   // rows per tile of a larger GEMM ...
-constexpr int TC_BIG_K = 4096;     // ... whose reduction is at least this long
-constexpr int TC_MAX_ROWS = 4096;  // rows of a call on the tensor cores (beyond: the CUDA-core GEMV, whose workspace is smaller)
-constexpr int TC_GROUP_ROWS = 512; // rows of one pass of block drafting
 constexpr int TC_PLANES = 3;       // bf16 planes of a float32 operand
-
-// A GEMM's rows as equal tiles (the MMA's N, a multiple of 16).  Up to TC_TILE_ROWS
-// keep two CTAs per SM (two accumulators of 80 columns and one of the small planes
-// in 256 TMEM columns, two stages of three planes in 112 KB).  More rows: with a
-// reduction of TC_BIG_K or more, tiles of up to TC_BIG_ROWS and one CTA per SM
-// (four accumulators of 128 columns, three stages): 120 rows at d 4096, gate and up
-// 110 -> 88 us, the O and down projections 39 -> 34; with a shorter one, an even
-// number of the small tiles: start and epilogue weigh more there, and two CTAs
-// overlap them (96 rows, d 1024: 11.7 us a launch against 12.7).
-struct TcTiles {
-    int nrt, npad;     // row tiles, rows per tile
-    int bps;           // CTAs per SM
-    __host__ __device__ int rows() const { return nrt * npad; }   // rows of an operand plane
-};
-inline TcTiles tc_tiles_of(long long rows, int most, int even, int bps) {
-    TcTiles t;
-    t.nrt = rows <= most ? 1 : (int)((rows + most - 1) / most + even - 1) / even * even;
-    t.npad = (int)(((rows + t.nrt - 1) / t.nrt + 15) / 16 * 16);
-    t.bps = bps;
-    return t;
-}
-inline TcTiles tc_tiles(long long rows, int K) {
-    return rows > TC_TILE_ROWS && K >= TC_BIG_K ? tc_tiles_of(rows, TC_BIG_ROWS, 1, 1)
-                                                : tc_tiles_of(rows, TC_TILE_ROWS, 2, 2);
-}
-// The LM head keeps two CTAs per SM at any number of rows, whose epilogues (the
-// sampling partials are most of an item's time) run beside each other's MMAs:
-// 96 rows, V 151936, d 1024, in two tiles of 48 132 us, in one of 96 161.  An even
-// number of tiles: pairs share the weights that they load.
-inline TcTiles tc_tiles_lm(long long rows) { return tc_tiles_of(rows, TC_TILE_ROWS, 2, 2); }
-// k-ranges of block drafting's GEMMs: those of one row tile, whatever the rows
-constexpr TcTiles TC_BLOCK_SPLITS{1, TC_TILE_ROWS, 2};
 
 struct TcArgs {
     int epi;           // TcEpi
@@ -143,14 +107,12 @@ bool tc_encode_weight(CUtensorMap *m, const void *w, int rows, int K);
 bool tc_encode_operand(CUtensorMap *m, const void *x, int planes, int prows, int npad, int K);
 // a single bf16 plane of `rows` rows read in place (rows past `rows` read as zero)
 bool tc_encode_rows(CUtensorMap *m, const void *x, int rows, int npad, int K);
-size_t tc_smem_bytes(int npad, int planes, int na);
 cudaError_t tc_set_attributes();
 // SwiGLU runs as one GEMM over the gate rows (map wa) and the up rows (map wb),
 // nout = 2 nout_a; its partials always go to `part`, and the reduction forms
 // silu(gate) * up.  Outputs narrower than the CTA slots are split along K
 // (tc_nsplit ranges per 128-feature, npad-row tile); the float32 partials are then summed
 // in range order by a reduction kernel that applies the epilogue.
-int tc_nsplit(int nout, int K, const TcTiles &t, int sms);
 cudaError_t launch_tc(const TcArgs &a, const CUtensorMap &wa, const CUtensorMap &xm, int sms, cudaStream_t s);
 // *planes_done (when given) tells whether the reduction did the follow-up work:
 // wrote the pl_* planes (TC_RESID), or RoPE and the K/V write of `rope`

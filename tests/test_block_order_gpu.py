@@ -89,3 +89,34 @@ def test_groups_do_not_change_one_another(block, T):
         own = propose(c, T, seqs)
         for k in own:
             np.testing.assert_array_equal(whole[k][seqs], own[k], err_msg=f"{k} of group {b0}")
+
+
+@pytest.mark.parametrize("B,block", [(63, 16), (66, 16), (160, 4), (13, 65)])
+def test_passes_do_not_change_one_another(B, block):
+    """Calls of more than 512 rows run in several passes over one workspace, the last one smaller: every group's results
+    are those of a call of its own."""
+    P = block - 1
+    group = 80 // P
+    full = 512 // P // group * group
+    assert B > full and B % full, "a smaller last pass"
+    c = make(TINY, np.random.default_rng(B).integers(1, 60, size=B), block, 17)
+    whole = propose(c, 1.0)
+    last = (B - 1) // group * group
+    for b0 in {0, full - group, (B // full) * full, last}:
+        seqs = list(range(b0, min(B, b0 + group)))
+        own = propose(c, 1.0, seqs)
+        for k in own:
+            np.testing.assert_array_equal(whole[k][seqs], own[k], err_msg=f"{k} of group {b0}")
+
+
+def test_workspaces_grow_with_the_batch():
+    """A workspace made for some batch is enough for every smaller one."""
+    from paper_2609_09338_gb300 import binding as ob
+    for shape in (TINY, replace(TINY, d_model=1024, n_q_heads=8, ffn_dim=4096, feat_dim=3072)):
+        ctx = ob.osprey_create(shape, ob.upload_weights(syn.make_weights(shape, 5)))
+        for max_new, max_pages in ((1, 4), (3, 40), (8, 300)):
+            sizes = [ob.osprey_draft_workspace_bytes(ctx, B, 4, max_new, max_pages) for B in [*range(1, 700), 4095, 4097]]
+            assert sizes == sorted(sizes), (max_new, max_pages)
+        for block in (4, 16, 24, 81):
+            sizes = [ob.osprey_dflash_workspace_bytes(ctx, B, block, 40) for B in range(1, 200)]
+            assert sizes == sorted(sizes), block
