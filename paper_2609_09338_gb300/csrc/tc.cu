@@ -50,14 +50,24 @@ __host__ __device__ constexpr uint32_t tc_tmem_cols(int bps) { return 512 / bps;
 // its last place at every step instead of rounding to nearest, so its error
 // grows with the steps that add to a large value.  The planes after the first,
 // 2^-8 and 2^-16 of it, therefore have an accumulator of their own, and calls of
-// more rows than a tile, which come out as accurate as the CUDA-core GEMV, take
+// more rows than a tile, whose rows the CUDA-core GEMV sums in float32, take
 // segments of 2 k-blocks: 8 steps at full size instead of 96.  Measured
 // against float64 on 96 sequences, d 1024 (logits, cached bf16 K values that
 // round otherwise; us a call): 8 k-blocks, one accumulator 1.9e-6, 1160, 4250;
 // 2 k-blocks, one accumulator 4.9e-7, 370, 5140; 4 k-blocks, two 2.8e-7, 220,
 // 3780; 2 k-blocks, two 1.7e-7, 170, 4020; the GEMV 1.6e-7, 220, 34500.
+// The LM head of such a batch takes segments of 1: logits 1.5e-7 off instead of
+// 1.7e-7 (the GEMV's 1.6e-7), for 3100 us a call instead of 2864.  What is left is
+// a bias of the leading logit, of one sign in every step: -2.2e-6 at 46 (segments
+// of 2: -5.5e-6), half a unit in the last place, where the GEMV has none; rms 4.3e-6
+// against 2.7e-6.
+// Block drafting keeps one accumulator, segments of 8 and the LM head's two planes
+// at every number of rows (TcArgs::block): 2.4e-5 at d 4096.
 #ifndef OSP_TC_SEGKB_FINE
 #define OSP_TC_SEGKB_FINE 2
+#endif
+#ifndef OSP_TC_SEGKB_LM
+#define OSP_TC_SEGKB_LM 1   // ... of its LM head
 #endif
 #ifndef OSP_TC_LM_NA
 #define OSP_TC_LM_NA 2   // LM head: weight tiles per stage that share one operand stage
@@ -1393,7 +1403,7 @@ cudaError_t launch_tc2(const TcArgs &a_in, const CUtensorMap &wa, const CUtensor
     if (a.epi == TC_GLU && (long long)a.nsplit * a.R * a.nout > a.part_cap) return cudaErrorInvalidValue;
     a.kbps = (nkb + a.nsplit - 1) / a.nsplit;
     a.sep = a.planes > 1 && !a.block;   // (0.1 % of a call, for a third of the accumulators' error)
-    a.segkb = a.fine ? OSP_TC_SEGKB_FINE : OSP_TC_SEGKB;
+    a.segkb = !a.fine ? OSP_TC_SEGKB : lm ? OSP_TC_SEGKB_LM : OSP_TC_SEGKB_FINE;
     const int bps = a.bps, tmem_cols = tc_tmem_cols(bps);
     // the LM head takes OSP_TC_LM_NA weight tiles per stage when two stages fit
     // and the double-buffered accumulators fit TMEM in one segment (the LM head's

@@ -15,8 +15,8 @@
 // inputs such as the target features use a single plane).  Two planes (16 bits)
 // were not enough: attention over thousands of cached keys turns a 1e-5 relative
 // error in q into logit errors two orders above the float32 path's.  A reduction
-// is accumulated in segments (a fresh TMEM accumulator each, of 8 k-blocks, or 2
-// where the rows were float32 dot products before) whose float32 sum the epilogue
+// is accumulated in segments (a fresh TMEM accumulator each, of 8 k-blocks, or 2 or
+// 1 where the rows were float32 dot products before) whose float32 sum the epilogue
 // keeps, and the planes after the first have an accumulator of their own: a
 // tensor-core accumulator truncates at every step.
 #pragma once
