@@ -1110,11 +1110,20 @@ __global__ void __launch_bounds__(PK_THREADS) lm_pick_kernel(const LmPickArgs a)
                 }
             }
             __syncthreads();
+            // Batches whose logits were float32 sums before (three planes): M is off by a few
+            // 1e-6 against the recomputed logits, and so would q be (1 + 7e-6 for a token of
+            // all the mass).  The group is scaled to its partial, which M and S come from.
+            const bool scaled = a.npl > TC_LM_PLANES;
+            const float4 part = scaled ? __ldcg(pp + s_grp[c]) : make_float4(0.f, 0.f, 0.f, 0.f);
             pk_group_logits(a, hrow, s_grp + c, 1, s_z);
             __syncthreads();
             if (warp == 0) {
                 const int id = s_grp[c] * TC_LM_GROUP + lane;
-                const float e = id < D.V ? __expf(s_z[lane] * invT - M) : 0.f;
+                float e = id < D.V ? __expf(s_z[lane] * invT - M) : 0.f;
+                if (scaled) {
+                    const float mass = weight(part.x, part.y), sum = warp_sum(e);
+                    if (mass > 0.f && sum > 0.f) e *= mass / sum;
+                }
                 const float cum = s_before + warp_incl_scan(e);
                 const unsigned hit = __ballot_sync(0xffffffffu, e > 0.f && target < cum);
                 const unsigned pos = __ballot_sync(0xffffffffu, e > 0.f);

@@ -19,8 +19,8 @@ from paper_2609_09338_gb300.workloads import TINY  # noqa: E402
 from test_draft_gpu import _built, _dev  # noqa: E402,F401
 
 
-@pytest.mark.parametrize("B", [81, 96, 130])
-def test_leading_logits_are_not_biased(B):
+def draft(B, T):
+    """A one-step call of B sequences whose leading logits are 46: its outputs, and its logits in float64."""
     from paper_2609_09338_gb300.binding import to_device_bf16
     from paper_2609_09338_gb300.session import DraftSession
     shape = replace(TINY, d_model=1024, vocab=8192)
@@ -28,9 +28,8 @@ def test_leading_logits_are_not_biased(B):
     w = syn.make_weights(shape, 41)
     rng = np.random.default_rng(42)
     embed = widen(w["embed"]) * np.float32(50)
-    succ = rng.permutation(V)
     w["embed"] = syn.bf16_bits(embed)
-    w["lm_head"] = syn.bf16_bits(widen(w["lm_head"]) + np.float32(47 / d) * embed[succ])
+    w["lm_head"] = syn.bf16_bits(widen(w["lm_head"]) + np.float32(47 / d) * embed[rng.permutation(V)])
     ctx = rng.integers(0, 40, size=B).astype(np.int32)
     kv = syn.make_kv_prefix(shape, ctx, 2, 43)
     di = syn.make_draft_inputs(shape, B, 1, 1, 44)
@@ -39,7 +38,7 @@ def test_leading_logits_are_not_biased(B):
     n0 = sess.kv.seq_len.clone()
     out, kept = sess.draft_buffers(with_logits=True), sess.draft_buffers()
     hidden = torch.zeros((B, 1, d), device="cuda")
-    args = (_dev(di["n_new"]), _dev(di["tokens"]), to_device_bf16(di["feats"]), 0.0, _dev(di["u_draft"]))
+    args = (_dev(di["n_new"]), _dev(di["tokens"]), to_device_bf16(di["feats"]), T, _dev(di["u_draft"]))
     sess.draft(*args, out)
     sess.kv.seq_len.copy_(n0)
     sess.draft_hidden(*args, kept, hidden)
@@ -48,12 +47,29 @@ def test_leading_logits_are_not_biased(B):
     x = hidden[:, 0].double()
     n = x * torch.rsqrt(x.square().mean(-1, keepdim=True) + shape.rms_eps) * _dev(widen(w["final_norm"])).double()
     z = n @ _dev(widen(w["lm_head"])).double().t()
+    assert 44 < float(z.max(-1).values.mean()) < 48
+    return out, z
+
+
+@pytest.mark.parametrize("B", [81, 96, 130])
+def test_leading_logits_are_not_biased(B):
+    out, z = draft(B, 0.0)
     M, at = z.max(-1)
-    assert 44 < float(M.mean()) < 48
-    got = out["draft_logits"][:, 0]
+    got = out["draft_logits"][:, 0].double()
     assert torch.equal(out["draft_tokens"][:, 0].long(), at)
-    err = torch.gather(got.double(), 1, at[:, None])[:, 0] - M
-    rms = float((got.double() - z).square().mean().sqrt() / z.square().mean().sqrt())
-    print(f"B {B}: bias {float(err.mean()):.2e}, rms {float(err.square().mean().sqrt()):.2e}, all logits {rms:.2e}")
-    assert abs(float(err.mean())) < 1.4 * 16 * 4 * 2.0 ** -24
+    bias = float((torch.gather(got, 1, at[:, None])[:, 0] - M).mean())
+    rms = float((got - z).square().mean().sqrt() / z.square().mean().sqrt())
+    assert abs(bias) < 1.4 * 16 * 4 * 2.0 ** -24
     assert rms < 1.6e-7   # the CUDA-core GEMV's
+
+
+@pytest.mark.parametrize("B", [81, 130])
+def test_probabilities_are_those_of_the_logits(B):
+    """q(token) = exp(z / T - M) / S with z, M and S of the same sums: a token of nearly all the mass has q = 1 up to the
+    rounding of its group's sum, its scaling and the division (a few 2^-24), not 1 + exp(the bias of M)."""
+    out, z = draft(B, 0.7)
+    tok = out["draft_tokens"][:, 0].long()
+    lead = tok == z.argmax(-1)
+    assert int(lead.sum()) > B // 2
+    q = torch.gather(torch.softmax(z / 0.7, -1), 1, tok[:, None])[:, 0]
+    assert float((out["draft_qx"][:, 0].double() / q - 1).abs()[lead].max()) < 8 * 2.0 ** -24
