@@ -110,13 +110,14 @@ const char *osprey_last_error(void);
  * The context picks the kernels a draft call uses:
  *   rows <= 2 per chain step: TMA-streamed GEMVs (weights read once per step);
  *   3..4096 rows: tcgen05 tensor-core GEMMs in tiles of up to 128 rows, float32
- *     activations split into three bf16 planes (24 mantissa bits) so results
- *     match the GEMV path's (the LM head's operand of up to 80 sequences into
- *     two planes, 16 bits: its logits differ from the GEMV path's by rounding
- *     of the operand's last bits);
+ *     activations split into three bf16 planes (24 mantissa bits), their sums
+ *     within a few 1e-7 of the GEMV path's (the LM head's operand of up to 80
+ *     sequences into two planes, 16 bits: its logits are 3e-6 to 6e-6 off);
  *   more rows: CUDA-core GEMVs, eight rows at a time;
  *   attention: clusters merged on chip while they fit one wave, else global
- *     partials.
+ *     partials; the extend rows of larger calls (rows x KV heads of two per SM
+ *     and more) 16 (row, head) queries at a time on tensor cores, q and the
+ *     weights split into three bf16 planes (block drafting row by row).
  * Two environment variables, read here, select the alternatives for testing:
  * OSPREY_TC=0 (CUDA-core GEMVs for batched rows) and OSPREY_ATTN_CLUSTER=0
  * (global-partials attention).  Two more select fused batch-1 chain steps,
@@ -229,8 +230,8 @@ int osprey_draft_step_topk(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
  *   at the last accepted depth, -1 if none), flags [B][K+1] (bit 3: a residual
  *   without float32 mass, p sampled instead; bit 4: the draw clamped to the
  *   last id with weight).
- * No workspace: one block per sequence keeps its walk on chip; rows off the
- * walked path are never read.  V <= 2^20.
+ * No workspace: a cluster of 8 blocks per sequence keeps its walk on chip; rows off
+ * the walked path are at most prefetched.  V <= 2^20.
  * Device errors: INVALID_ARG for a candidate outside [0, V) (that sequence gets
  * n_accepted 0 and out_tokens -1). */
 int osprey_verify_tree(int B, int K, int topk, int V, int logits_dtype, const void *target_logits,

@@ -1182,8 +1182,11 @@ extern "C" int osprey_verify_tree(int B, int K, int topk, int V, int logits_dtyp
 // Workspace: the verify layout (counters, partials, decisions, chunk sums), then
 // for one group of up to TC_TILE_ROWS sequences the operand planes of their
 // decision rows [TC_PLANES][npad][d] bf16, the
-// recomputed decision-row logits [rows][V] float (the draft step's LM-head GEMM:
-// the same operand planes, unsplit, so the rows come out the same).
+// recomputed decision-row logits [rows][V] float by the draft step's LM-head GEMM:
+// for 3 to TC_TILE_ROWS sequences the same operand planes, tiles and segments, so the
+// same logits bit for bit.  A draft of fewer sequences (streamed GEMV) or of more
+// (three planes, shorter segments) has float32 logits; two planes put q 1e-4 off
+// those at logits of 40.
 struct HiddenWs {
     uint16_t *planes;
     float *z;
@@ -1305,7 +1308,7 @@ extern "C" int osprey_verify_hidden(osprey_ctx *ctx, int B, int K, int logits_dt
         ta.y = hw.z;
         ta.x = hw.z;
         ta.ldy = V;
-        ta.status = dev_status;   // unsplit, like the draft step's LM head: the same logits bit for bit
+        ta.status = dev_status;   // unsplit, like the draft step's LM head
         if ((e = launch_tc(ta, ctx->tm_lm, xm, ctx->sms, s)) != cudaSuccess) return cuda_fail(e, "decision-row lm head");
         // 4. the emitted token of each sequence of the group
         if ((e = launch_verify_hidden_sample(a, b0, n, s)) != cudaSuccess) return cuda_fail(e, "verify sample launch");

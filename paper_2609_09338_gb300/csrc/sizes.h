@@ -43,8 +43,8 @@ inline TcTiles tc_tiles(long long rows, int K) {
 }
 // The LM head keeps two CTAs per SM at any number of rows, whose epilogues (the
 // sampling partials are most of an item's time) run beside each other's MMAs:
-// 96 rows, V 151936, d 1024, in two tiles of 48 132 us, in one of 96 161.  An even
-// number of tiles: pairs share the weights that they load.
+// 96 rows, V 151936, d 1024, in two tiles of 48 132 us, in one of 96 161 (both with
+// segments of 2 k-blocks).  An even number of tiles: pairs share weights through L2.
 inline TcTiles tc_tiles_lm(long long rows) { return tc_tiles_of(rows, TC_TILE_ROWS, 2, 2); }
 // k-ranges of block drafting's GEMMs: those of one row tile, whatever the rows
 constexpr TcTiles TC_BLOCK_SPLITS{1, TC_TILE_ROWS, 2};

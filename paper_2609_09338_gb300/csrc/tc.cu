@@ -35,9 +35,9 @@ constexpr int TC_THREADS = 192;
 constexpr int TC_ABYTES = 128 * 128;    // weight tile: 128 rows x 64 bf16
 constexpr int TC_MAXST = 8;
 // Two CTAs per SM are two TMA producers, MMA chains and epilogues; one has all of
-// TMEM and shared memory, and tiles of up to TC_BIG_ROWS rows (tc_tiles).  An MMA reads its 4 KB of weights from shared memory however
-// many rows it multiplies (32 cycles; 16 rows more take 4), so 128 rows at once
-// cost two thirds of twice 64.
+// TMEM and shared memory, and tiles of up to TC_BIG_ROWS rows (tc_tiles).  An MMA
+// reads its 4 KB of weights from shared memory however many rows it multiplies (32
+// cycles; 16 rows more take 4), so 128 rows at once cost two thirds of twice 64.
 // Two CTAs, the system's share and the static part fit 228 KB: 100 KB left the
 // third stage of 48 rows and the fifth of 16 out (16 sequences, 2 layers of d
 // 2048: 1992 us a call, with it 1970).
@@ -1374,7 +1374,7 @@ static cudaError_t tc_launch(int grid, size_t smem, cudaStream_t s, const CUtens
                              const CUtensorMap &xm, const TcArgs &a, int nst) {
     // opted into its shared memory, and so loaded, at its first launch: with every
     // instance loaded beside them, calls that use none (one sequence, batch-1 weights
-    // in L2) took 679 us instead of 672
+    // in L2) took 678 us instead of 673
     static std::atomic<int> done[kMaxDevices];
     const cudaError_t es = once_per_device(done, [] {
         return cudaFuncSetAttribute(tc_kernel<EPI, NA, BPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,

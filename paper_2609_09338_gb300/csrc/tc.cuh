@@ -67,7 +67,7 @@ struct TcArgs {
     // head's segments by groups of TC_TILE_ROWS rows, runs and merges of the sampler.
     bool block;
     bool whole;        // TC_LM_BLOCK: the whole reduction in one segment
-    bool wide;         // TC_STORE of the LM head: the LM head's tiles, so the same sums bit for bit
+    bool wide;         // TC_STORE of the LM head: the LM head's tiles and segments at these rows
     float *y;          // TC_STORE: [R][ldy] float32 output
     int ldy;
     float *x;          // TC_RESID: [R][ldy] float32, +=

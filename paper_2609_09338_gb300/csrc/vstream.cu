@@ -32,7 +32,7 @@
 // Logits-free form (HID): vs_stats reads the target rows only and the decision
 // takes q_i(x_i) and (M, log S) from the draft step; vs_sample takes a group's
 // draft rows from `zrec` (float32 whatever the target's type).  V 200064, B 64,
-// K 8, bf16: 165 us a call, of which the target's 230 MB take 55; with unstreamed
+// K 8, bf16: 162 us a call, of which the target's 230 MB take 55; with unstreamed
 // kernels for the rows and two launches for the decision rows' operand 238.
 // Both kernels are launched as programmatic dependents: barrier set-up overlaps
 // the previous kernel's tail, and every global read follows griddepcontrol.wait.

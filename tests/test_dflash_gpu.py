@@ -107,9 +107,17 @@ def test_block_matches_oracle(T):
 
 
 def test_blocks_in_several_tensor_core_groups():
-    """6 sequences x 16 proposals = 96 rows: one group of 5 sequences (80 rows),
-    then one of 1, each a pass over the weights."""
-    checked, total = check_block(run_block(TINY, [30, 1, 64, 17, 5, 90], 17, 0.0, 83), seqs=[0, 4, 5])
+    """33 sequences x 16 proposals = 528 rows: groups of 5 sequences (80 rows), six of
+    them a pass over the weights, then a second pass of one group of 3."""
+    ctx = np.random.default_rng(83).integers(1, 90, size=33)
+    checked, total = check_block(run_block(TINY, ctx, 17, 0.0, 83), seqs=[0, 4, 5, 29, 30, 32])
+    assert checked >= total // 2
+
+
+def test_sampled_blocks_of_several_groups():
+    """8 sequences x 15 proposals = 120 rows, sampled: two groups, two row tiles.  Ids are
+    the oracle's wherever u lies farther from a boundary than the logits' error moves it."""
+    checked, total = check_block(run_block(TINY, [30, 1, 64, 17, 5, 90, 200, 41], 16, 1.0, 85, peaked=True))
     assert checked >= total // 2
 
 

@@ -46,7 +46,8 @@ def test_wide_rows(d):
 
 
 def test_block_rows_beyond_a_tile():
-    """Ten blocks of 11 positions (100 rows, two row tiles in one group) give what each gives in a call of its own."""
+    """Ten blocks of 11 positions (100 rows: two row tiles, groups of 8 and 2 sequences) give what each gives in a call of
+    its own."""
     from paper_2609_09338_gb300.binding import to_device_bf16
     from paper_2609_09338_gb300.session import DflashSession
     B, block = 10, 11
@@ -74,8 +75,8 @@ def test_block_rows_beyond_a_tile():
     tok, z = propose(list(range(B)))
     for b in (0, 4, 8, 9):
         t1, z1 = propose([b])
-        # the split of the reductions differs: float32 sums in another order, and a cached bf16 row may round the
-        # other way (2^-8 of a key, attended with weight <= 1)
+        # the key ranges of the attention differ with a group's rows: float32 sums in another order, and a cached
+        # bf16 row may round the other way (2^-8 of a key, attended with weight <= 1)
         assert np.abs(z[b] - z1[0]).max() < 2e-2
         gap = np.sort(z1[0], -1)
         sure = gap[:, -1] - gap[:, -2] > 4e-2
