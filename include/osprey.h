@@ -115,9 +115,8 @@ const char *osprey_last_error(void);
  *     sequences into two planes, 16 bits: its logits are 3e-6 to 6e-6 off);
  *   more rows: CUDA-core GEMVs, eight rows at a time;
  *   attention: clusters merged on chip while they fit one wave, else global
- *     partials; the extend rows of larger calls (rows x KV heads of two per SM
- *     and more) 16 (row, head) queries at a time on tensor cores, q and the
- *     weights split into three bf16 planes (block drafting row by row).
+ *     partials; many extend rows over long contexts 16 (row, head) queries at a
+ *     time on tensor cores, q and the weights split into three bf16 planes.
  * Two environment variables, read here, select the alternatives for testing:
  * OSPREY_TC=0 (CUDA-core GEMVs for batched rows) and OSPREY_ATTN_CLUSTER=0
  * (global-partials attention).  Two more select fused batch-1 chain steps,

@@ -616,12 +616,8 @@ static int draft_step_impl(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
         // (one block per SM); beyond that the global-partials kernel keeps more
         // loads in flight
         auto clusters = [&](int rows) { return ctx->attn_cs && (long long)rows * D.Hkv * ctx->attn_cs <= ctx->sms; };
-        // several rows a sequence share their keys: one pass over them for 16 queries
-        // (row, head) instead of one a row (96 x 8 rows: 356 us a launch against 592;
-        // 16 x 6 rows: 99 against 141).  Below one wave of the decode
-        // kernel's blocks, which then have every page in flight at once, it is the
-        // slower one (1 x 8 rows at 2048 keys: 51 us against 24).
-        const int mt = !block && !clusters(R) && rows_per_seq > 1 && (long long)R * D.Hkv >= 2 * ctx->sms
+        // several rows a sequence share their keys where that pays
+        const int mt = !block && !clusters(R) && attn_rows_pays(R, D.Hq, D.Hkv, rows_per_seq, max_ctx)
                            ? attn_rows_tiles(D, rows_per_seq) : 0;
         auto attention = [&](const AttnArgs &all) {
             cudaError_t e2 = cudaSuccess;

@@ -98,4 +98,19 @@ inline long long attn_ranges(long long R, int Hkv, int max_ctx, int sms) {
     return std::max(R, std::min(R * cap, std::max(R * by_len, (4LL * sms + Hkv * R - 1) / Hkv)));
 }
 
+// Whether a sequence's extend rows share one pass over their keys (attn_rows_kernel,
+// 16 (row, head) queries a block) instead of streaming them once a row.  A launch of
+// it takes 25 to 35 us more to start, split and merge; the row-by-row kernel takes
+// about 15 us a million of (G + 2) x rows x KV heads x keys.  Measured over 1..32
+// sequences of 2, 4 and 8 rows, 256..16384 keys, G 2 and 4 (582 calls): the two cross
+// at 4.2 to 5 million, and with less than half a tile of queries the shared pass never
+// wins.  With the line at 6 million no call is 2 % slower than row by row, and all
+// together are 0.2 % off the better of the two; a line by rows x KV heads alone was
+// 3.2 % off it and up to 17 % slower, at 256 to 1024 keys.  The keys are the page
+// table's capacity.
+inline bool attn_rows_pays(long long R, int Hq, int Hkv, int rows_per_seq, int max_ctx) {
+    const int G = Hq / Hkv;
+    return rows_per_seq > 1 && rows_per_seq * G >= 8 && R * Hkv * (G + 2) * max_ctx >= 6000000LL;
+}
+
 }  // namespace osp
