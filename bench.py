@@ -360,14 +360,15 @@ def lm_head_label(B, block=False):
     """The LM-head launches the probes bracket, by the number of rows (the draft
     step's kernel selection)."""
     if block:
-        return ("tc_kernel<LM> + lm_pick_kernel over every block row (tcgen05 LM head with per-32-id sampling "
+        return ("tc_kernel<LM_BLOCK> + block_pick_kernel over every block row (tcgen05 LM head with per-32-id sampling "
                 "partials in its epilogue, then the pick; the operand planes come from the last down projection)")
     if B <= 2:
         return "stream_kernel<LM> (final RMSNorm + TMA-streamed LM-head GEMV + on-chip sampling)"
     if B <= 80:
         return ("tc_kernel<LM> + lm_pick_kernel (tcgen05 LM head, two weight tiles per stage, per-32-id sampling "
                 "partials in its epilogue, then the pick)")
-    return "lm_head_kernel (CUDA-core LM head + on-chip sampling)"
+    return ("tc_kernel<LM> + lm_pick_kernel (tcgen05 LM head in row tiles, three operand planes, per-32-id sampling "
+            "partials in its epilogue, then the pick)")
 
 
 def config_of(wl, ctx):
