@@ -229,7 +229,7 @@ int osprey_draft_step_topk(osprey_ctx *ctx, const osprey_kv *kv, int B, int K, i
  *   at the last accepted depth, -1 if none), flags [B][K+1] (bit 3: a residual
  *   without float32 mass, p sampled instead; bit 4: the draw clamped to the
  *   last id with weight).
- * No workspace: a cluster of 8 blocks per sequence keeps its walk on chip; rows off
+ * No workspace: a cluster of blocks per sequence keeps its walk on chip; rows off
  * the walked path are at most prefetched.  V <= 2^20.
  * Device errors: INVALID_ARG for a candidate outside [0, V) (that sequence gets
  * n_accepted 0 and out_tokens -1). */

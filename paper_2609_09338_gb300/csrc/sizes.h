@@ -113,4 +113,32 @@ inline bool attn_rows_pays(long long R, int Hq, int Hkv, int rows_per_seq, int m
     return rows_per_seq > 1 && rows_per_seq * G >= 8 && R * Hkv * (G + 2) * max_ctx >= 6000000LL;
 }
 
+// Blocks of a tree walk's cluster, as 8 >> the index returned: the size whose waves
+// take the least.  at_once: clusters of 8, 4, 2 and 1 blocks that the device holds;
+// cached: their slices of two rows fit shared memory.  A walk takes a fixed time
+// (barriers, exchanges: what one block takes for 95 KB of a row, 3 KB more a block of
+// the cluster; greedy, without exponentials, 300 KB) and the row over the blocks, a
+// third more where later passes read it again.  Walks differ in length, so waves
+// overlap: x times what fits takes x + 0.4.
+// us a call with clusters of 8 always / as chosen / one block a sequence in its first
+// form (K 3, topk 2): float32, T 1, V 151936, 16 sequences 47 / 47 / 116, 64 134 / 82 /
+// 140, 256 464 / 251 / 262; V 4096, 32 28 / 22 / 24, 128 95 / 25 / 25, 512 345 / 40 /
+// 76; bf16, V 32000, 32 31 / 29 / 46, 512 375 / 120 / 146.  Of 234 such calls (V 4001
+// to 200064, 1 to 512 sequences, greedy too) 6 are 4 to 10 % slower than in the first
+// form, all of 96 sequences and more (float32 V 50304, bf16 V 32000 greedy).
+inline int tree_cluster(int B, double row_kb, bool greedy, const bool (&cached)[4], const long long (&at_once)[4]) {
+    int pick = 0;
+    double best = 0;
+    for (int i = 0; i < 4; ++i) {
+        const int c = 8 >> i;
+        const double x = (double)B / at_once[i], row = row_kb / c * (greedy || cached[i] ? 1. : 1.35);
+        const double cost = (x <= 1 ? 1. : x + 0.4) * ((greedy ? 300 : 95) + 3 * c + row);
+        if (i == 0 || cost < best) {
+            best = cost;
+            pick = i;
+        }
+    }
+    return pick;
+}
+
 }  // namespace osp

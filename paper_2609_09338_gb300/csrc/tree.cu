@@ -11,8 +11,9 @@
 // end it with a draw from the last residual.  Greedy: the node's argmax is
 // accepted if it is a candidate (the first such).
 //
-// One cluster of 8 blocks (512 threads each) per sequence walks its tree: block k
-// takes the k-th range of the vocabulary.  A walk is a chain of dependent passes
+// One cluster of up to 8 blocks (512 threads each) per sequence walks its tree: block k
+// takes the k-th range of the vocabulary; many sequences or short rows take fewer
+// blocks each (tree_cluster).  A walk is a chain of dependent passes
 // over one or two rows, so its time is the passes' latency.  One block a sequence
 // pulled 1.2 MB a depth through one SM; 8 blocks pull it through as many, by bulk
 // copies to shared memory, so the passes after the first (a rejection's residual
@@ -27,15 +28,18 @@
 #include <cooperative_groups.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "internal.h"
+#include "sizes.h"
 #include "tma.cuh"
 
 namespace osp {
 
 namespace cg = cooperative_groups;
 
-constexpr int TR_CS = 8;          // blocks per cluster (an exchange has a lane per block)
+constexpr int TR_CS = 8;          // blocks per cluster at most (an exchange has a lane per block)
 constexpr int TR_THREADS = 512;
 constexpr int TR_WARPS = TR_THREADS / 32;
 constexpr int TR_CH = 256;       // ids per chunk: 32 lanes x 8
@@ -43,6 +47,7 @@ constexpr int TR_U = 1;          // chunks a warp loads before using them
 constexpr int TR_UG = 4;         // ... in an argmax pass
 constexpr int TR_NP = 4;         // pieces a slice arrives in
 constexpr size_t TREE_SMEM_CAP = 216 * 1024;
+constexpr size_t TREE_SMEM_SM = 228 * 1024, TREE_SMEM_BLOCK = 6 * 1024;   // of an SM; a block's static part and the system's
 constexpr float TR_LOG2E = 1.4426950408889634f;
 
 __device__ __forceinline__ float tr_ex2(float x) {
@@ -293,12 +298,16 @@ template <typename T, bool VEC>
 __device__ int tr_argmax(TrCtx<T> &t, const T *z) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, V = t.V;
     AM am{-INFINITY, 0x7fffffff};
+    // Chunks past the slice: skipped by a branch in float32 (64 registers, the loads of
+    // TR_UG chunks together: 256 sequences of V 151936 90 us, without it 130), loaded as
+    // -inf in bf16 (40 registers, three blocks an SM: 512 of V 32000 35 us, with it 50).
     for (int c0 = t.c_lo + warp; c0 < t.c_hi; c0 += TR_WARPS * TR_UG) {
         float f[TR_UG][8];
 #pragma unroll
         for (int u = 0; u < TR_UG; ++u) {
-            const int c = c0 + u * TR_WARPS;
-            if (c >= t.c_hi) continue;
+            int c = c0 + u * TR_WARPS;
+            if (sizeof(T) == 4 && c >= t.c_hi) continue;
+            if (sizeof(T) == 2) c = c < t.c_hi ? c : (V + TR_CH - 1) / TR_CH;   // past the row: -inf (see below)
             if (VEC) {
                 tr_load8<T, VEC>(z, c, V, f[u]);
             } else {   // unaligned rows: 32 consecutive ids a load instead of a vector per lane
@@ -312,7 +321,7 @@ __device__ int tr_argmax(TrCtx<T> &t, const T *z) {
 #pragma unroll
         for (int u = 0; u < TR_UG; ++u) {
             const int c = c0 + u * TR_WARPS;
-            if (c >= t.c_hi) continue;
+            if (sizeof(T) == 4 && c >= t.c_hi) continue;
 #pragma unroll
             for (int e = 0; e < 8; ++e)
                 if (f[u][e] > am.v) am = AM{f[u][e], c * TR_CH + (VEC ? lane * 8 + e : e * 32 + lane)};
@@ -478,7 +487,7 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
     T *slice = (T *)dyn;
     TrCtx<T> t{cluster, rank, cs, c_lo, min(nch, c_lo + slice_chunks), V, 0, 0, cached != 0,
                (float *)(slice + 2 * rows), slice, slice + rows, slots, full, a.status};
-    if (threadIdx.x == 0) {
+    if (!GREEDY && threadIdx.x == 0) {
         for (int p = 0; p < TR_NP; ++p) mbar_init(&full[p], 1);
         mbar_fence_init();
     }
@@ -503,7 +512,7 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
     }
     // every block has started (its shared memory may be written), and the defaults
     // above come before what other blocks of the cluster write over them
-    __threadfence();
+    if (cs > 1) __threadfence();
     cluster.sync();
     if (!ok) {   // the same in every block
         if (!GREEDY && VEC && t.cached)   // the copies under way land before the block can exit
@@ -608,35 +617,89 @@ __global__ void __launch_bounds__(TR_THREADS) tree_verify_kernel(const VerifyTre
     }
 }
 
+// What an SM and the device hold of a kernel at once, queried once per device:
+// blocks per SM by registers and threads, and clusters of 8, 4, 2 and 1 blocks with
+// that many blocks an SM and with one (clusters stay within a GPC).
+struct TreeFit {
+    std::atomic<int> per_sm, full[4], one[4];
+};
+
+// A cluster's slices of V ids: chunks a block, bytes of shared memory, and whether
+// they hold two rows (else the later passes read the rows again, from L2).
+struct TreeSlice {
+    int chunks;
+    size_t smem;
+    bool cached;
+};
+template <typename T, bool GREEDY>
+static TreeSlice tree_slice(int V, int cs) {
+    const int chunks = ((V + TR_CH - 1) / TR_CH + cs - 1) / cs;
+    const size_t both = (size_t)chunks * (2 * TR_CH * sizeof(T) + sizeof(float));
+    const bool cached = !GREEDY && both <= TREE_SMEM_CAP;
+    return TreeSlice{chunks, cached ? both : chunks * sizeof(float), cached};
+}
+
+template <typename K>
+static cudaLaunchConfig_t tree_config(K, int clusters, int cs, size_t smem, cudaStream_t s, cudaLaunchAttribute (&attr)[2]) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)clusters * cs);
+    cfg.blockDim = dim3(TR_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cs;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cs > 1 ? 2 : 1;   // (a block alone is a cluster of one)
+    return cfg;
+}
+
 template <typename T, bool VEC, bool GREEDY>
 static cudaError_t tree_launch(const VerifyTreeArgs &a, cudaStream_t s) {
     auto *kernel = tree_verify_kernel<T, VEC, GREEDY>;
     static std::atomic<int> done[kMaxDevices];
-    cudaError_t e = once_per_device(done, [&] { return allow_smem(kernel); });
-    if (e != cudaSuccess) return e;
-    const int nch = (a.V + TR_CH - 1) / TR_CH;
-    const int cs = TR_CS;
-    const int slice = (nch + cs - 1) / cs;
-    // two rows of a slice in shared memory; a vocabulary too large for that
-    // (V > 8 x 26k at 8 blocks) is read again by the later passes, from L2
-    size_t smem = (size_t)slice * (2 * TR_CH * sizeof(T) + sizeof(float));
-    const int cached = !GREEDY && smem <= TREE_SMEM_CAP;
-    if (!cached) smem = (size_t)slice * sizeof(float);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)a.B * cs);
-    cfg.blockDim = dim3(TR_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
+    static TreeFit fits[kMaxDevices];
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    e = cudaLaunchKernelEx(&cfg, kernel, a, slice, cached);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    TreeFit &fit = fits[dev % kMaxDevices];
+    e = once_per_device(done, [&] {
+        cudaError_t q = allow_smem(kernel);
+        int n = 0;
+        if (q == cudaSuccess) q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, TR_THREADS, 0);
+        fit.per_sm = std::max(n, 1);
+        for (int i = 0; i < 3 && q == cudaSuccess; ++i) {
+            cudaLaunchConfig_t cfg = tree_config(kernel, 1, TR_CS >> i, 0, nullptr, attr);
+            q = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+            fit.full[i] = std::max(n, 1);
+            cfg.dynamicSmemBytes = TREE_SMEM_CAP;
+            if (q == cudaSuccess) q = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
+            fit.one[i] = std::max(n, 1);
+        }
+        if (q == cudaSuccess) q = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        fit.full[3] = fit.per_sm * n;
+        fit.one[3] = n;
+        return q;
+    });
+    if (e != cudaSuccess) return e;
+    TreeSlice slices[4];
+    bool cached[4];
+    long long at_once[4];
+    for (int i = 0; i < 4; ++i) {
+        slices[i] = tree_slice<T, GREEDY>(a.V, TR_CS >> i);
+        const int fits = (int)(TREE_SMEM_SM / (slices[i].smem + TREE_SMEM_BLOCK));   // blocks of an SM by shared memory
+        cached[i] = slices[i].cached;
+        at_once[i] = fits >= (int)fit.per_sm ? (int)fit.full[i] : (int)fit.one[i] * std::max(fits, 1);
+    }
+    const int pick = tree_cluster(a.B, (double)a.V * sizeof(T) / 1024, GREEDY, cached, at_once);
+    const int cs = TR_CS >> pick;
+    const TreeSlice sl = slices[pick];
+    const cudaLaunchConfig_t cfg = tree_config(kernel, a.B, cs, sl.smem, s, attr);
+    e = cudaLaunchKernelEx(&cfg, kernel, a, sl.chunks, (int)sl.cached);
     count_launch();
     return e;
 }
