@@ -969,11 +969,16 @@ __global__ void __launch_bounds__(VS_THREADS, OSP_VS_BPS) vs_sample(const Verify
 
 // ---------------------------------------------------------------------------
 // 0: not streamed; 1: every row starts on 16 bytes; 2: the tensors do, their rows
-// need not.
+// need not.  (Greedy rows off 16 bytes: streamed only where that is faster.)
 int verify_stream_mode(const VerifyArgs &a) {
     if ((uintptr_t)a.target % 16 || (uintptr_t)a.draft % 16 || a.K + 1 > 32) return 0;
     const int s = a.dtype == OSPREY_F32 ? 4 : 2;
-    return (size_t)a.V * s % 16 == 0 ? 1 : 2;
+    if ((size_t)a.V * s % 16 == 0) return 1;
+    // an argmax alone hides no masks: many float32 rows off 16 bytes are faster with an
+    // element a load (9 rows of V 100001 x 16 18 us against 22, of V 200001 x 64 92
+    // against 99; 5 of V 20001 x 64, 26 MB, 19 against 16)
+    const size_t bytes = (size_t)a.B * (a.K + 1) * a.V * s;
+    return a.temperature == 0.f && a.dtype == OSPREY_F32 && bytes >= (32u << 20) ? 0 : 2;
 }
 
 // Opt each kernel into the ring's shared memory once per device.  The flag

@@ -19,7 +19,8 @@ from test_verify_hidden_gpu import _inputs, _run_hidden  # noqa: E402
 
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("V,B,K,T", [(1, 3, 2, 1.0), (5, 9, 3, 0.7), (1025, 7, 3, 1.0), (2049, 6, 4, 0.0), (4097, 5, 2, 1.0),
-                                     (4094, 6, 3, 1.0), (40963, 33, 5, 0.7), (2047, 300, 2, 1.0)])
+                                     (4094, 6, 3, 1.0), (40963, 33, 5, 0.7), (2047, 300, 2, 1.0),
+                                     (50021, 43, 3, 0.0)])   # (greedy float32 of 32 MB and more: not streamed)
 def test_rows_at_any_alignment(V, B, K, T, dtype):
     vi = syn.make_verify_inputs(V, B, K, T, 0.7, seed=V + B + K)
     g, o = _run(vi, T, dtype), _oracle(vi, T, dtype)
