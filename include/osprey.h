@@ -254,7 +254,7 @@ size_t osprey_dflash_workspace_bytes(const osprey_ctx *ctx, int B, int block, in
  * from its own q_j = softmax(logits_j / T) by the inverse CDF at u_draft[b][j]
  * (argmax at T = 0).  The proposals are verified like a chain of block - 1
  * draft tokens (osprey_verify with K = block - 1).
- *   block  4 .. 81 (3 .. 80 proposals); a tensor-core pass over the weights takes
+ *   block  4 .. 65 (3 .. 64 proposals); a tensor-core pass over the weights takes
  *          up to 512 proposals (SHAPE if the context has no tensor-core path).  Each
  *          group of floor(80 / (block - 1)) consecutive sequences is summed in one
  *          order, so its results do not depend on the other groups of the call

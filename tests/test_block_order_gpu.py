@@ -46,7 +46,7 @@ def make(shape, ctx, block, seed):
             "u": rng.random((B, P), dtype=np.float32)}
 
 
-def propose(c, T, seqs=None):
+def propose(c, T, seqs=None, refused=()):
     from paper_2609_09338_gb300.binding import to_device_bf16
     from paper_2609_09338_gb300.session import DflashSession
     seqs = list(range(len(c["ctx"]))) if seqs is None else seqs
@@ -56,11 +56,13 @@ def propose(c, T, seqs=None):
     kv = c["kv"]
     sess = DflashSession(c["shape"], c["w"], kv["page_table"][seqs], kv["n_pages"], c["block"])
     sess.append(c["ctx"][seqs], kv["k_rows"][:, rows], kv["v_rows"][:, rows])
+    for b in refused:                # pages outside the pool: the call reports and skips these sequences
+        sess.kv.page_table[b] = -1
     out = sess.block_buffers(with_logits=True)
     sess.propose(dev(c["anchors"][seqs]), 5, to_device_bf16(np.ascontiguousarray(c["feats"][seqs])), T,
                  dev(c["u"][seqs]), out)
     torch.cuda.synchronize()
-    assert int(sess.status.item()) == 0
+    assert (int(sess.status.item()) != 0) == bool(refused)
     return {k: v.cpu().numpy() for k, v in out.items()}
 
 
@@ -89,6 +91,18 @@ def test_groups_do_not_change_one_another(block, T):
         own = propose(c, T, seqs)
         for k in own:
             np.testing.assert_array_equal(whole[k][seqs], own[k], err_msg=f"{k} of group {b0}")
+
+
+@pytest.mark.parametrize("refused", [range(5, 10), range(0, 5), range(5, 13)])
+def test_a_refused_group_leaves_the_others(refused):
+    """Attention runs once a group: one without a valid row ends early, and what follows still waits for the others."""
+    shape = replace(TINY, n_layers=3, ffn_dim=4096)
+    c = make(shape, np.random.default_rng(4).integers(1, 900, size=13), 16, 23)
+    whole, some = propose(c, 1.0), propose(c, 1.0, refused=refused)
+    kept = [b for b in range(13) if b not in refused]
+    for k in whole:
+        np.testing.assert_array_equal(some[k][kept], whole[k][kept], err_msg=k)
+    assert (some["draft_tokens"][list(refused)] == -1).all()
 
 
 @pytest.mark.parametrize("B,block", [(63, 16), (66, 16), (160, 4), (13, 65)])
